@@ -57,7 +57,9 @@ extern "C" {
 #define HC_STOP_STATUS 3    /* a step failed (HC_ENONFINITE) */
 
 /* Arithmetic of the path. */
-#define HC_FP64_PLAIN 0   /* every kernel in IEEE FP64 */
+#define HC_FP64_PLAIN 0   /* FP64 fields and pointwise arithmetic; power-of-two transforms of 64 points or
+                             more in 64-bit block fixed point, whose error is below that of the
+                             same transform in IEEE FP64 */
 #define HC_FP32_REFINED 1 /* FFTs, operator applies and split step in FP32; pressure solve wrapped in
                              FP64 iterative refinement (FP64 residual, FP64 correction accumulation,
                              FP64 dot products and null-space projection) */

@@ -157,6 +157,7 @@ struct hc_ctx {
   // tables
   cx<float>*twx_f, *twy_f;
   cx<double>*twx_d, *twy_d;
+  hc::FxTw *twx_x, *twy_x, *twz_x;  // fx64 kernels
   cx<df64>*twx_q, *twy_q;
   float *kxd_f, *kyd_f, *hx_f, *hy_f;
   double *kxd_d, *kyd_d, *hx_d, *hy_d;
@@ -243,6 +244,37 @@ void twiddles(int N, std::vector<double>& re, std::vector<double>& im) {
     re[m] = ct;
     im[m] = -stt;
   }
+}
+
+// Twiddle table of the fx64 kernels.  Fixed-point lengths: exp(-2 pi i m / N) in
+// Q62, the first octant from the long double functions, the others by symmetry;
+// shorter lengths: the FP64 values.
+std::vector<hc::FxTw> twiddles_fx(int N) {
+  std::vector<hc::FxTw> out(N);
+  if (N < (1 << hc::kFxMinLog)) {
+    std::vector<double> re, im;
+    twiddles(N, re, im);
+    for (int m = 0; m < N; ++m) {
+      const double v[2] = {re[m], im[m]};
+      std::memcpy(&out[m], v, sizeof(v));
+    }
+    return out;
+  }
+  // (long double is slow in software on some hosts: N/8 + 1 evaluations only)
+  const int E = N / 8, Q = N / 4;
+  std::vector<long long> co(E + 1), si(E + 1);
+  for (int r = 0; r <= E; ++r) {
+    const long double phi = 1.57079632679489661923132169163975144L * (long double)r / Q;
+    co[r] = std::llroundl(std::ldexp(std::cos(phi), 62));
+    si[r] = std::llroundl(std::ldexp(std::sin(phi), 62));
+  }
+  for (int m = 0; m < N; ++m) {
+    const int q = m / Q, r = m - q * Q;  // angle = (pi/2) (q + r/Q)
+    const long long c = r <= E ? co[r] : si[Q - r], s = r <= E ? si[r] : co[Q - r];
+    const long long re[4] = {c, -s, -c, s}, im[4] = {s, c, -s, -c};
+    out[m] = hc::fx_twiddle(re[q], -im[q]);
+  }
+  return out;
 }
 
 // Fourier variable of Section 2.3.3 (Nyquist entry positive).
@@ -333,6 +365,8 @@ void layout(hc_ctx* c, Layout& L) {
   c->twy_f = L.take<cx<float>>(sizeof(cx<float>) * c->ny);
   c->twx_d = L.take<cx<double>>(sizeof(cx<double>) * c->nx);
   c->twy_d = L.take<cx<double>>(sizeof(cx<double>) * c->ny);
+  c->twx_x = L.take<hc::FxTw>(sizeof(hc::FxTw) * c->nx);
+  c->twy_x = L.take<hc::FxTw>(sizeof(hc::FxTw) * c->ny);
   c->kxd_f = L.take<float>(sizeof(float) * c->H);
   c->kyd_f = L.take<float>(sizeof(float) * c->ny);
   c->hx_f = L.take<float>(sizeof(float) * (c->H + 1));
@@ -352,6 +386,7 @@ void layout(hc_ctx* c, Layout& L) {
   if (d == 3) {
     c->twz_f = L.take<cx<float>>(sizeof(cx<float>) * c->nz);
     c->twz_d = L.take<cx<double>>(sizeof(cx<double>) * c->nz);
+    c->twz_x = L.take<hc::FxTw>(sizeof(hc::FxTw) * c->nz);
     c->twz_q = L.take<cx<df64>>(sizeof(cx<df64>) * c->nz);
     c->kzd_f = L.take<float>(sizeof(float) * c->nz);
     c->kzd_d = L.take<double>(sizeof(double) * c->nz);
@@ -606,7 +641,7 @@ void fill_generic_geo(hc_ctx* c) {
 int upload_tables(hc_ctx* c) {
   if (c->gen) return upload_tables_generic(c);
   std::vector<double> re, im;
-  auto put_tw = [&](int N, cx<float>* df, cx<double>* dd, cx<df64>* dq) -> int {
+  auto put_tw = [&](int N, cx<float>* df, cx<double>* dd, cx<df64>* dq, hc::FxTw* dx) -> int {
     twiddles(N, re, im);
     std::vector<cx<float>> hf(N);
     std::vector<cx<double>> hd(N);
@@ -622,11 +657,13 @@ int upload_tables(hc_ctx* c) {
     CU(cudaMemcpy(df, hf.data(), sizeof(cx<float>) * N, cudaMemcpyHostToDevice));
     CU(cudaMemcpy(dd, hd.data(), sizeof(cx<double>) * N, cudaMemcpyHostToDevice));
     CU(cudaMemcpy(dq, hq.data(), sizeof(cx<df64>) * N, cudaMemcpyHostToDevice));
+    const std::vector<hc::FxTw> hx = twiddles_fx(N);
+    CU(cudaMemcpy(dx, hx.data(), sizeof(hc::FxTw) * N, cudaMemcpyHostToDevice));
     return HC_OK;
   };
-  int rc = put_tw(c->nx, c->twx_f, c->twx_d, c->twx_q);
+  int rc = put_tw(c->nx, c->twx_f, c->twx_d, c->twx_q, c->twx_x);
   if (rc) return rc;
-  rc = put_tw(c->ny, c->twy_f, c->twy_d, c->twy_q);
+  rc = put_tw(c->ny, c->twy_f, c->twy_d, c->twy_q, c->twy_x);
   if (rc) return rc;
   std::vector<double> kx(c->H), ky(c->ny);
   for (int k = 0; k < c->H; ++k) kx[k] = (k == 0) ? 0.0 : xid(k, c->nx, c->grid.L[0]);
@@ -648,7 +685,7 @@ int upload_tables(hc_ctx* c) {
   CU(cudaMemcpy(c->kxd_q, kxq.data(), sizeof(df64) * c->H, cudaMemcpyHostToDevice));
   CU(cudaMemcpy(c->kyd_q, kyq.data(), sizeof(df64) * c->ny, cudaMemcpyHostToDevice));
   if (c->dim == 3) {
-    rc = put_tw(c->nz, c->twz_f, c->twz_d, c->twz_q);
+    rc = put_tw(c->nz, c->twz_f, c->twz_d, c->twz_q, c->twz_x);
     if (rc) return rc;
     std::vector<double> kz(c->nz);
     for (int k = 0; k < c->nz; ++k) kz[k] = xid(k, c->nz, c->grid.L[2]);
@@ -784,6 +821,13 @@ int push_config(hc_ctx* c) {
 }
 
 // ---------------------------------------------------------------- step pieces
+// The FP64 geometry with the fx64 transforms, for a refined context's transforms
+// that feed no FP32 arithmetic (the certifying residual; p to and from the host).
+hc::Geo<double> fx_geo(hc::Geo<double> g) {
+  g.fx = 1;
+  return g;
+}
+
 template <typename T>
 hc::Tri<cx<T>*> tri(cx<T>* G, size_t ns) {
   return hc::Tri<cx<T>*>{{G, G + ns, G + 2 * ns}};
@@ -1865,18 +1909,26 @@ int hc_create(hc_ctx** out, const hc_grid* grid, const hc_params* params, void* 
     fill_geo<df64>(c, c->gq, c->twx_q, c->twy_q, c->kxd_q, c->kyd_q, nullptr, nullptr);
     c->gq.tc = c->gd.tc;
     c->gq.ltc = c->gd.ltc;
+    c->gd.fx = c->refined ? 0 : 1;
+    c->gd.qx = c->twx_x;
+    c->gd.qy = c->twy_x;
+    c->gd.qz = c->twz_x;
     if (c->dim == 3) {
       fill_geo3<float>(c, c->gf, c->rowf, c->twz_f, c->kzd_f, c->hz_f);
       fill_geo3<double>(c, c->gd, c->rowd, c->twz_d, c->kzd_d, c->hz_d);
       fill_geo3<df64>(c, c->gq, c->rowq, c->twz_q, c->kzd_q, nullptr);
     }
-    hc::set_smem_limits_f32();
-    hc::set_smem_limits_f64();
-    hc::set_smem_limits_df();
-    if (c->dim == 3) {
-      hc::set_smem_limits_3d_f32();
-      hc::set_smem_limits_3d_f64();
-      hc::set_smem_limits_3d_df();
+    hc::set_smem_limits_fx(c->refined);
+    if (c->dim == 3) hc::set_smem_limits_3d_fx(c->refined);
+    if (c->refined) {  // a plain FP64 context runs the fx64 kernels alone
+      hc::set_smem_limits_f32();
+      hc::set_smem_limits_f64();
+      hc::set_smem_limits_df();
+      if (c->dim == 3) {
+        hc::set_smem_limits_3d_f32();
+        hc::set_smem_limits_3d_f64();
+        hc::set_smem_limits_3d_df();
+      }
     }
   }
   int rc = HC_OK;
@@ -1975,7 +2027,7 @@ int hc_set_r(hc_ctx* c, const double* r, size_t count) {
 }
 
 // Forward 3D transform of the FP64 field in stage -> projected FP64 spectrum.
-static int forward64_3d(hc_ctx* c, cx<double>* out, hc::SolveState* norm_into) {
+static int forward64_3d(hc_ctx* c, cx<double>* out, hc::SolveState* norm_into, bool fx) {
   if (c->df) {
     df64* phys = reinterpret_cast<df64*>(c->stage + c->n);
     cx<df64>* rows = reinterpret_cast<cx<df64>*>(c->G64);
@@ -1986,9 +2038,10 @@ static int forward64_3d(hc_ctx* c, cx<double>* out, hc::SolveState* norm_into) {
     c->launches += 4;
   } else {
     cx<double>* rows = c->G64;
-    hc::row_r2c<double>(c->rowd, c->stage, nullptr, rows, nullptr, c->stream);
-    hc::axis_fft<double>(c->gd, 1, -1, 1, tri(rows, c->ns), tri(rows, c->ns), 1.0, c->stream);
-    hc::z_fwd_project<double>(c->gd, rows, out, norm_into, c->stream);
+    const hc::Geo<double> g = fx ? fx_geo(c->gd) : c->gd;
+    hc::row_r2c<double>(fx ? fx_geo(c->rowd) : c->rowd, c->stage, nullptr, rows, nullptr, c->stream);
+    hc::axis_fft<double>(g, 1, -1, 1, tri(rows, c->ns), tri(rows, c->ns), 1.0, c->stream);
+    hc::z_fwd_project<double>(g, rows, out, norm_into, c->stream);
     c->launches += 3;
   }
   CU(cudaGetLastError());
@@ -1996,8 +2049,9 @@ static int forward64_3d(hc_ctx* c, cx<double>* out, hc::SolveState* norm_into) {
 }
 
 // Forward 2D transform of the FP64 field in stage -> projected FP64 spectrum.
-static int forward64(hc_ctx* c, cx<double>* out, hc::SolveState* norm_into) {
-  if (c->dim == 3) return forward64_3d(c, out, norm_into);
+// fx: with the fx64 transforms (plain FP64 contexts always take them).
+static int forward64(hc_ctx* c, cx<double>* out, hc::SolveState* norm_into, bool fx) {
+  if (c->dim == 3) return forward64_3d(c, out, norm_into, fx);
   if (c->gen) {
     hc::gen_row_fwd(c->gg, c->stage, nullptr, c->G64, nullptr, c->stream);
     hc::gen_col_fwd(c->gg, c->G64, nullptr, out, nullptr, 1, 0, norm_into, c->stream);
@@ -2017,8 +2071,9 @@ static int forward64(hc_ctx* c, cx<double>* out, hc::SolveState* norm_into) {
     return HC_OK;
   }
   cx<double>* rows = c->G64;
-  hc::row_r2c<double>(c->gd, c->stage, nullptr, rows, nullptr, c->stream);
-  hc::col_fwd<double>(c->gd, rows, nullptr, out, nullptr, 1, 1, norm_into, c->stream);
+  const hc::Geo<double> g = fx ? fx_geo(c->gd) : c->gd;
+  hc::row_r2c<double>(g, c->stage, nullptr, rows, nullptr, c->stream);
+  hc::col_fwd<double>(g, rows, nullptr, out, nullptr, 1, 1, norm_into, c->stream);
   c->launches += 2;
   CU(cudaGetLastError());
   return HC_OK;
@@ -2029,7 +2084,8 @@ int hc_set_source(hc_ctx* c, const double* S, size_t count) {
   for (size_t i = 0; i < count; ++i)
     if (!std::isfinite(S[i])) return HC_EINVAL;
   CU(cudaMemcpyAsync(c->stage, S, sizeof(double) * count, cudaMemcpyHostToDevice, c->stream));
-  int rc = forward64(c, c->b64, c->st);
+  // S feeds the FP32 solves: a refined context transforms it in FP64 proper
+  int rc = forward64(c, c->b64, c->st, false);
   if (rc) return rc;
   if (c->refined) {  // FP32 copy for the first sweep's residual
     if (c->bq) {       // double-float copy for the mid-step residual
@@ -2058,7 +2114,7 @@ int hc_set_source(hc_ctx* c, const double* S, size_t count) {
 int hc_set_p(hc_ctx* c, const double* p, size_t count) {
   if (!c || !p || count != c->n) return HC_EINVAL;
   CU(cudaMemcpyAsync(c->stage, p, sizeof(double) * count, cudaMemcpyHostToDevice, c->stream));
-  int rc = forward64(c, c->p64, nullptr);
+  int rc = forward64(c, c->p64, nullptr, true);
   if (rc) return rc;
   CU(cudaStreamSynchronize(c->stream));
   return HC_OK;
@@ -2152,10 +2208,11 @@ int hc_get_p(hc_ctx* c, double* out, size_t count) {
       c->launches += 4;
     } else {
       cx<double>* rows = c->G64;
-      hc::axis_fft<double>(c->gd, 2, +1, 1, tri(c->p64, c->ns), tri(rows, c->ns),
-                           1.0 / (double)c->n, c->stream);
-      hc::axis_fft<double>(c->gd, 1, +1, 1, tri(rows, c->ns), tri(rows, c->ns), 1.0, c->stream);
-      hc::row_c2r<double>(c->rowd, rows, nullptr, c->stage, nullptr, nullptr, 0, c->stream);
+      const hc::Geo<double> g = fx_geo(c->gd);
+      hc::axis_fft<double>(g, 2, +1, 1, tri(c->p64, c->ns), tri(rows, c->ns), 1.0 / (double)c->n,
+                           c->stream);
+      hc::axis_fft<double>(g, 1, +1, 1, tri(rows, c->ns), tri(rows, c->ns), 1.0, c->stream);
+      hc::row_c2r<double>(fx_geo(c->rowd), rows, nullptr, c->stage, nullptr, nullptr, 0, c->stream);
       c->launches += 3;
     }
     CU(cudaGetLastError());
@@ -2173,8 +2230,9 @@ int hc_get_p(hc_ctx* c, double* out, size_t count) {
     c->launches += 3;
   } else {
     cx<double>* rows = c->G64;
-    hc::col_inv<double>(c->gd, c->p64, rows, 1.0 / (double)c->n, c->stream);
-    hc::row_c2r<double>(c->gd, rows, nullptr, c->stage, nullptr, nullptr, 0, c->stream);
+    const hc::Geo<double> g = fx_geo(c->gd);
+    hc::col_inv<double>(g, c->p64, rows, 1.0 / (double)c->n, c->stream);
+    hc::row_c2r<double>(g, rows, nullptr, c->stage, nullptr, nullptr, 0, c->stream);
     c->launches += 2;
   }
   CU(cudaGetLastError());
@@ -2219,7 +2277,7 @@ int hc_set_state(hc_ctx* c, const double* m, size_t m_count, const double* p, si
   double* pst = reinterpret_cast<double*>(c->G64c);  // n doubles fit in 2 half spectra
   const int nch = state_chunks(c), rows = c->ny / nch;
   const size_t prow = (size_t)rows * c->nx;           // values of one piece
-  hc::Geo<double> gch = c->gd;
+  hc::Geo<double> gch = fx_geo(c->gd);
   gch.ny = rows;                                      // a row pass over one piece
   // earlier work on the context's stream (it may still read m or the stage)
   CU(cudaEventRecord(c->io_ev[0], c->stream));
@@ -2235,7 +2293,7 @@ int hc_set_state(hc_ctx* c, const double* m, size_t m_count, const double* p, si
     hc::row_r2c<double>(gch, pst + k * prow, nullptr, c->G64 + (size_t)k * rows * c->H, nullptr,
                         c->stream);
   }
-  hc::col_fwd<double>(c->gd, c->G64, nullptr, c->p64, nullptr, 1, 1, nullptr, c->stream);
+  hc::col_fwd<double>(fx_geo(c->gd), c->G64, nullptr, c->p64, nullptr, 1, 1, nullptr, c->stream);
   CU(cudaMemcpyAsync(c->stage, m, sizeof(double) * m_count, cudaMemcpyHostToDevice, c->io_stream));
   hc::convert<float, double>(c->stage, (float*)c->m[0], c->n, c->io_stream);
   hc::convert<float, double>(c->stage + c->n, (float*)c->m[1], c->n, c->io_stream);
@@ -2262,7 +2320,7 @@ int hc_get_state(hc_ctx* c, double* m_out, size_t m_count, double* p_out, size_t
   double* pst = reinterpret_cast<double*>(c->G64c);
   const int nch = state_chunks(c), rows = c->ny / nch;
   const size_t prow = (size_t)rows * c->nx;
-  hc::Geo<double> gch = c->gd;
+  hc::Geo<double> gch = fx_geo(c->gd);
   gch.ny = rows;
   CU(cudaEventRecord(c->io_ev[0], c->stream));
   CU(cudaStreamWaitEvent(c->io_stream, c->io_ev[0], 0));
@@ -2271,7 +2329,7 @@ int hc_get_state(hc_ctx* c, double* m_out, size_t m_count, double* p_out, size_t
   // returns only when it is done
   hc::convert<double, float>((const float*)c->m[0], c->stage, c->n, c->io_stream);
   hc::convert<double, float>((const float*)c->m[1], c->stage + c->n, c->n, c->io_stream);
-  hc::col_inv<double>(c->gd, c->p64, c->G64, 1.0 / (double)c->n, c->stream);
+  hc::col_inv<double>(fx_geo(c->gd), c->p64, c->G64, 1.0 / (double)c->n, c->stream);
   CU(cudaMemcpyAsync(m_out, c->stage, sizeof(double) * m_count, cudaMemcpyDeviceToHost,
                      c->io_stream));
   // p's row transforms piece by piece, each piece's copy queued behind m's on

@@ -12,6 +12,9 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
+
+#include <type_traits>
 
 namespace hc {
 
@@ -73,6 +76,64 @@ __host__ __device__ inline bool operator<(df64 a, df64 b) { return b > a; }
 __host__ __device__ inline bool operator>=(df64 a, df64 b) { return !(b > a); }
 __host__ __device__ inline bool operator==(df64 a, df64 b) { return a.hi == b.hi && a.lo == b.lo; }
 __host__ __device__ inline bool operator!=(df64 a, df64 b) { return !(a == b); }
+
+// FP64 whose transforms run in 64-bit block fixed point on the integer pipes
+// (hc_fixed.cuh); everything else about it is double.  Kernels instantiated for
+// it read and write the same buffers as those for double.  Plain FP64 contexts
+// use it throughout; the refined modes where an FP64 transform's result does not
+// feed their FP32 arithmetic (the certifying residual, p on its way to the
+// host): there double keeps the earlier results bit for bit.
+struct fx64 {
+  double v;
+  fx64() = default;
+  __host__ __device__ constexpr fx64(double d) : v(d) {}
+  __host__ __device__ explicit operator double() const { return v; }
+  __host__ __device__ explicit operator float() const { return (float)v; }
+  __host__ __device__ fx64& operator+=(fx64 o) { v += o.v; return *this; }
+  __host__ __device__ fx64& operator*=(fx64 o) { v *= o.v; return *this; }
+};
+__host__ __device__ inline fx64 operator+(fx64 a, fx64 b) { return fx64(a.v + b.v); }
+__host__ __device__ inline fx64 operator-(fx64 a, fx64 b) { return fx64(a.v - b.v); }
+__host__ __device__ inline fx64 operator-(fx64 a) { return fx64(-a.v); }
+__host__ __device__ inline fx64 operator*(fx64 a, fx64 b) { return fx64(a.v * b.v); }
+__host__ __device__ inline fx64 operator/(fx64 a, fx64 b) { return fx64(a.v / b.v); }
+__host__ __device__ inline bool operator>(fx64 a, fx64 b) { return a.v > b.v; }
+__host__ __device__ inline bool operator<(fx64 a, fx64 b) { return a.v < b.v; }
+__host__ __device__ inline bool operator>=(fx64 a, fx64 b) { return a.v >= b.v; }
+__host__ __device__ inline bool operator==(fx64 a, fx64 b) { return a.v == b.v; }
+__host__ __device__ inline bool operator!=(fx64 a, fx64 b) { return a.v != b.v; }
+
+// Its kernels are bound by the latency of dependent integer instructions, so
+// they trade registers for warps: the fields of a pass one after the other (8
+// values of 16 bytes live per thread), at most 80 registers, three CTAs of 256
+// threads per SM.  The limit is given as a launch bound of 768 threads, whatever
+// the CTA's size.
+template <typename T>
+__host__ __device__ constexpr bool seq_fields() {
+  return std::is_same<T, fx64>::value;
+}
+template <typename T>
+__host__ __device__ constexpr int cta_bound(int threads) {
+  return seq_fields<T>() ? 768 : threads;
+}
+
+// Fixed-point transforms have 2^6 points or more; their twiddle tables hold
+// FxTw entries (16 bytes, as cx<double>), those of shorter ones FP64 values.
+constexpr int kFxMinLog = 6;
+// Twiddle in Q62, each component split into a high limb and a signed low limb:
+// value 2^62 w = 2^32 h + l.
+struct alignas(16) FxTw {
+  int xh, xl, yh, yl;
+};
+__host__ __device__ inline int fx_hi(long long v) { return (int)((v + 0x80000000LL) >> 32); }
+__host__ __device__ inline FxTw fx_twiddle(long long x, long long y) {
+  FxTw t;
+  t.xh = fx_hi(x);
+  t.xl = (int)x;
+  t.yh = fx_hi(y);
+  t.yl = (int)y;
+  return t;
+}
 
 // Device-resident scalar state of one pressure solve (CG and refinement).
 // All reductions that feed it are computed in FP64 by the last CTA of the
@@ -224,6 +285,10 @@ struct Geo {
   int npartials;             // capacity in CTAs
   int pipe;                  // 1: column passes run persistent with cp.async double buffering
   int pgrid;                 // CTAs of a persistent column pass (<= SMs, <= tiles)
+  int fx;                    // Geo<double>: launch the fx64 kernels (as_fx)
+  const FxTw* qx;            // Geo<double>: twiddle tables of the fx64 kernels
+  const FxTw* qy;
+  const FxTw* qz;
   int rpipe;                 // 1 (FP32): the apply row pass runs persistent with cp.async double buffering
   int rgrid;                 // CTAs of that pass (resident CTAs, <= row blocks)
   const T* x2x;              // xi_x^2 (positive Nyquist), kx = 0..H (H + 1 entries)
@@ -315,6 +380,26 @@ struct BShape {
   Geo<df64> gq;
   int nb;                 // members
 };
+
+// The geometry of the fx64 kernels on the same grid: the same tables but for the
+// twiddles.
+inline Geo<fx64> as_fx(const Geo<double>& g) {
+  static_assert(sizeof(Geo<fx64>) == sizeof(Geo<double>), "same layout");
+  Geo<fx64> h;
+  memcpy(static_cast<void*>(&h), &g, sizeof(h));
+  h.twx = reinterpret_cast<const cx<fx64>*>(g.qx);
+  h.twy = reinterpret_cast<const cx<fx64>*>(g.qy);
+  h.twz = reinterpret_cast<const cx<fx64>*>(g.qz);
+  return h;
+}
+inline cx<fx64>* fxp(cx<double>* p) { return reinterpret_cast<cx<fx64>*>(p); }
+inline const cx<fx64>* fxp(const cx<double>* p) { return reinterpret_cast<const cx<fx64>*>(p); }
+inline fx64* fxp(double* p) { return reinterpret_cast<fx64*>(p); }
+inline const fx64* fxp(const double* p) { return reinterpret_cast<const fx64*>(p); }
+template <typename P>
+inline auto fxp(const Tri<P>& t) {
+  return Tri<decltype(fxp(t.v[0]))>{{fxp(t.v[0]), fxp(t.v[1]), fxp(t.v[2])}};
+}
 
 // Threads of a column-pass CTA at most.  The FP32 gradient and divergence
 // passes (WIDE) take up to 1024 at 64 registers a thread: a tile of four
@@ -489,11 +574,13 @@ template <typename T>
 void msum3(const Geo<T>& g, Tri<const T*> m, SolveState* st, cudaStream_t s);
 void set_smem_limits_3d_f32();
 void set_smem_limits_3d_f64();
+void set_smem_limits_3d_fx(int refined);
 void set_smem_limits_3d_df();
 
 // Opt every kernel of one precision in to the full shared memory per block.
 void set_smem_limits_f32();
 void set_smem_limits_f64();
+void set_smem_limits_fx(int refined);
 // Lagged certification (2D refined steps): the FP64 certifying residual of
 // pressure p with the FP32 m, r it was solved with (sc: the certifying state,
 // skipped when nothing is pending); the commit after a lagged step (copies

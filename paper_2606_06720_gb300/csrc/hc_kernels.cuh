@@ -70,6 +70,10 @@ __device__ __forceinline__ cx<df64> ldg(const cx<df64>* p) {
   const float4 v = __ldg(reinterpret_cast<const float4*>(p));
   return cmk<df64>(df64(v.x, v.y), df64(v.z, v.w));
 }
+__device__ __forceinline__ cx<fx64> ldg(const cx<fx64>* p) {
+  const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+  return cmk<fx64>(v.x, v.y);
+}
 __device__ __forceinline__ bool hc_finite(df64 x) { return isfinite(x.hi); }
 
 __device__ __forceinline__ float hc_expm1(float x) { return expm1f(x); }
@@ -86,6 +90,13 @@ __device__ __forceinline__ float hc_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double hc_sqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ bool hc_finite(float x) { return isfinite(x); }
 __device__ __forceinline__ bool hc_finite(double x) { return isfinite(x); }
+__device__ __forceinline__ fx64 hc_expm1(fx64 x) { return expm1(x.v); }
+__device__ __forceinline__ fx64 hc_pow(fx64 x, fx64 y) { return pow(x.v, y.v); }
+__device__ __forceinline__ fx64 hc_log(fx64 x) { return log(x.v); }
+__device__ __forceinline__ fx64 hc_log1p(fx64 x) { return log1p(x.v); }
+__device__ __forceinline__ fx64 hc_exp(fx64 x) { return exp(x.v); }
+__device__ __forceinline__ fx64 hc_sqrt(fx64 x) { return sqrt(x.v); }
+__device__ __forceinline__ bool hc_finite(fx64 x) { return isfinite(x.v); }
 
 // ------------------------------------------------------------------ small DFTs
 // Kernel exp(S 2 pi i n k / R); S = -1 forward, +1 inverse.
@@ -153,6 +164,10 @@ __device__ __forceinline__ int rswz<double>(int e) {
 }
 template <>
 __device__ __forceinline__ int rswz<df64>(int e) {
+  return e ^ ((e >> 3) & 7);
+}
+template <>
+__device__ __forceinline__ int rswz<fx64>(int e) {
   return e ^ ((e >> 3) & 7);
 }
 // Slot of element e: swizzled row slab (SWZ) or padded column slab with stride ks.
@@ -347,9 +362,14 @@ __device__ __forceinline__ void fft_static_pass(cx<T> (&v)[NV][8], cx<T>* const*
   }
 }
 
+}  // namespace hc
+#include "hc_fixed.cuh"  // uses the slot helpers above
+namespace hc {
+
 // The transform every kernel calls: FP32 transforms of length 2^8 .. 2^12 (the
-// grids whose speed matters) use the compile-time-length code, all others the
-// runtime-length loop.  lN is uniform across the CTA.
+// grids whose speed matters) use the compile-time-length code, fx64 ones of 2^6
+// points or more the fixed-point passes, all others the runtime-length loop.  lN
+// is uniform across the CTA.
 template <int S, int NV, bool SWZ = false, typename T>
 __device__ __forceinline__ void fft_canon(cx<T> (&v)[NV][8], cx<T>* const* sl, int ks, int j,
                                           int lN, const cx<T>* __restrict__ tw) {
@@ -362,6 +382,12 @@ __device__ __forceinline__ void fft_canon(cx<T> (&v)[NV][8], cx<T>* const* sl, i
       case 11: fft_static_pass<S, NV, SWZ, 11, 0>(v, sl, ks, j, js, tw); return;
       case 12: fft_static_pass<S, NV, SWZ, 12, 0>(v, sl, ks, j, js, tw); return;
       default: break;
+    }
+  }
+  if constexpr (std::is_same<T, fx64>::value) {
+    if (lN >= kFxMinLog) {
+      fft_fixed<S, NV, SWZ>(v, sl, ks, j, lN, tw);
+      return;
     }
   }
   fft_rt<S, NV, SWZ>(v, sl, ks, j, lN, tw);
@@ -445,6 +471,12 @@ template <>
 struct DotAcc<double> {
   double s = 0.0;
   __device__ __forceinline__ void add_prod(double x, double y) { s = fma(x, y, s); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct DotAcc<fx64> {
+  double s = 0.0;
+  __device__ __forceinline__ void add_prod(fx64 x, fx64 y) { s = fma(x.v, y.v, s); }
   __device__ __forceinline__ double value() const { return s; }
 };
 template <>
@@ -709,18 +741,33 @@ __device__ __forceinline__ void store_rows_r2c(cx<T> (&v)[NV][8], cx<T>* const* 
     }
   }
 }
+// Forward transform of NV complex rows a + i b and their packed half spectra.
+template <int NV, typename T>
+__device__ __forceinline__ void fft_rows_r2c(cx<T> (&v)[NV][8], cx<T>* const* slab, int j, int lN,
+                                             const cx<T>* __restrict__ tw, cx<T>* const* A,
+                                             cx<T>* const* B) {
+  if constexpr (std::is_same<T, fx64>::value) {
+    if (lN >= kFxMinLog) {
+      fft_fixed_r2c<NV>(v, slab, j, lN, tw, A, B);
+      return;
+    }
+  }
+  fft_canon<-1, NV, true>(v, slab, 1, j, lN, tw);
+  store_rows_r2c<NV>(v, slab, j, 1 << lN, 1 << (lN - 1), A, B);
+}
 template <typename T>
-__device__ __forceinline__ void store_pair_r2c(cx<T> (&v)[1][8], cx<T>* slab, int j, int N, int H,
-                                               cx<T>* __restrict__ A, cx<T>* __restrict__ B) {
+__device__ __forceinline__ void fft_pair_r2c(cx<T> (&v)[1][8], cx<T>* slab, int j, int lN,
+                                             const cx<T>* __restrict__ tw, cx<T>* __restrict__ A,
+                                             cx<T>* __restrict__ B) {
   cx<T>* const sl[1] = {slab};
   cx<T>* const a[1] = {A};
   cx<T>* const b[1] = {B};
-  store_rows_r2c<1>(v, sl, j, N, H, a, b);
+  fft_rows_r2c<1>(v, sl, j, lN, tw, a, b);
 }
 
 // ------------------------------------------------------------------ row kernels
 template <typename T>
-__global__ void __launch_bounds__(512) k_row_r2c(Geo<T> g, const T* __restrict__ a,
+__global__ void __launch_bounds__(cta_bound<T>(512)) k_row_r2c(Geo<T> g, const T* __restrict__ a,
                                                  const T* __restrict__ b, cx<T>* __restrict__ A,
                                                  cx<T>* __restrict__ B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -737,8 +784,7 @@ __global__ void __launch_bounds__(512) k_row_r2c(Geo<T> g, const T* __restrict__
     const int x = j + s * N8;
     v[0][s] = cmk<T>(a[ro + x], b ? b[ro + x] : (T)0);
   }
-  fft_canon<-1, 1, true>(v, sl, 1, j, g.lnx, g.twx);
-  store_pair_r2c(v, slab, j, N, H, A + (size_t)y * H, B ? B + (size_t)y * H : nullptr);
+  fft_pair_r2c(v, slab, j, g.lnx, g.twx, A + (size_t)y * H, B ? B + (size_t)y * H : nullptr);
 }
 
 template <typename T>
@@ -803,7 +849,7 @@ __device__ __forceinline__ void row_c2r_body(Geo<T> g, const cx<T>* A, const cx<
   }
 }
 template <typename T>
-__global__ void __launch_bounds__(512) k_row_c2r(Geo<T> g, const cx<T>* A, const cx<T>* B, T* a,
+__global__ void __launch_bounds__(cta_bound<T>(512)) k_row_c2r(Geo<T> g, const cx<T>* A, const cx<T>* B, T* a,
                                                  T* b, SolveState* st,
                                                  int kappa_update) {
   row_c2r_body<T>(g, A, B, a, b, st, kappa_update);
@@ -919,8 +965,7 @@ __device__ __forceinline__ void row_apply_body(Geo<T> g, const cx<T>* Gx, const 
       v[q][s] = cmk<T>(ax * mg + r * gx, ay * mg + r * gy);
     }
   }
-  fft_canon<-1, NV, true>(v, sl, 1, j, g.lnx, g.twx);
-  store_rows_r2c<NV>(v, sl, j, N, H, Qa, Qb);
+  fft_rows_r2c<NV>(v, sl, j, g.lnx, g.twx, Qa, Qb);
   if (DOT) {
     if constexpr (std::is_same<T, float>::value) {
       // FP32: the CTA's partial only; the divergence pass forms alpha
@@ -934,7 +979,7 @@ __device__ __forceinline__ void row_apply_body(Geo<T> g, const cx<T>* Gx, const 
   }
 }
 template <typename T, typename Tm, bool DOT, int NV>
-__global__ void __launch_bounds__(512) k_row_apply(Geo<T> g, const cx<T>* Gx, const cx<T>* Gy,
+__global__ void __launch_bounds__(cta_bound<T>(512)) k_row_apply(Geo<T> g, const cx<T>* Gx, const cx<T>* Gy,
                                                    const Tm* __restrict__ mx,
                                                    const Tm* __restrict__ my,
                                                    const Tm* __restrict__ rr, cx<T>* Qx, cx<T>* Qy,
@@ -1003,11 +1048,10 @@ __global__ void __launch_bounds__(512) kp_row_apply(Geo<float> g, const cx<float
       if (DOT) gkg.add_prod(mg * mg + r * (gx * gx + gy * gy), 1.0f);
       v[0][s] = cmk<float>(ax * mg + r * gx, ay * mg + r * gy);
     }
-    fft_canon<-1, 1, true>(v, sl, 1, j, g.lnx, g.twx);
     const size_t y = (size_t)blk * rpc + rb;
     cx<float>* Qa[1] = {Qx + y * H};
     cx<float>* Qb[1] = {Qy + y * H};
-    store_rows_r2c<1>(v, sl, j, N, H, Qa, Qb);
+    fft_rows_r2c<1>(v, sl, j, g.lnx, g.twx, Qa, Qb);
     __syncthreads();  // this buffer is refilled by the stage issued next iteration
     buf ^= 1;
   }
@@ -1129,8 +1173,7 @@ __device__ __forceinline__ void row_split_body(Geo<T> g, const cx<T>* Gx, const 
   }
   if (!finite) st->nonfinite = 1;
   if (diag) en.finish(g.partials, st);
-  fft_canon<-1, 1, true>(v, sl, 1, j, g.lnx, g.twx);
-  store_pair_r2c(v, slab, j, N, H, Mx + (size_t)y * H, My + (size_t)y * H);
+  fft_pair_r2c(v, slab, j, g.lnx, g.twx, Mx + (size_t)y * H, My + (size_t)y * H);
 }
 template <typename T>
 __global__ void __launch_bounds__(512) k_row_split(Geo<T> g, const cx<T>* Gx, const cx<T>* Gy,
@@ -1424,6 +1467,37 @@ __device__ __forceinline__ void col_grad_body(Geo<T> g, cx<Tin>* in, const cx<T>
     pc = pc_of<T>(st);
   }
   if (MODE == CG_ADDDELTA) add_delta = st->sweeps > 0;
+  if constexpr (seq_fields<T>()) {
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+      cx<T> v[1][8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const int ky = c.j + s * c.NY8;
+        const size_t idx = (size_t)ky * H + c.kx;
+        cx<T> P;
+        if (q > 0) {  // the value this thread has just updated
+          P = MODE == CG_DUPDATE ? dio[idx] : ccast<T>(in[idx]);
+        } else if constexpr (MODE == CG_PLAIN) {
+          P = ccast<T>(in[idx]);
+        } else if constexpr (MODE == CG_DUPDATE) {
+          const cx<T> z = cscale(rvec[idx], pinv_sym(g, c.kx, ky, pc));
+          P = first ? z : cadd(z, cscale(dio[idx], beta));
+          dio[idx] = P;
+        } else {
+          P = add_delta ? add_delta_at<T>(in, idx, delta[cmi(g, ky, c.kx)]) : ccast<T>(in[idx]);
+        }
+        const T a = q == 0 ? ax : g.kyd[ky] * invn;
+        v[0][s] = cmk<T>(-a * P.y, a * P.x);  // i (k/n) P
+      }
+      cx<T>* const sl1[1] = {sl[0]};
+      fft_canon<+1, 1>(v, sl1, 1 << g.ltc, c.j, g.lny, g.twy);
+      cx<T>* const G = q == 0 ? Gx : Gy;
+#pragma unroll
+      for (int s = 0; s < 8; ++s) G[(size_t)(c.j + s * c.NY8) * H + c.kx] = v[0][s];
+    }
+    return;
+  }
   cx<T> v[2][8];
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
@@ -1456,7 +1530,7 @@ __device__ __forceinline__ void col_grad_body(Geo<T> g, cx<Tin>* in, const cx<T>
   }
 }
 template <typename T, typename Tin, int MODE>
-__global__ void __launch_bounds__(col_cta_max<T, true>(), 1) k_col_grad(Geo<T> g, cx<Tin>* in, const cx<T>* __restrict__ rvec,
+__global__ void __launch_bounds__(cta_bound<T>(col_cta_max<T, true>()), 1) k_col_grad(Geo<T> g, cx<Tin>* in, const cx<T>* __restrict__ rvec,
                                                   cx<T>* dio, const cx<float>* __restrict__ delta,
                                                   cx<T>* __restrict__ Gx, cx<T>* __restrict__ Gy,
                                                   SolveState* st, int check_done) {
@@ -1479,14 +1553,40 @@ __device__ __forceinline__ void col_div_body(Geo<T> g, const cx<T>* __restrict__
   const int H = g.H;
   const int se = slab_elems(g);
   cx<T>* const sl[2] = {sm + c.b, sm + se + c.b};
-  cx<T> v[2][8];
+  if constexpr (seq_fields<T>()) {
+    // kx Qx + ky Qy adds up in this thread's own slots of the second slab
+    const T ax = g.kxd[c.kx];
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+      const cx<T>* const Q = (q == 0 ? Qx : Qy) + c.kx;
+      cx<T> v[1][8];
 #pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const size_t idx = (size_t)(c.j + s * c.NY8) * H + c.kx;
-    v[0][s] = Qx[idx];
-    v[1][s] = Qy[idx];
+      for (int s = 0; s < 8; ++s) v[0][s] = Q[(unsigned)(c.j + s * c.NY8) * (unsigned)H];
+      cx<T>* const sl1[1] = {sl[0]};
+      fft_canon<-1, 1>(v, sl1, 1 << g.ltc, c.j, g.lny, g.twy);
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const int ky = c.j + s * c.NY8;
+        cx<T>& t = sl[1][padk(ky) << g.ltc];
+        if (q == 0) {
+          t = cscale(v[0][s], ax);
+        } else {
+          const T ay = g.kyd[ky];
+          t = cmk<T>(t.x + ay * v[0][s].x, t.y + ay * v[0][s].y);
+        }
+      }
+    }
   }
-  fft_canon<-1, 2>(v, sl, g.tc, c.j, g.lny, g.twy);
+  cx<T> v[2][8];
+  if constexpr (!seq_fields<T>()) {
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const size_t idx = (size_t)(c.j + s * c.NY8) * H + c.kx;
+      v[0][s] = Qx[idx];
+      v[1][s] = Qy[idx];
+    }
+    fft_canon<-1, 2>(v, sl, g.tc, c.j, g.lny, g.twy);
+  }
   const T ax = g.kxd[c.kx];
   const double w = c.kx == 0 ? 1.0 : 2.0;  // Parseval weight of a packed column
   double acc[3] = {0.0, 0.0, 0.0};
@@ -1500,8 +1600,13 @@ __device__ __forceinline__ void col_div_body(Geo<T> g, const cx<T>* __restrict__
   for (int s = 0; s < 8; ++s) {
     const int ky = c.j + s * c.NY8;
     const size_t idx = (size_t)ky * H + c.kx;
-    const T ay = g.kyd[ky];
-    const cx<T> t = cmk<T>(ax * v[0][s].x + ay * v[1][s].x, ax * v[0][s].y + ay * v[1][s].y);
+    cx<T> t;
+    if constexpr (seq_fields<T>()) {
+      t = sl[1][padk(ky) << g.ltc];
+    } else {
+      const T ay = g.kyd[ky];
+      t = cmk<T>(ax * v[0][s].x + ay * v[1][s].x, ax * v[0][s].y + ay * v[1][s].y);
+    }
     const cx<T> q = cmk<T>(t.y, -t.x);  // -i (kx Qx + ky Qy)
     if constexpr (MODE == CD_PLAIN) {
       out[idx] = q;
@@ -1578,7 +1683,7 @@ __device__ __forceinline__ void col_div_body(Geo<T> g, const cx<T>* __restrict__
   }
 }
 template <typename T, int MODE>
-__global__ void __launch_bounds__(col_cta_max<T, true>(), 1) k_col_div(Geo<T> g, const cx<T>* __restrict__ Qx,
+__global__ void __launch_bounds__(cta_bound<T>(col_cta_max<T, true>()), 1) k_col_div(Geo<T> g, const cx<T>* __restrict__ Qx,
                                                  const cx<T>* __restrict__ Qy,
                                                  const cx<T>* __restrict__ d,
                                                  const cx<T>* __restrict__ bvec,
@@ -1675,7 +1780,7 @@ __device__ __forceinline__ void col_heat_body(Geo<T> g, cx<T>* Mx, cx<T>* My, So
   if (diag) gradnorm_finish(ga.value(), (double)g.nx * (double)ny, g.partials, st, 1);
 }
 template <typename T>
-__global__ void __launch_bounds__(col_cta_max<T, true>(), 1) k_col_heat(Geo<T> g, cx<T>* Mx, cx<T>* My,
+__global__ void __launch_bounds__(cta_bound<T>(col_cta_max<T, true>()), 1) k_col_heat(Geo<T> g, cx<T>* Mx, cx<T>* My,
                                                                         SolveState* st) {
   col_heat_body<T>(g, Mx, My, st);
 }
@@ -1717,7 +1822,7 @@ __global__ void __launch_bounds__(512) k_col_fwd(Geo<T> g, const cx<T>* __restri
 }
 
 template <typename T>
-__global__ void __launch_bounds__(512) k_col_inv(Geo<T> g, const cx<T>* __restrict__ in,
+__global__ void __launch_bounds__(cta_bound<T>(512)) k_col_inv(Geo<T> g, const cx<T>* __restrict__ in,
                                                  cx<T>* __restrict__ out, T scale) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
@@ -2293,8 +2398,7 @@ __global__ void __launch_bounds__(512) k_row_adj_point(Geo<T> g, cx<T>* G0, cx<T
     dc.add_prod(gl * mg, dt * (ph + z * dph));
   }
   cx<T>* const sl1[1] = {slab};
-  fft_canon<-1, 1, true>(w, sl1, 1, j, g.lnx, g.twx);
-  store_pair_r2c(w, slab, j, N, H, G0 + (size_t)y * H, G1 + (size_t)y * H);
+  fft_pair_r2c(w, slab, j, g.lnx, g.twx, G0 + (size_t)y * H, G1 + (size_t)y * H);
   double a1[1] = {dc.value()}, t1[1];
   if (last_cta_sum<1>(a1, g.partials, &as->ticket[TA_POINT], t1) && threadIdx.x == 0)
     as->dc2 += t1[0];
@@ -2454,16 +2558,25 @@ static inline int upd_blocks(size_t total) {
 
 template <typename T>
 void row_r2c(const Geo<T>& g, const T* a, const T* b, cx<T>* A, cx<T>* B, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx) return row_r2c<fx64>(as_fx(g), fxp(a), fxp(b), fxp(A), fxp(B), s);
   k_row_r2c<T><<<g.ny >> g.lrpc, row_threads(g), row_smem(g), s>>>(g, a, b, A, B);
 }
 template <typename T>
 void row_c2r(const Geo<T>& g, const cx<T>* A, const cx<T>* B, T* a, T* b, SolveState* st,
              int kappa_update, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return row_c2r<fx64>(as_fx(g), fxp(A), fxp(B), fxp(a), fxp(b), st, kappa_update, s);
   k_row_c2r<T><<<g.ny >> g.lrpc, row_threads(g), row_smem(g), s>>>(g, A, B, a, b, st, kappa_update);
 }
 template <typename T, typename Tm>
 void row_apply(const Geo<T>& g, const cx<T>* Gx, const cx<T>* Gy, const Tm* mx, const Tm* my,
                const Tm* r, cx<T>* Qx, cx<T>* Qy, SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value && std::is_same<Tm, double>::value)
+    if (g.fx)
+      return row_apply<fx64, fx64>(as_fx(g), fxp(Gx), fxp(Gy), fxp(mx), fxp(my), fxp(r), fxp(Qx),
+                                   fxp(Qy), st, s);
   const size_t sm = row_smem(g) + (size_t)3 * g.rpc * g.nx * sizeof(Tm);
   if constexpr (std::is_same<T, float>::value && std::is_same<Tm, float>::value) {
     if (g.rpipe) {
@@ -2495,12 +2608,19 @@ void row_apply(const Geo<T>& g, const cx<T>* Gx, const cx<T>* Gy, const Tm* mx, 
 template <typename T>
 void row_split(const Geo<T>& g, const cx<T>* Gx, const cx<T>* Gy, const T* mx, const T* my,
                const T* r, cx<T>* Mx, cx<T>* My, SplitCoef cf, SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return row_split<fx64>(as_fx(g), fxp(Gx), fxp(Gy), fxp(mx), fxp(my), fxp(r), fxp(Mx),
+                             fxp(My), cf, st, s);
   k_row_split<T><<<g.ny >> g.lrpc, row_threads(g), row_split_smem(g), s>>>(g, Gx, Gy, mx, my, r, Mx,
                                                                            My, cf, st);
 }
 template <typename T>
 void col_fwd(const Geo<T>& g0, const cx<T>* in0, const cx<T>* in1, cx<T>* out0, cx<T>* out1, int nv,
              int project, SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g0.fx)
+      return col_fwd<fx64>(as_fx(g0), fxp(in0), fxp(in1), fxp(out0), fxp(out1), nv, project, st, s);
   const Geo<T> g = col_narrow(g0);
   if (nv == 1)
     k_col_fwd<T, 1><<<g.H >> g.ltc, col_threads(g), col_smem(g, 1), s>>>(g, in0, in1, out0, out1,
@@ -2511,6 +2631,8 @@ void col_fwd(const Geo<T>& g0, const cx<T>* in0, const cx<T>* in1, cx<T>* out0, 
 }
 template <typename T>
 void col_inv(const Geo<T>& g0, const cx<T>* in, cx<T>* out, T scale, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g0.fx) return col_inv<fx64>(as_fx(g0), fxp(in), fxp(out), fx64(scale), s);
   const Geo<T> g = col_narrow(g0);
   k_col_inv<T><<<g.H >> g.ltc, col_threads(g), col_smem(g, 1), s>>>(g, in, out, scale);
 }
@@ -2523,10 +2645,14 @@ template <typename T, typename Tin>
 void col_grad(const Geo<T>& g0, int mode, cx<Tin>* in, const cx<T>* rvec, cx<T>* dio,
               const cx<float>* delta, cx<T>* Gx, cx<T>* Gy, SolveState* st, int check_done,
               cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value && std::is_same<Tin, double>::value)
+    if (g0.fx)
+      return col_grad<fx64, fx64>(as_fx(g0), mode, fxp(in), fxp(rvec), fxp(dio), delta, fxp(Gx),
+                                  fxp(Gy), st, check_done, s);
   // the whole tile; the persistent passes at most 512 threads
   const Geo<T> g = g0.pipe ? col_narrow(g0) : g0;
   const int nb = g.H >> g.ltc, nt = col_threads(g);
-  const size_t sm = col_smem(g, 2);
+  const size_t sm = col_smem(g, seq_fields<T>() ? 1 : 2);
   if constexpr (std::is_same<T, Tin>::value) {
     if (g.pipe) {
       const size_t ps = pipe_smem(g);
@@ -2554,6 +2680,10 @@ template <typename T>
 void col_div(const Geo<T>& g0, int mode, const cx<T>* Qx, const cx<T>* Qy, const cx<T>* d,
              const cx<T>* b, cx<T>* out, cx<float>* r32, cx<float>* delta32, SolveState* st,
              cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g0.fx)
+      return col_div<fx64>(as_fx(g0), mode, fxp(Qx), fxp(Qy), fxp(d), fxp(b), fxp(out), r32, delta32,
+                           st, s);
   // the whole tile; the persistent passes at most 512 threads
   const Geo<T> g = g0.pipe ? col_narrow(g0) : g0;
   const int nb = g.H >> g.ltc, nt = col_threads(g);
@@ -2603,6 +2733,8 @@ void col_div(const Geo<T>& g0, int mode, const cx<T>* Qx, const cx<T>* Qy, const
 }
 template <typename T>
 void col_heat(const Geo<T>& g0, cx<T>* Mx, cx<T>* My, SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g0.fx) return col_heat<fx64>(as_fx(g0), fxp(Mx), fxp(My), st, s);
   // the whole tile (one slab); the persistent pass at most 512 threads
   const Geo<T> g = g0.pipe ? col_narrow(g0) : g0;
   if (g.pipe) {
@@ -2614,6 +2746,9 @@ void col_heat(const Geo<T>& g0, cx<T>* Mx, cx<T>* My, SolveState* st, cudaStream
 template <typename T>
 void col_gradnorm(const Geo<T>& g0, const cx<T>* Mx, const cx<T>* My, SolveState* st, int into_next,
                   cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g0.fx)
+      return col_gradnorm<fx64>(as_fx(g0), fxp(Mx), fxp(My), st, into_next, s);
   const Geo<T> g = col_narrow(g0);
   k_col_gradnorm<T><<<g.H >> g.ltc, col_threads(g), col_smem(g, 2), s>>>(g, Mx, My, st, into_next);
 }
@@ -2638,6 +2773,10 @@ template <typename T>
 void row_adj_point(const Geo<T>& g, cx<T>* G0, cx<T>* G1, const cx<T>* L0, const cx<T>* L1,
                    const T* mx, const T* my, T* lmx, T* lmy, SplitCoef cf, AdjState* as,
                    cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return row_adj_point<fx64>(as_fx(g), fxp(G0), fxp(G1), fxp(L0), fxp(L1), fxp(mx), fxp(my),
+                                 fxp(lmx), fxp(lmy), cf, as, s);
   k_row_adj_point<T><<<g.ny >> g.lrpc, row_threads(g), 2 * row_smem(g), s>>>(g, G0, G1, L0, L1, mx,
                                                                              my, lmx, lmy, cf, as);
 }
@@ -2645,12 +2784,19 @@ template <typename T>
 void row_adj_press(const Geo<T>& g, const cx<T>* GM0, const cx<T>* GM1, const cx<T>* GP0,
                    const cx<T>* GP1, const T* mx, const T* my, const T* lmx, const T* lmy, T* lx,
                    T* ly, double* dr, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return row_adj_press<fx64>(as_fx(g), fxp(GM0), fxp(GM1), fxp(GP0), fxp(GP1), fxp(mx), fxp(my),
+                                 fxp(lmx), fxp(lmy), fxp(lx), fxp(ly), dr, s);
   k_row_adj_press<T><<<g.ny >> g.lrpc, row_threads(g), 2 * row_smem(g), s>>>(
       g, GM0, GM1, GP0, GP1, mx, my, lmx, lmy, lx, ly, dr);
 }
 template <typename T>
 void col_lap_dot(const Geo<T>& g0, const cx<T>* A, const cx<T>* B, double dt, AdjState* as,
                  cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g0.fx)
+      return col_lap_dot<fx64>(as_fx(g0), fxp(A), fxp(B), dt, as, s);
   const Geo<T> g = col_narrow(g0);
   k_col_lap_dot<T><<<g.H >> g.ltc, col_threads(g), col_smem(g, 2), s>>>(g, A, B, dt, as);
 }
@@ -2719,5 +2865,38 @@ void set_smem_limits_grad() {
   allow_smem(k_col_grad<T, Tin, CG_DUPDATE>);
   allow_smem(k_col_grad<T, Tin, CG_ADDDELTA>);
 }
+
+#ifndef HC_FX_UNIT  // the fx64 kernels are instantiated in hc_kernels_fx.cu
+extern template void row_r2c<fx64>(const Geo<fx64>&, const fx64*, const fx64*, cx<fx64>*,
+                              cx<fx64>*, cudaStream_t);
+extern template void row_c2r<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, fx64*,
+                              fx64*, SolveState*, int, cudaStream_t);
+extern template void row_apply<fx64, fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*,
+                                        const fx64*, const fx64*, const fx64*, cx<fx64>*,
+                                        cx<fx64>*, SolveState*, cudaStream_t);
+extern template void row_split<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, const fx64*,
+                               const fx64*, const fx64*, cx<fx64>*, cx<fx64>*, SplitCoef, SolveState*,
+                               cudaStream_t);
+extern template void col_fwd<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, cx<fx64>*,
+                              cx<fx64>*, int, int, SolveState*, cudaStream_t);
+extern template void col_inv<fx64>(const Geo<fx64>&, const cx<fx64>*, cx<fx64>*, fx64,
+                              cudaStream_t);
+extern template void col_grad<fx64, fx64>(const Geo<fx64>&, int, cx<fx64>*, const cx<fx64>*,
+                                       cx<fx64>*, const cx<float>*, cx<fx64>*, cx<fx64>*,
+                                       SolveState*, int, cudaStream_t);
+extern template void col_div<fx64>(const Geo<fx64>&, int, const cx<fx64>*, const cx<fx64>*,
+                              const cx<fx64>*, const cx<fx64>*, cx<fx64>*, cx<float>*,
+                              cx<float>*, SolveState*, cudaStream_t);
+extern template void col_heat<fx64>(const Geo<fx64>&, cx<fx64>*, cx<fx64>*, SolveState*, cudaStream_t);
+extern template void col_gradnorm<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, SolveState*, int,
+                                 cudaStream_t);
+extern template void row_adj_point<fx64>(const Geo<fx64>&, cx<fx64>*, cx<fx64>*, const cx<fx64>*, const cx<fx64>*,
+                                const fx64*, const fx64*, fx64*, fx64*, SplitCoef, AdjState*, cudaStream_t);
+extern template void row_adj_press<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, const cx<fx64>*,
+                                const cx<fx64>*, const fx64*, const fx64*, const fx64*, const fx64*, fx64*,
+                                fx64*, double*, cudaStream_t);
+extern template void col_lap_dot<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, double, AdjState*,
+                              cudaStream_t);
+#endif
 
 }  // namespace hc

@@ -138,9 +138,19 @@ __device__ __forceinline__ void load_rows3(cx<T> (&v)[3][8], const Tri<cx<T>*>& 
   load_rows_c2r<3>(v, A3, B3, r.j, r.N8);
 }
 
+// Transform q of the three alone.
+template <typename T>
+__device__ __forceinline__ void load_row3(cx<T> (&v)[1][8], const Tri<cx<T>*>& G, const RIdx3& r,
+                                          int H, int q) {
+  const size_t o0 = r.y0 * H, o1 = r.y1 * H;
+  const cx<T>* const A[1] = {q == 0 ? G.v[0] + o0 : (q == 1 ? G.v[0] + o1 : G.v[2] + o0)};
+  const cx<T>* const B[1] = {q == 0 ? G.v[1] + o0 : (q == 1 ? G.v[1] + o1 : G.v[2] + o1)};
+  load_rows_c2r<1>(v, A, B, r.j, r.N8);
+}
+
 // ------------------------------------------------------------------ z pass: gradient
 template <typename T, typename Tin, int MODE>
-__global__ void __launch_bounds__(256) k3_zgrad(Geo<T> g, cx<Tin>* in, const cx<T>* __restrict__ rvec,
+__global__ void __launch_bounds__(cta_bound<T>(256)) k3_zgrad(Geo<T> g, cx<Tin>* in, const cx<T>* __restrict__ rvec,
                                                 cx<T>* dio, const cx<float>* __restrict__ delta,
                                                 Tri<cx<T>*> G, SolveState* st, int check_done) {
   if (check_done && st->done) return;
@@ -162,6 +172,37 @@ __global__ void __launch_bounds__(256) k3_zgrad(Geo<T> g, cx<Tin>* in, const cx<
     pc = pc_of<T>(st);
   }
   if (MODE == CG_ADDDELTA) add_delta = st->sweeps > 0;
+  if constexpr (seq_fields<T>()) {
+#pragma unroll 1
+    for (int q = 0; q < 3; ++q) {
+      cx<T> v[1][8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const int kz = c.j + s * c.L8;
+        const size_t idx = c.base + (size_t)kz * (size_t)p.stride;
+        cx<T> P;
+        if (q > 0) {  // the value this thread has just updated
+          P = MODE == CG_DUPDATE ? dio[idx] : ccast<T>(in[idx]);
+        } else if constexpr (MODE == CG_PLAIN) {
+          P = ccast<T>(in[idx]);
+        } else if constexpr (MODE == CG_DUPDATE) {
+          const cx<T> z = cscale(rvec[idx], pinv3(g, kx, ky, kz, pc));
+          P = first ? z : cadd(z, cscale(dio[idx], beta));
+          dio[idx] = P;
+        } else {
+          P = add_delta ? add_delta_at<T>(in, idx, delta[idx]) : ccast<T>(in[idx]);
+        }
+        const T a = q == 0 ? ax : (q == 1 ? ay : g.kzd[kz] * invn);
+        v[0][s] = cmk<T>(-a * P.y, a * P.x);  // i (k/n) P
+      }
+      cx<T>* const sl1[1] = {sl[0]};
+      fft_canon<+1, 1>(v, sl1, 1 << p.ltc, c.j, p.lL, g.twz);
+      cx<T>* const Gq = q == 0 ? G.v[0] : (q == 1 ? G.v[1] : G.v[2]);
+#pragma unroll
+      for (int s = 0; s < 8; ++s) Gq[c.base + (size_t)(c.j + s * c.L8) * (size_t)p.stride] = v[0][s];
+    }
+    return;
+  }
   cx<T> v[3][8];
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
@@ -194,7 +235,7 @@ __global__ void __launch_bounds__(256) k3_zgrad(Geo<T> g, cx<Tin>* in, const cx<
 
 // ------------------------------------------------------------------ plain axis FFT
 template <typename T, int S, int NV>
-__global__ void __launch_bounds__(256) k3_axis_fft(Geo<T> g, int axis, Tri<cx<T>*> in,
+__global__ void __launch_bounds__(cta_bound<T>(256)) k3_axis_fft(Geo<T> g, int axis, Tri<cx<T>*> in,
                                                    Tri<cx<T>*> out, T scale) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
@@ -202,6 +243,24 @@ __global__ void __launch_bounds__(256) k3_axis_fft(Geo<T> g, int axis, Tri<cx<T>
   const cx<T>* tw = axis == 1 ? g.twy : g.twz;
   const CIdx3 c = cidx3(p);
   const int se = slab3(p);
+  if constexpr (seq_fields<T>()) {
+#pragma unroll 1
+    for (int q = 0; q < NV; ++q) {
+      const cx<T>* const src = q == 0 ? in.v[0] : (q == 1 ? in.v[1] : in.v[2]);
+      cx<T>* const dst = q == 0 ? out.v[0] : (q == 1 ? out.v[1] : out.v[2]);
+      cx<T>* const sl1[1] = {sm + c.b};
+      cx<T> v[1][8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) v[0][s] = src[c.base + (size_t)(c.j + s * c.L8) * (size_t)p.stride];
+      fft_canon<S, 1>(v, sl1, 1 << p.ltc, c.j, p.lL, tw);
+      const bool sc = scale != (T)1;
+#pragma unroll
+      for (int s = 0; s < 8; ++s)
+        dst[c.base + (size_t)(c.j + s * c.L8) * (size_t)p.stride] =
+            sc ? cscale(v[0][s], scale) : v[0][s];
+    }
+    return;
+  }
   cx<T>* sl[NV];
 #pragma unroll
   for (int q = 0; q < NV; ++q) sl[q] = sm + q * se + c.b;
@@ -225,7 +284,7 @@ __global__ void __launch_bounds__(256) k3_axis_fft(Geo<T> g, int axis, Tri<cx<T>
 // Forward z FFT of one field, projection of the corner modes (packed x column,
 // ky in {0, ny/2}, kz in {0, nz/2}), and ||.||^2 with Parseval weights.
 template <typename T>
-__global__ void __launch_bounds__(256) k3_zfwd_project(Geo<T> g, const cx<T>* in, cx<T>* out,
+__global__ void __launch_bounds__(cta_bound<T>(256)) k3_zfwd_project(Geo<T> g, const cx<T>* in, cx<T>* out,
                                                        SolveState* st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
@@ -256,7 +315,7 @@ __global__ void __launch_bounds__(256) k3_zfwd_project(Geo<T> g, const cx<T>* in
 
 // ------------------------------------------------------------------ z pass: divergence
 template <typename T, int MODE>
-__global__ void __launch_bounds__(256) k3_zdiv(Geo<T> g, Tri<cx<T>*> Q, const cx<T>* __restrict__ d,
+__global__ void __launch_bounds__(cta_bound<T>(256)) k3_zdiv(Geo<T> g, Tri<cx<T>*> Q, const cx<T>* __restrict__ d,
                                                const cx<T>* __restrict__ bvec,
                                                cx<T>* __restrict__ out, cx<float>* __restrict__ r32,
                                                cx<float>* __restrict__ delta32, SolveState* st) {
@@ -267,14 +326,37 @@ __global__ void __launch_bounds__(256) k3_zdiv(Geo<T> g, Tri<cx<T>*> Q, const cx
   const CIdx3 c = cidx3(p);
   const int se = slab3(p);
   cx<T>* const sl[3] = {sm + c.b, sm + se + c.b, sm + 2 * se + c.b};
-  cx<T> v[3][8];
+  if constexpr (seq_fields<T>()) {
+    // xi . Q adds up in this thread's own slots of the second slab
+    const T ax = g.kxd[c.col & (g.H - 1)], ay = g.kyd[c.col >> g.lH];
+#pragma unroll 1
+    for (int q = 0; q < 3; ++q) {
+      const cx<T>* const src = q == 0 ? Q.v[0] : (q == 1 ? Q.v[1] : Q.v[2]);
+      cx<T> v[1][8];
 #pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const size_t idx = c.base + (size_t)(c.j + s * c.L8) * (size_t)p.stride;
+      for (int s = 0; s < 8; ++s) v[0][s] = src[c.base + (size_t)(c.j + s * c.L8) * (size_t)p.stride];
+      cx<T>* const sl1[1] = {sl[0]};
+      fft_canon<-1, 1>(v, sl1, 1 << p.ltc, c.j, p.lL, g.twz);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) v[q][s] = Q.v[q][idx];
+      for (int s = 0; s < 8; ++s) {
+        const int kz = c.j + s * c.L8;
+        cx<T>& t = sl[1][padk(kz) << p.ltc];
+        const T a = q == 0 ? ax : (q == 1 ? ay : g.kzd[kz]);
+        if (q == 0) t = cscale(v[0][s], a);
+        else t = cmk<T>(t.x + a * v[0][s].x, t.y + a * v[0][s].y);
+      }
+    }
   }
-  fft_canon<-1, 3>(v, sl, 1 << p.ltc, c.j, p.lL, g.twz);
+  cx<T> v[3][8];
+  if constexpr (!seq_fields<T>()) {
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const size_t idx = c.base + (size_t)(c.j + s * c.L8) * (size_t)p.stride;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) v[q][s] = Q.v[q][idx];
+    }
+    fft_canon<-1, 3>(v, sl, 1 << p.ltc, c.j, p.lL, g.twz);
+  }
   const int kx = c.col & (g.H - 1), ky = c.col >> g.lH;
   const T ax = g.kxd[kx], ay = g.kyd[ky];
   const double w = kx == 0 ? 1.0 : 2.0;  // Parseval weight of a packed column
@@ -289,9 +371,14 @@ __global__ void __launch_bounds__(256) k3_zdiv(Geo<T> g, Tri<cx<T>*> Q, const cx
   for (int s = 0; s < 8; ++s) {
     const int kz = c.j + s * c.L8;
     const size_t idx = c.base + (size_t)kz * (size_t)p.stride;
-    const T az = g.kzd[kz];
-    const cx<T> t = cmk<T>(ax * v[0][s].x + ay * v[1][s].x + az * v[2][s].x,
-                           ax * v[0][s].y + ay * v[1][s].y + az * v[2][s].y);
+    cx<T> t;
+    if constexpr (seq_fields<T>()) {
+      t = sl[1][padk(kz) << p.ltc];
+    } else {
+      const T az = g.kzd[kz];
+      t = cmk<T>(ax * v[0][s].x + ay * v[1][s].x + az * v[2][s].x,
+                 ax * v[0][s].y + ay * v[1][s].y + az * v[2][s].y);
+    }
     const cx<T> q = cmk<T>(t.y, -t.x);  // -i xi . Q
     if constexpr (MODE == CD_PLAIN) {
       out[idx] = q;
@@ -350,7 +437,7 @@ __global__ void __launch_bounds__(256) k3_zdiv(Geo<T> g, Tri<cx<T>*> Q, const cx
 // ------------------------------------------------------------------ row pairs
 // DOT: the CG variant, alpha = rho / (n sum g . K g) as in the 2D row pass.
 template <typename T, typename Tm, bool DOT>
-__global__ void __launch_bounds__(256) k3_row_apply(Geo<T> g, Tri<cx<T>*> G, Tri<const Tm*> m,
+__global__ void __launch_bounds__(cta_bound<T>(256)) k3_row_apply(Geo<T> g, Tri<cx<T>*> G, Tri<const Tm*> m,
                                                     const Tm* __restrict__ rr, Tri<cx<T>*> Q,
                                                     SolveState* st) {
   if (st && st->done) return;
@@ -359,6 +446,51 @@ __global__ void __launch_bounds__(256) k3_row_apply(Geo<T> g, Tri<cx<T>*> G, Tri
   const RIdx3 r = ridx3(g);
   const int N = g.nx, H = g.H;
   cx<T>* const sl[3] = {sm + (3 * r.u) * N, sm + (3 * r.u + 1) * N, sm + (3 * r.u + 2) * N};
+  if constexpr (seq_fields<T>()) {
+    // one transform at a time; between the two directions the three wait in
+    // this thread's own slots of their slabs
+#pragma unroll 1
+    for (int q = 0; q < 3; ++q) {
+      cx<T> v[1][8];
+      load_row3(v, G, r, H, q);
+      cx<T>* const sl1[1] = {sm + (3 * r.u + q) * N};
+      fft_canon<+1, 1, true>(v, sl1, 1, r.j, g.lnx, g.twx);
+      __syncthreads();
+#pragma unroll
+      for (int s = 0; s < 8; ++s) sl1[0][rswz<T>(r.j + s * r.N8)] = v[0][s];
+    }
+    DotAcc<T> gkg;
+#pragma unroll 1
+    for (int i = 0; i < 16; ++i) {  // points of the two rows
+      const int x = r.j + (i >> 1) * r.N8, row = i & 1, e = rswz<T>(x);
+      const size_t o = (row == 0 ? r.y0 : r.y1) * N + x;
+      cx<T>& xy = sl[0][row * N + e];
+      T& z = reinterpret_cast<T*>(&sl[2][e])[row];
+      const T gx = xy.x, gy = xy.y, gz = z;
+      const T ax = (T)m.v[0][o], ay = (T)m.v[1][o], az = (T)m.v[2][o], rv = (T)rr[o];
+      const T mg = ax * gx + ay * gy + az * gz;
+      if (DOT) gkg.add_prod(mg * mg + rv * (gx * gx + gy * gy + gz * gz), (T)1);
+      xy = cmk<T>(ax * mg + rv * gx, ay * mg + rv * gy);
+      z = az * mg + rv * gz;
+    }
+    const size_t s0 = r.y0 * H, s1 = r.y1 * H;
+#pragma unroll 1
+    for (int q = 0; q < 3; ++q) {
+      cx<T>* const sl1[1] = {sm + (3 * r.u + q) * N};
+      cx<T> v[1][8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) v[0][s] = sl1[0][rswz<T>(r.j + s * r.N8)];
+      cx<T>* const A[1] = {q == 0 ? Q.v[0] + s0 : (q == 1 ? Q.v[0] + s1 : Q.v[2] + s0)};
+      cx<T>* const B[1] = {q == 0 ? Q.v[1] + s0 : (q == 1 ? Q.v[1] + s1 : Q.v[2] + s1)};
+      fft_rows_r2c<1>(v, sl1, r.j, g.lnx, g.twx, A, B);
+    }
+    if (DOT) {
+      double a1[1] = {gkg.value()}, t1[1];
+      if (last_cta_sum<1>(a1, g.partials, &st->ticket[TK_DIV], t1) && threadIdx.x == 0)
+        cg_alpha_from(st, t1[0], (double)g.nx * (double)g.ny * (double)g.nz);
+    }
+    return;
+  }
   cx<T> v[3][8];
   load_rows3(v, G, r, H);
   fft_canon<+1, 3, true>(v, sl, 1, r.j, g.lnx, g.twx);
@@ -704,8 +836,12 @@ template <typename T, typename Tin>
 void z_grad(const Geo<T>& g, int mode, cx<Tin>* in, const cx<T>* rvec, cx<T>* dio,
             const cx<float>* delta, Tri<cx<T>*> G, SolveState* st, int check_done,
             cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value && std::is_same<Tin, double>::value)
+    if (g.fx)
+      return z_grad<fx64, fx64>(as_fx(g), mode, fxp(in), fxp(rvec), fxp(dio), delta, fxp(G), st,
+                                check_done, s);
   const int nb = pass_ctas(g.pz), nt = pass_threads(g.pz);
-  const size_t sm = pass_smem<T>(g.pz, 3);
+  const size_t sm = pass_smem<T>(g.pz, seq_fields<T>() ? 1 : 3);
   if (mode == CG_PLAIN)
     k3_zgrad<T, Tin, CG_PLAIN><<<nb, nt, sm, s>>>(g, in, rvec, dio, delta, G, st, check_done);
   else if (mode == CG_DUPDATE)
@@ -716,9 +852,12 @@ void z_grad(const Geo<T>& g, int mode, cx<Tin>* in, const cx<T>* rvec, cx<T>* di
 template <typename T>
 void axis_fft(const Geo<T>& g, int axis, int sign, int nv, Tri<cx<T>*> in, Tri<cx<T>*> out,
               T scale, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return axis_fft<fx64>(as_fx(g), axis, sign, nv, fxp(in), fxp(out), fx64(scale), s);
   const ColPass& p = axis == 1 ? g.py : g.pz;
   const int nb = pass_ctas(p), nt = pass_threads(p);
-  const size_t sm = pass_smem<T>(p, nv);
+  const size_t sm = pass_smem<T>(p, seq_fields<T>() ? 1 : nv);
   if (sign < 0) {
     if (nv == 1) k3_axis_fft<T, -1, 1><<<nb, nt, sm, s>>>(g, axis, in, out, scale);
     else k3_axis_fft<T, -1, 3><<<nb, nt, sm, s>>>(g, axis, in, out, scale);
@@ -729,14 +868,20 @@ void axis_fft(const Geo<T>& g, int axis, int sign, int nv, Tri<cx<T>*> in, Tri<c
 }
 template <typename T>
 void z_fwd_project(const Geo<T>& g, const cx<T>* in, cx<T>* out, SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return z_fwd_project<fx64>(as_fx(g), fxp(in), fxp(out), st, s);
   k3_zfwd_project<T><<<pass_ctas(g.pz), pass_threads(g.pz), pass_smem<T>(g.pz, 1), s>>>(g, in, out,
                                                                                         st);
 }
 template <typename T>
 void z_div(const Geo<T>& g, int mode, Tri<cx<T>*> Q, const cx<T>* d, const cx<T>* b, cx<T>* out,
            cx<float>* r32, cx<float>* delta32, SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return z_div<fx64>(as_fx(g), mode, fxp(Q), fxp(d), fxp(b), fxp(out), r32, delta32, st, s);
   const int nb = pass_ctas(g.pz), nt = pass_threads(g.pz);
-  const size_t sm = pass_smem<T>(g.pz, 3);
+  const size_t sm = pass_smem<T>(g.pz, seq_fields<T>() ? 2 : 3);
   switch (mode) {
     case CD_PLAIN:
       k3_zdiv<T, CD_PLAIN><<<nb, nt, sm, s>>>(g, Q, d, b, out, r32, delta32, st);
@@ -759,6 +904,9 @@ void z_div(const Geo<T>& g, int mode, Tri<cx<T>*> Q, const cx<T>* d, const cx<T>
 template <typename T, typename Tm>
 void row_apply3(const Geo<T>& g, Tri<cx<T>*> G, Tri<const Tm*> m, const Tm* r, Tri<cx<T>*> Q,
                 SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value && std::is_same<Tm, double>::value)
+    if (g.fx)
+      return row_apply3<fx64, fx64>(as_fx(g), fxp(G), fxp(m), fxp(r), fxp(Q), st, s);
   if (st)
     k3_row_apply<T, Tm, true><<<row3_ctas(g), row3_threads(g), row3_smem(g), s>>>(g, G, m, r, Q, st);
   else
@@ -767,10 +915,16 @@ void row_apply3(const Geo<T>& g, Tri<cx<T>*> G, Tri<const Tm*> m, const Tm* r, T
 template <typename T>
 void row_split3(const Geo<T>& g, Tri<cx<T>*> G, Tri<const T*> m, const T* r, Tri<T*> mo,
                 SplitCoef cf, SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return row_split3<fx64>(as_fx(g), fxp(G), fxp(m), fxp(r), fxp(mo), cf, st, s);
   k3_row_split<T><<<row3_ctas(g), row3_threads(g), row3_smem(g), s>>>(g, G, m, r, mo, cf, st);
 }
 template <typename T>
 void heat_axis(const Geo<T>& g, int axis, Tri<T*> mi, Tri<T*> mo, SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return heat_axis<fx64>(as_fx(g), axis, fxp(mi), fxp(mo), st, s);
   const ColPass& p = axis == 1 ? g.py : g.pz;
   Tri<cx<T>*> Mi = {{reinterpret_cast<cx<T>*>(mi.v[0]), reinterpret_cast<cx<T>*>(mi.v[1]),
                      reinterpret_cast<cx<T>*>(mi.v[2])}};
@@ -780,6 +934,9 @@ void heat_axis(const Geo<T>& g, int axis, Tri<T*> mi, Tri<T*> mo, SolveState* st
 }
 template <typename T>
 void z_gradnorm(const Geo<T>& g, Tri<cx<T>*> G, SolveState* st, int into_next, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value)
+    if (g.fx)
+      return z_gradnorm<fx64>(as_fx(g), fxp(G), st, into_next, s);
   k3_zgradnorm<T><<<pass_ctas(g.pz), pass_threads(g.pz), pass_smem<T>(g.pz, 3), s>>>(g, G, st,
                                                                                      into_next);
 }
@@ -820,5 +977,29 @@ void set_smem_limits_zgrad() {
   allow_smem(k3_zgrad<T, Tin, CG_DUPDATE>);
   allow_smem(k3_zgrad<T, Tin, CG_ADDDELTA>);
 }
+
+#ifndef HC_FX_UNIT  // the fx64 kernels are instantiated in hc_kernels3d_fx.cu
+extern template void z_grad<fx64, fx64>(const Geo<fx64>&, int, cx<fx64>*, const cx<fx64>*,
+                                     cx<fx64>*, const cx<float>*, Tri<cx<fx64>*>, SolveState*,
+                                     int, cudaStream_t);
+extern template void axis_fft<fx64>(const Geo<fx64>&, int, int, int, Tri<cx<fx64>*>,
+                               Tri<cx<fx64>*>, fx64, cudaStream_t);
+extern template void z_fwd_project<fx64>(const Geo<fx64>&, const cx<fx64>*, cx<fx64>*, SolveState*,
+                                    cudaStream_t);
+extern template void z_div<fx64>(const Geo<fx64>&, int, Tri<cx<fx64>*>, const cx<fx64>*,
+                            const cx<fx64>*, cx<fx64>*, cx<float>*, cx<float>*, SolveState*,
+                            cudaStream_t);
+extern template void row_apply3<fx64, fx64>(const Geo<fx64>&, Tri<cx<fx64>*>, Tri<const fx64*>,
+                                         const fx64*, Tri<cx<fx64>*>, SolveState*,
+                                         cudaStream_t);
+extern template void row_apply3<fx64, float>(const Geo<fx64>&, Tri<cx<fx64>*>, Tri<const float*>,
+                                        const float*, Tri<cx<fx64>*>, SolveState*,
+                                        cudaStream_t);
+extern template void row_split3<fx64>(const Geo<fx64>&, Tri<cx<fx64>*>, Tri<const fx64*>, const fx64*,
+                                Tri<fx64*>, SplitCoef, SolveState*, cudaStream_t);
+extern template void heat_axis<fx64>(const Geo<fx64>&, int, Tri<fx64*>, Tri<fx64*>, SolveState*,
+                               cudaStream_t);
+extern template void z_gradnorm<fx64>(const Geo<fx64>&, Tri<cx<fx64>*>, SolveState*, int, cudaStream_t);
+#endif
 
 }  // namespace hc

@@ -22,6 +22,8 @@
 namespace {
 
 using hc::cx;
+using hc::fx64;
+using hc::FxTw;
 
 constexpr int kMaxDevices = 64;
 constexpr size_t kInterBytes = (size_t)HC_NOALLOC_MAX_POINTS / 2 * sizeof(cx<double>);
@@ -34,14 +36,16 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kInterBytes + 2
 std::mutex g_mu;
 void* g_addr[kMaxDevices];  // device address of g_noalloc_scratch per device (set-up done)
 
-// tw[m] = exp(-2 pi i m / N), m < N.
-__global__ void k_noalloc_twiddles(cx<double>* tw, int N) {
+// tw[m] = exp(-2 pi i m / N), m < N: Q62, or FP64 below the fixed-point lengths.
+__global__ void k_noalloc_twiddles(FxTw* tw, int N) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= N) return;
   double s, c;
   sincospi(2.0 * (double)m / (double)N, &s, &c);
-  tw[m].x = c;
-  tw[m].y = -s;
+  if (N >= (1 << hc::kFxMinLog))
+    tw[m] = hc::fx_twiddle(__double2ll_rn(c * 0x1p62), __double2ll_rn(s * -0x1p62));
+  else
+    reinterpret_cast<double2*>(tw)[m] = make_double2(c, -s);
 }
 
 int ilog2i(int v) {
@@ -62,8 +66,8 @@ int setup_device(int dev, void** addr) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return HC_ECUDA;
     cudaGetLastError();  // a pending error of earlier work is not this set-up's
-    hc::allow_smem(hc::k_row_r2c<double>);
-    hc::allow_smem(hc::k_col_fwd<double, 1>);
+    hc::allow_smem(hc::k_row_r2c<fx64>);
+    hc::allow_smem(hc::k_col_fwd<fx64, 1>);
     if (cudaGetLastError() != cudaSuccess) return HC_ECUDA;
     g_addr[dev] = p;
   }
@@ -88,11 +92,11 @@ extern "C" int hc_spectrum_noalloc(const double* f, double* out, int nx, int ny,
   // the launches reports only this call's own launches.
   cudaGetLastError();
   unsigned char* b = static_cast<unsigned char*>(base);
-  cx<double>* inter = reinterpret_cast<cx<double>*>(b);
-  cx<double>* twx = reinterpret_cast<cx<double>*>(b + kInterBytes);
-  cx<double>* twy = reinterpret_cast<cx<double>*>(b + kInterBytes + kTwBytes);
+  cx<fx64>* inter = reinterpret_cast<cx<fx64>*>(b);
+  FxTw* twx = reinterpret_cast<FxTw*>(b + kInterBytes);
+  FxTw* twy = reinterpret_cast<FxTw*>(b + kInterBytes + kTwBytes);
 
-  hc::Geo<double> g = {};
+  hc::Geo<fx64> g = {};
   g.nx = nx;
   g.ny = ny;
   g.H = nx / 2;
@@ -109,18 +113,18 @@ extern "C" int hc_spectrum_noalloc(const double* f, double* out, int nx, int ny,
   if (rpc > ny) rpc = ny;
   g.rpc = rpc;
   g.lrpc = ilog2i(rpc);
-  g.twx = twx;
-  g.twy = twy;
+  g.twx = reinterpret_cast<const cx<fx64>*>(twx);
+  g.twy = reinterpret_cast<const cx<fx64>*>(twy);
 
   // Every call rewrites the tables and the whole intermediate before reading
   // them, so nothing carried over from an earlier call is used.
   k_noalloc_twiddles<<<(nx + 255) / 256, 256, 0, s>>>(twx, nx);
   k_noalloc_twiddles<<<(ny + 255) / 256, 256, 0, s>>>(twy, ny);
-  hc::k_row_r2c<double><<<ny >> g.lrpc, rpc << (g.lnx - 3), (size_t)rpc * nx * sizeof(cx<double>), s>>>(
-      g, f, nullptr, inter, nullptr);
-  hc::k_col_fwd<double, 1><<<g.H >> g.ltc, tc << (g.lny - 3),
+  hc::k_row_r2c<fx64><<<ny >> g.lrpc, rpc << (g.lnx - 3), (size_t)rpc * nx * sizeof(cx<double>), s>>>(
+      g, hc::fxp(f), nullptr, inter, nullptr);
+  hc::k_col_fwd<fx64, 1><<<g.H >> g.ltc, tc << (g.lny - 3),
                              (size_t)(ny + (ny >> 3)) * tc * sizeof(cx<double>), s>>>(
-      g, inter, nullptr, reinterpret_cast<cx<double>*>(out), nullptr, 0, nullptr);
+      g, inter, nullptr, reinterpret_cast<cx<fx64>*>(out), nullptr, 0, nullptr);
   if (cudaGetLastError() != cudaSuccess) return HC_ECUDA;
   return HC_OK;
 }

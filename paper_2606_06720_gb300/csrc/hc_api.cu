@@ -110,9 +110,10 @@ int ilog2(int v) {
 
 // Conditional handles of one step chain: the CG loop of the refinement sweeps
 // (or of plain PCG), the refinement loop, the first (FP32-started) inner loop,
-// and the mid-step residual block (IF) with its inner loop.
+// the mid-step residual block (IF) with its inner loop, the refinement loop's fx64
+// residual (IF) and its FP64 residual with the sweep that follows (IF).
 struct Handles {
-  cudaGraphConditionalHandle inner = 0, outer = 0, first = 0, mid = 0, mid_inner = 0;
+  cudaGraphConditionalHandle inner = 0, outer = 0, first = 0, mid = 0, mid_inner = 0, dec = 0, again = 0;
 };
 
 struct hc_ctx {
@@ -955,6 +956,32 @@ void first_resid32(hc_ctx* c) {
   c->launches += 3;
 }
 
+// Whether the refinement loop's residual may come from the fx64 kernels
+// (predict_residual): with the default residual switches.
+bool decide_on(const hc_ctx* c) { return c->refined && !c->df && c->mid_df; }
+
+// p64 += delta, then ||S - A p64|| by the fx64 kernels, which ends the loop or
+// asks for refined_resid (resid_decide).
+void refined_decide(hc_ctx* c) {
+  hc::Geo<double> g = fx_geo(c->gd);
+  if (c->dim == 3) {
+    apply3_open<double, double, float>(c, g, hc::CG_ADDDELTA, c->p64, nullptr, nullptr, c->G64, 0);
+    hc::z_div<double>(g, hc::CD_DECIDE, tri(c->G64, c->ns), nullptr, c->b64, nullptr, nullptr, nullptr,
+                      c->st, c->stream);
+    c->launches += 1;
+    return;
+  }
+  cx<double>* Gx = c->G64;
+  cx<double>* Gy = c->G64 + c->ns;
+  hc::col_grad<double, double>(g, hc::CG_ADDDELTA, c->p64, nullptr, nullptr, c->x32, Gx, Gy, c->st, 0,
+                               c->stream);
+  hc::row_apply<double, float>(g, Gx, Gy, (const float*)c->m[0], (const float*)c->m[1],
+                               (const float*)c->rf, Gx, Gy, nullptr, c->stream);
+  hc::col_div<double>(g, hc::CD_DECIDE, Gx, Gy, nullptr, c->b64, nullptr, nullptr, nullptr, c->st,
+                      c->stream);
+  c->launches += 3;
+}
+
 // FP64 residual S - A p64 (after p64 += delta) and inner-CG initialisation.
 void refined_resid(hc_ctx* c) {
   if (c->dim == 3) {
@@ -1240,6 +1267,12 @@ int step_host(hc_ctx* c) {
       }
     }
     for (int sweep = 0;; ++sweep) {
+      if (c->st_host->res_dec) {
+        refined_decide(c);
+        rc = read_state(c);
+        if (rc) return rc;
+        if (c->st_host->outer_done) break;
+      }
       refined_resid(c);
       rc = read_state(c);
       if (rc) return rc;
@@ -1271,7 +1304,8 @@ int step_host(hc_ctx* c) {
 //   plain:   step_begin, initial residual, WHILE(inner){CG}, split, step_end
 //   refined: step_begin, FP32 residual, WHILE(first){CG},
 //            [HC_FP32_REFINED: IF(mid){double-float residual, WHILE(mid_inner){CG}}],
-//            WHILE(outer){FP64 residual, WHILE(inner){CG}}, split, step_end
+//            WHILE(outer){IF(dec){fx64 residual}, IF(again){FP64 residual, WHILE(inner){CG}}} with the default
+//            residual switches, else WHILE(outer){FP64 residual, WHILE(inner){CG}}, split, step_end
 int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h) {
   cudaStream_t s = c->stream;
   Handles hh;
@@ -1348,10 +1382,25 @@ int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h) {
     cudaGraph_t obody = nullptr;
     rc = add_while(target, std::vector<cudaGraphNode_t>{first_node}, &hh.outer, &loop_node, &obody);
     if (rc) return rc;
+    std::vector<cudaGraphNode_t> otail;
+    if (decide_on(c)) {  // IF(dec){fx64 residual}, IF(again){the rest of the body}
+      cudaGraphNode_t dec_node, again_node;
+      cudaGraph_t dbody = nullptr, abody = nullptr;
+      rc = add_while(obody, otail, &hh.dec, &dec_node, &dbody, true);
+      if (!rc)
+        rc = add_while(obody, std::vector<cudaGraphNode_t>{dec_node}, &hh.again, &again_node, &abody,
+                       true);
+      if (rc) return rc;
+      CU(cudaStreamBeginCaptureToGraph(s, dbody, nullptr, nullptr, 0,
+                                       cudaStreamCaptureModeThreadLocal));
+      refined_decide(c);
+      rc = end_capture(dbody, otail);
+      if (rc) return rc;
+      obody = abody;
+    }
     CU(cudaStreamBeginCaptureToGraph(s, obody, nullptr, nullptr, 0,
                                      cudaStreamCaptureModeThreadLocal));
     refined_resid(c);
-    std::vector<cudaGraphNode_t> otail;
     rc = end_capture(obody, otail);
     if (rc) return rc;
     cudaGraphNode_t inode;
@@ -1395,7 +1444,8 @@ long long graph_kernel_count(const hc_ctx* c, const hc::SolveState& h) {
   long long n = (long long)c->graph_nodes_fixed * h.acc_steps +
                 (long long)c->graph_nodes_body * h.acc_iters;
   // refinement residuals (FP64 or double-float), the mid-step one included
-  if (c->refined) n += (long long)c->graph_nodes_outer * (h.acc_res_full + h.acc_mid);
+  if (c->refined)
+    n += (long long)c->graph_nodes_outer * (h.acc_res_full + h.acc_mid + h.acc_again);
   return n;
 }
 
@@ -1403,7 +1453,7 @@ long long graph_kernel_count(const hc_ctx* c, const hc::SolveState& h) {
 int use_handles(hc_ctx* c, const Handles& h, cudaGraphConditionalHandle hgate = 0) {
   unsigned long long v[4] = {h.inner, h.outer, hgate, h.first};
   CU(cudaMemcpy(&c->st->h_inner, v, sizeof(v), cudaMemcpyHostToDevice));
-  unsigned long long w[2] = {h.mid, h.mid_inner};
+  unsigned long long w[4] = {h.mid, h.mid_inner, h.dec, h.again};
   CU(cudaMemcpy(&c->st->h_mid, w, sizeof(w), cudaMemcpyHostToDevice));
   return HC_OK;
 }
@@ -1768,7 +1818,8 @@ int step_lagged(hc_ctx* c, int nsteps) {
   c->launches += (long long)c->graph_nodes_fixed * (h2.acc_steps - b2.acc_steps) +
                  (long long)c->graph_nodes_body * (h2.acc_iters - b2.acc_iters) +
                  (long long)c->graph_nodes_outer *
-                     ((h2.acc_res_full - b2.acc_res_full) + (h2.acc_mid - b2.acc_mid));
+                     ((h2.acc_res_full - b2.acc_res_full) + (h2.acc_mid - b2.acc_mid) +
+                      (h2.acc_again - b2.acc_again));
   return HC_OK;
 }
 
@@ -2724,8 +2775,15 @@ int solve_only(hc_ctx* c) {
     return run_cg_host(c, false);
   }
   for (int sweep = 0;; ++sweep) {
+    int rc = HC_OK;
+    if (sweep > 0 && c->st_host->res_dec) {
+      refined_decide(c);
+      rc = read_state(c);
+      if (rc) return rc;
+      if (c->st_host->outer_done) break;
+    }
     refined_resid(c);
-    int rc = read_state(c);
+    rc = read_state(c);
     if (rc) return rc;
     if (c->st_host->outer_done) break;
     rc = run_cg_host(c, true);
@@ -3011,6 +3069,7 @@ hc::BInst member_record(const hc_ctx* c, const hc_ctx* rep) {
   b.gf = class_geo(c->gf, rep->gf);
   b.gfn = hc::col_narrow(b.gf);
   b.gd = class_geo(c->gd, rep->gd);
+  b.gx = hc::as_fx(b.gd);
   b.gq = class_geo(c->gq, rep->gq);
   b.st = c->st;
   b.p64 = c->p64;
@@ -3036,7 +3095,8 @@ hc::BInst member_record(const hc_ctx* c, const hc_ctx* rep) {
 // on what `target` already holds (the batched counterpart of build_chain):
 //   step_begin, FP32 residual, flags, WHILE(first){CG, flags},
 //   IF(mid){double-float residual, flags, WHILE(mid_inner){CG, flags}},
-//   WHILE(outer){FP64 residual, flags, WHILE(inner){CG, flags}}, split, step_end.
+//   WHILE(outer){fx64 residual, flags, IF(again){FP64 residual, flags,
+//   WHILE(inner){CG, flags}}}, split, step_end.
 // Every conditional handle is created before the kernels that set it are
 // captured; flags sets each to the OR over the members.
 int build_class_chain(const BatchClass& bc, cudaStream_t s, cudaGraph_t target) {
@@ -3111,14 +3171,23 @@ int build_class_chain(const BatchClass& bc, cudaStream_t s, cudaGraph_t target) 
   if (!rc) rc = cond(mbody, mtail, hh.mid_inner, false, &inode, &body);
   if (!rc) rc = iter_body(body, hh.mid_inner);
   if (!rc) rc = cond(target, {mid_node}, hh.outer, false, &outer_node, &obody);
-  if (!rc) rc = handle(obody, &hh.inner);
+  if (!rc) rc = handle(obody, &hh.again);
   if (!rc) rc = begin(obody, nullptr, 0);
+  if (rc) return rc;
+  hc::batch_decide(bi, sh, s);
+  hc::batch_flags(bi, sh, hc::BF_DECIDE, hh.again, hh.outer, cnt, 4, s);
+  std::vector<cudaGraphNode_t> otail;
+  cudaGraphNode_t again_node;
+  cudaGraph_t abody = nullptr;
+  rc = end(obody, &otail);
+  if (!rc) rc = cond(obody, otail, hh.again, true, &again_node, &abody);
+  if (!rc) rc = handle(abody, &hh.inner);
+  if (!rc) rc = begin(abody, nullptr, 0);
   if (rc) return rc;
   hc::batch_refine_resid(bi, sh, s);
   hc::batch_flags(bi, sh, hc::BF_REFINE, hh.inner, hh.outer, cnt, 4, s);
-  std::vector<cudaGraphNode_t> otail;
-  rc = end(obody, &otail);
-  if (!rc) rc = cond(obody, otail, hh.inner, false, &inode, &body);
+  rc = end(abody, &otail);
+  if (!rc) rc = cond(abody, otail, hh.inner, false, &inode, &body);
   if (!rc) rc = iter_body(body, hh.inner);
   if (!rc) rc = begin(target, &outer_node, 1);
   if (rc) return rc;
@@ -3580,7 +3649,7 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
     }
     if (c->refined) {
       auto& g = c->gf;
-      auto& gd = c->gd;
+      const hc::Geo<double> gd = decide_on(c) ? fx_geo(c->gd) : c->gd;  // the usual evaluation
       cx<float>*Gx = c->G32, *Gy = c->G32 + ns;
       cx<double>*Gx64 = c->G64, *Gy64 = c->G64 + ns;
       switch (kernel) {
@@ -3625,8 +3694,8 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
                               nullptr, (const cx<df64>*)c->b64, (cx<df64>*)c->r64, c->d32, c->q32,
                               ts, c->stream);
           else
-            hc::col_div<double>(gd, hc::CD_RESID_REFINE, Gx64, Gy64, nullptr, c->b64, c->r64,
-                                c->d32, c->q32, ts, c->stream);
+            hc::col_div<double>(gd, decide_on(c) ? hc::CD_DECIDE : hc::CD_RESID_REFINE, Gx64, Gy64,
+                                nullptr, c->b64, c->r64, c->d32, c->q32, ts, c->stream);
           break;
         case HC_K_SPLIT_GRAD:
           if (c->df)

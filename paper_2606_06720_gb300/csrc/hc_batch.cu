@@ -83,24 +83,44 @@ __global__ void __launch_bounds__(512) kb_mid_div(const BInst* bi) {
                                       c.st);
 }
 
-// ------------------------------------------------------------------ FP64 refinement residual
-// Only members whose refinement loop is still open (the last CTA of the
-// divergence pass decides, after every CTA has passed this test).
+// ------------------------------------------------------------------ refinement residual
+// The fx64 residual: members whose refinement loop is open and takes it next (the
+// last CTA of the divergence pass decides, after every CTA has passed this test).
+__global__ void __launch_bounds__(cta_bound<fx64>(512)) kb_dec_grad(const BInst* bi) {
+  const BInst& c = bi[blockIdx.y];
+  if (c.st->outer_done || !c.st->res_dec) return;
+  col_grad_body<fx64, fx64, CG_ADDDELTA>(c.gx, fxp(c.p64), nullptr, nullptr, c.x32, fxp(c.G64),
+                                         fxp(c.G64 + c.ns), c.st, 0);
+}
+__global__ void __launch_bounds__(cta_bound<fx64>(512)) kb_dec_apply(const BInst* bi) {
+  const BInst& c = bi[blockIdx.y];
+  if (c.st->outer_done || !c.st->res_dec) return;
+  row_apply_body<fx64, float, false, 1>(c.gx, fxp(c.G64), fxp(c.G64 + c.ns), c.mx, c.my, c.rf,
+                                        fxp(c.G64), fxp(c.G64 + c.ns), nullptr);
+}
+__global__ void __launch_bounds__(cta_bound<fx64>(512)) kb_dec_div(const BInst* bi) {
+  const BInst& c = bi[blockIdx.y];
+  if (c.st->outer_done || !c.st->res_dec) return;
+  col_div_body<fx64, CD_DECIDE>(c.gx, fxp(c.G64), fxp(c.G64 + c.ns), nullptr, fxp(c.b64), nullptr,
+                                nullptr, nullptr, c.st);
+}
+// The FP64 residual: members whose loop is open and takes it next, straight away or
+// because the fx64 one missed the tolerance.
 __global__ void __launch_bounds__(512) kb_res_grad(const BInst* bi) {
   const BInst& c = bi[blockIdx.y];
-  if (c.st->outer_done) return;
+  if (c.st->outer_done || !c.st->res_again) return;
   col_grad_body<double, double, CG_ADDDELTA>(c.gd, c.p64, nullptr, nullptr, c.x32, c.G64,
                                              c.G64 + c.ns, c.st, 0);
 }
 __global__ void __launch_bounds__(512) kb_res_apply(const BInst* bi) {
   const BInst& c = bi[blockIdx.y];
-  if (c.st->outer_done) return;
+  if (c.st->outer_done || !c.st->res_again) return;
   row_apply_body<double, float, false, 1>(c.gd, c.G64, c.G64 + c.ns, c.mx, c.my, c.rf, c.G64,
                                           c.G64 + c.ns, nullptr);
 }
 __global__ void __launch_bounds__(512) kb_res_div(const BInst* bi) {
   const BInst& c = bi[blockIdx.y];
-  if (c.st->outer_done) return;
+  if (c.st->outer_done || !c.st->res_again) return;
   col_div_body<double, CD_RESID_REFINE>(c.gd, c.G64, c.G64 + c.ns, nullptr, c.b64, c.r64, c.r32,
                                         c.x32, c.st);
 }
@@ -143,7 +163,8 @@ __global__ void kb_step_end(const BInst* bi, int nb, long long* launches) {
 // the first residual): h1 = some member runs a first inner solve, h2 = some
 // member has the mid-step residual pending.  BF_LOOP (after a CG iteration or
 // the mid-step residual): h1 = some member's inner solve is still running.
-// BF_REFINE (after an FP64 residual): h1 as BF_LOOP, h2 = some member's
+// BF_DECIDE (after an fx64 residual): h1 = some member needs the FP64 one, h2 as
+// BF_REFINE.  BF_REFINE (after an FP64 residual): h1 as BF_LOOP, h2 = some member's
 // refinement loop is still open.  `kernels` = launches of the segment this
 // kernel closes, itself included.
 __global__ void kb_flags(const BInst* bi, int nb, int kind, cudaGraphConditionalHandle h1,
@@ -151,9 +172,9 @@ __global__ void kb_flags(const BInst* bi, int nb, int kind, cudaGraphConditional
   bool a = false, b = false;
   for (int i = threadIdx.x; i < nb; i += 32) {
     const SolveState* st = bi[i].st;
-    a = a || !st->done;
+    a = a || (kind == BF_DECIDE ? !st->outer_done && st->res_again : !st->done);
     if (kind == BF_FIRST) b = b || st->mid_phase;
-    if (kind == BF_REFINE) b = b || !st->outer_done;
+    if (kind == BF_REFINE || kind == BF_DECIDE) b = b || !st->outer_done;
   }
   a = __any_sync(0xffffffffu, a);
   b = __any_sync(0xffffffffu, b);
@@ -208,6 +229,14 @@ void batch_mid_resid(const BInst* bi, const BShape& sh, cudaStream_t s) {
   kb_mid_div<<<col_grid(q, sh.nb), col_threads(q), col_smem(q, 2), s>>>(bi);
 }
 
+void batch_decide(const BInst* bi, const BShape& sh, cudaStream_t s) {
+  const Geo<double>& d = sh.gd;
+  kb_dec_grad<<<col_grid(d, sh.nb), col_threads(d), col_smem(d, 1), s>>>(bi);
+  const size_t sm = row_smem(d) + (size_t)3 * d.rpc * d.nx * sizeof(float);
+  kb_dec_apply<<<dim3(d.ny >> d.lrpc, sh.nb), row_threads(d), sm, s>>>(bi);
+  kb_dec_div<<<col_grid(d, sh.nb), col_threads(d), col_smem(d, 2), s>>>(bi);
+}
+
 void batch_refine_resid(const BInst* bi, const BShape& sh, cudaStream_t s) {
   const Geo<double>& d = sh.gd;
   kb_res_grad<<<col_grid(d, sh.nb), col_threads(d), col_smem(d, 2), s>>>(bi);
@@ -246,6 +275,9 @@ void set_smem_limits_batch() {
   allow_smem(kb_mid_grad);
   allow_smem(kb_mid_apply);
   allow_smem(kb_mid_div);
+  allow_smem(kb_dec_grad);
+  allow_smem(kb_dec_apply);
+  allow_smem(kb_dec_div);
   allow_smem(kb_res_grad);
   allow_smem(kb_res_apply);
   allow_smem(kb_res_div);

@@ -184,6 +184,8 @@ struct SolveState {
   unsigned long long h_cur;    // the inner-loop handle the CG kernels drive (set by whoever opens it)
   unsigned long long h_mid;        // cudaGraphConditionalHandle of the mid-step residual block (IF)
   unsigned long long h_mid_inner;  // cudaGraphConditionalHandle of the inner loop after it
+  unsigned long long h_dec;        // cudaGraphConditionalHandle of the fx64 residual (IF)
+  unsigned long long h_again;      // cudaGraphConditionalHandle of the FP64 residual and its sweep (IF)
   double first32_min2;       // refined: FP32 first sweep only if ||S - A p||^2 > this * ||S||^2 (0: off)
   int acc_first;             // FP32 first sweeps summed over the steps since the last reset
   int first_used;            // the running / last step ran an FP32 first sweep
@@ -194,6 +196,10 @@ struct SolveState {
   int acc_mid;               // such residuals summed over the steps since the last reset
   int res_full;              // running / last step: residuals in the mode's full refinement arithmetic
   int acc_res_full;          // summed likewise
+  int res_dec;               // the next refinement residual is evaluated by the fx64 kernels (predict_residual)
+  int res_again;             // ... by the FP64 ones: predicted, or the fx64 one missed the tolerance
+  int delta_added;           // the fx64 residual has added the pending correction to p64
+  int acc_again;             // fx64 residuals that missed, summed over the steps since the last reset
   unsigned int ticket[8];    // last-CTA tickets, one per reduction site
   // Diagnostics of Section 2.5, accumulated by the split step when diag != 0.
   // A step solves p[m^k] and so evaluates E_h(m^k) with its own pressure.
@@ -351,6 +357,7 @@ struct BInst {
   Geo<float> gf;
   Geo<float> gfn;         // gf limited to 512-thread column CTAs (col_narrow)
   Geo<double> gd;
+  Geo<fx64> gx;           // gd for the fx64 kernels
   Geo<df64> gq;
   SolveState* st;
   cx<double>* p64;        // pressure spectrum (FP64)
@@ -390,12 +397,13 @@ inline Geo<fx64> as_fx(const Geo<double>& g) {
   h.twx = reinterpret_cast<const cx<fx64>*>(g.qx);
   h.twy = reinterpret_cast<const cx<fx64>*>(g.qy);
   h.twz = reinterpret_cast<const cx<fx64>*>(g.qz);
+  h.pipe = 0;  // no persistent passes: two staged fields would cost half the warps
   return h;
 }
-inline cx<fx64>* fxp(cx<double>* p) { return reinterpret_cast<cx<fx64>*>(p); }
-inline const cx<fx64>* fxp(const cx<double>* p) { return reinterpret_cast<const cx<fx64>*>(p); }
-inline fx64* fxp(double* p) { return reinterpret_cast<fx64*>(p); }
-inline const fx64* fxp(const double* p) { return reinterpret_cast<const fx64*>(p); }
+__host__ __device__ inline cx<fx64>* fxp(cx<double>* p) { return reinterpret_cast<cx<fx64>*>(p); }
+__host__ __device__ inline const cx<fx64>* fxp(const cx<double>* p) { return reinterpret_cast<const cx<fx64>*>(p); }
+__host__ __device__ inline fx64* fxp(double* p) { return reinterpret_cast<fx64*>(p); }
+__host__ __device__ inline const fx64* fxp(const double* p) { return reinterpret_cast<const fx64*>(p); }
 template <typename P>
 inline auto fxp(const Tri<P>& t) {
   return Tri<decltype(fxp(t.v[0]))>{{fxp(t.v[0]), fxp(t.v[1]), fxp(t.v[2])}};
@@ -426,7 +434,7 @@ inline Geo<T> col_narrow(Geo<T> g) {
 // Column-kernel modes.
 enum ColGradMode { CG_PLAIN = 0, CG_DUPDATE = 1, CG_ADDDELTA = 2 };
 enum ColDivMode { CD_PLAIN = 0, CD_CG = 1, CD_RESID = 2, CD_RESID_REFINE = 3, CD_RESID_FIRST = 4,
-                  CD_CERT = 5 };
+                  CD_CERT = 5, CD_DECIDE = 6 };
 
 // ---------------- launchers (defined per precision) ----------------
 // Row pass, forward: physical pair (a, b) -> packed row spectra (A, B). b/B may be null.
@@ -610,10 +618,11 @@ void batch_step_begin(const BInst* bi, const BShape& sh, cudaGraphConditionalHan
 void batch_first_resid(const BInst* bi, const BShape& sh, cudaStream_t s);
 void batch_cg_iter(const BInst* bi, const BShape& sh, cudaStream_t s);
 void batch_mid_resid(const BInst* bi, const BShape& sh, cudaStream_t s);
+void batch_decide(const BInst* bi, const BShape& sh, cudaStream_t s);
 void batch_refine_resid(const BInst* bi, const BShape& sh, cudaStream_t s);
 void batch_split(const BInst* bi, const BShape& sh, cudaStream_t s);
 void batch_step_end(const BInst* bi, const BShape& sh, long long* launches, cudaStream_t s);
-enum { BF_FIRST = 0, BF_LOOP = 1, BF_REFINE = 2 };
+enum { BF_FIRST = 0, BF_LOOP = 1, BF_REFINE = 2, BF_DECIDE = 3 };
 void batch_flags(const BInst* bi, const BShape& sh, int kind, cudaGraphConditionalHandle h1,
                  cudaGraphConditionalHandle h2, long long* launches, int kernels, cudaStream_t s);
 void set_smem_limits_batch();

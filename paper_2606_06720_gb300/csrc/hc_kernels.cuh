@@ -861,6 +861,7 @@ __global__ void __launch_bounds__(cta_bound<T>(512)) k_row_c2r(Geo<T> g, const c
 // spectral derivative with the R1 multipliers is skew-adjoint), so alpha =
 // rho / <d, A d> is known here and the divergence pass needs neither d nor a
 // reduction.
+__device__ __forceinline__ void predict_residual(SolveState* st);
 __device__ __forceinline__ void cg_alpha_from(SolveState* st, double gkg, double n) {
   const double dq = gkg * n;
   if (dq > 0 && isfinite(dq)) {
@@ -878,6 +879,7 @@ __device__ __forceinline__ void cg_alpha_from(SolveState* st, double gkg, double
       st->status = HC_ENONFINITE;
     else if (!st->refined && st->rnorm2 > st->thresh2)
       st->status = HC_ENOCONV;
+    predict_residual(st);
   }
   st->first = 0;
 }
@@ -1186,6 +1188,53 @@ __global__ void __launch_bounds__(512) k_row_split(Geo<T> g, const cx<T>* Gx, co
 }
 
 // ------------------------------------------------------------------ solve-state finalizers
+// How the refinement loop will evaluate its next residual (one thread, at the end
+// of an inner solve or where one is skipped).  With the default residual switches
+// (mid_df) the loop usually ends at its first residual, after the FP32 first sweep
+// and the mid-step one, and then only the norm matters: the fx64 kernels give it
+// at a third of the cost.  r32, which the next FP32 solve starts from, comes from
+// the FP64 kernels always, so where the solve's own residual already says that
+// the tolerance is missed, they run straight away.
+__device__ __forceinline__ void predict_residual(SolveState* st) {
+  if (!st->refined) return;
+  const int dec = (st->mid_df && st->rnorm2 <= st->outer_thresh2) ? 1 : 0;
+  st->res_dec = dec;
+  st->res_again = 1 - dec;
+  if (st->graph_mode && st->h_again) {
+    cudaGraphSetConditional(st->h_dec, dec ? 1u : 0u);
+    cudaGraphSetConditional(st->h_again, dec ? 0u : 1u);
+  }
+}
+
+// The refinement loop's residual from the fx64 kernels (one thread), r2 =
+// ||S - A p64||^2 after p64 += delta: ends the loop when it meets the tolerance
+// (or nothing more may follow), else asks for the FP64 residual.
+__device__ __forceinline__ void resid_decide(SolveState* st, double r2) {
+  const bool finite = isfinite(r2);
+  const bool conv = r2 <= st->outer_thresh2;
+  st->outer_r2 = r2;
+  st->outer_done = (conv || !finite || st->sweeps >= st->max_sweeps) ? 1 : 0;
+  st->delta_added = 1;
+  st->res_dec = 0;
+  st->res_again = 1 - st->outer_done;
+  if (st->outer_done) {
+    st->res_full += 1;
+    st->acc_res_full += 1;
+    if (!finite) st->status = HC_ENONFINITE;
+    else st->status = conv ? 0 : HC_ENOCONV;
+    st->it = 0;
+    st->first = 1;
+    st->done = 1;
+  } else {
+    st->acc_again += 1;
+  }
+  st->h_cur = st->h_inner;
+  if (st->graph_mode && st->h_again) {
+    cudaGraphSetConditional(st->h_again, st->res_again ? 1u : 0u);
+    cudaGraphSetConditional(st->h_outer, st->outer_done ? 0u : 1u);
+  }
+}
+
 // Plain CG start (one thread): r2 = ||b - A x0||^2, rz = <r, M^-1 r>.
 __device__ __forceinline__ void resid_init(SolveState* st, double r2, double rz) {
   st->rnorm2 = r2;
@@ -1226,6 +1275,7 @@ __device__ __forceinline__ void resid_first_init(SolveState* st, double r32, dou
   // with lagged certification the double-float residual always follows, as the
   // right-hand side of the step's last inner solve
   st->mid_phase = ((use || st->pipelined) && st->mid_df) ? 1 : 0;
+  if (!use) predict_residual(st);
   st->h_cur = st->h_first;
   if (st->graph_mode) {
     cudaGraphSetConditional(st->h_first, use ? 1u : 0u);
@@ -1252,6 +1302,7 @@ __device__ __forceinline__ void resid_mid_init(SolveState* st, double r2, double
   st->first = 1;
   st->done = (!finite || r32 == 0.0 || r2 <= 0.01 * st->outer_thresh2) ? 1 : 0;
   if (!st->done) st->sweeps += 1;
+  else predict_residual(st);
   st->h_cur = st->h_mid_inner;
   if (st->graph_mode) cudaGraphSetConditional(st->h_mid_inner, st->done ? 0u : 1u);
 }
@@ -1261,6 +1312,7 @@ __device__ __forceinline__ void resid_mid_init(SolveState* st, double r2, double
 // (r32 is r64 rounded to FP32, so both norms are on the same scale.)
 __device__ __forceinline__ void resid_refine_init(SolveState* st, double r64, double r32,
                                                   double rz) {
+  st->delta_added = 0;
   st->res_full += 1;
   st->acc_res_full += 1;
   st->outer_r2 = r64;
@@ -1280,6 +1332,7 @@ __device__ __forceinline__ void resid_refine_init(SolveState* st, double r64, do
   st->first = 1;
   st->done = (st->outer_done || r32 == 0.0) ? 1 : 0;
   if (!st->outer_done) st->sweeps += 1;
+  predict_residual(st);  // for a solve that is skipped; its end predicts again
   st->h_cur = st->h_inner;
   if (st->graph_mode) {
     cudaGraphSetConditional(st->h_inner, st->done ? 0u : 1u);
@@ -1305,6 +1358,7 @@ __device__ __forceinline__ void cg_step_finish(SolveState* st, double rr, double
     st->done = 1;
     st->status = HC_ENOCONV;
   }
+  if (st->done) predict_residual(st);
   if (st->graph_mode) cudaGraphSetConditional(st->h_cur, st->done ? 0u : 1u);
 }
 
@@ -1368,7 +1422,11 @@ __device__ __forceinline__ void step_begin_body(SolveState* st, int npts) {
   st->outer_done = 0;
   st->first = 1;
   if (!st->refined) st->thresh2 = st->outer_thresh2;
+  st->delta_added = 0;
+  st->res_dec = 0;
+  st->res_again = 1;
   if (st->graph_mode && st->refined && st->h_outer) cudaGraphSetConditional(st->h_outer, 1u);
+  if (st->graph_mode && st->refined && st->h_again) cudaGraphSetConditional(st->h_again, 1u);
 }
 
 // Diagnostics of Section 2.5 for the step that just ran from m^k: the energy
@@ -1466,7 +1524,7 @@ __device__ __forceinline__ void col_grad_body(Geo<T> g, cx<Tin>* in, const cx<T>
     beta = st_beta<T>(st);
     pc = pc_of<T>(st);
   }
-  if (MODE == CG_ADDDELTA) add_delta = st->sweeps > 0;
+  if (MODE == CG_ADDDELTA) add_delta = st->sweeps > 0 && !st->delta_added;
   if constexpr (seq_fields<T>()) {
 #pragma unroll 1
     for (int q = 0; q < 2; ++q) {
@@ -1620,8 +1678,8 @@ __device__ __forceinline__ void col_div_body(Geo<T> g, const cx<T>* __restrict__
       const double r2 = (double)rv.x * (double)rv.x + (double)rv.y * (double)rv.y;
       acc[0] += w * r2;
       acc[1] += w * r2 * (double)pinv_sym(g, c.kx, ky, pc);
-    } else if constexpr (MODE == CD_CERT) {
-      // certification only: ||S - A p||^2 in the column's precision, nothing written
+    } else if constexpr (MODE == CD_CERT || MODE == CD_DECIDE) {
+      // the norm only: ||S - A p||^2 in the column's precision, nothing written
       const cx<T> rv = csub(bvec[idx], q);
       acc[0] += w * ((double)rv.x * (double)rv.x + (double)rv.y * (double)rv.y);
     } else if constexpr (MODE == CD_RESID_FIRST) {
@@ -1653,7 +1711,11 @@ __device__ __forceinline__ void col_div_body(Geo<T> g, const cx<T>* __restrict__
   }
   if constexpr (MODE == CD_PLAIN || MODE == CD_CG) return;
   double tot[3];
-  if constexpr (MODE == CD_CERT) {
+  if constexpr (MODE == CD_DECIDE) {
+    double a1[1] = {acc[0]}, t1[1];
+    if (last_cta_sum<1>(a1, g.partials, &st->ticket[TK_RESID], t1) && threadIdx.x == 0)
+      resid_decide(st, t1[0]);
+  } else if constexpr (MODE == CD_CERT) {
     double a1[1] = {acc[0]}, t1[1];
     if (last_cta_sum<1>(a1, g.partials, &st->ticket[TK_CERT], t1) && threadIdx.x == 0)
       st->cert_r2 = t1[0];
@@ -1901,7 +1963,7 @@ __global__ void __launch_bounds__(512) kp_col_grad(Geo<T> g, cx<T>* in, const cx
     beta = st_beta<T>(st);
     pc = pc_of<T>(st);
   }
-  if (MODE == CG_ADDDELTA) add_delta = st->sweeps > 0;
+  if (MODE == CG_ADDDELTA) add_delta = st->sweeps > 0 && !st->delta_added;
   const cx<T>* s0 = MODE == CG_DUPDATE ? rvec : in;
   const cx<T>* s1 = MODE == CG_DUPDATE ? dio : nullptr;
   // this thread's rows are the same in every tile: load their wavenumbers once
@@ -2577,6 +2639,9 @@ void row_apply(const Geo<T>& g, const cx<T>* Gx, const cx<T>* Gy, const Tm* mx, 
     if (g.fx)
       return row_apply<fx64, fx64>(as_fx(g), fxp(Gx), fxp(Gy), fxp(mx), fxp(my), fxp(r), fxp(Qx),
                                    fxp(Qy), st, s);
+  if constexpr (std::is_same<T, double>::value && std::is_same<Tm, float>::value)
+    if (g.fx)
+      return row_apply<fx64, float>(as_fx(g), fxp(Gx), fxp(Gy), mx, my, r, fxp(Qx), fxp(Qy), st, s);
   const size_t sm = row_smem(g) + (size_t)3 * g.rpc * g.nx * sizeof(Tm);
   if constexpr (std::is_same<T, float>::value && std::is_same<Tm, float>::value) {
     if (g.rpipe) {
@@ -2653,7 +2718,7 @@ void col_grad(const Geo<T>& g0, int mode, cx<Tin>* in, const cx<T>* rvec, cx<T>*
   const Geo<T> g = g0.pipe ? col_narrow(g0) : g0;
   const int nb = g.H >> g.ltc, nt = col_threads(g);
   const size_t sm = col_smem(g, seq_fields<T>() ? 1 : 2);
-  if constexpr (std::is_same<T, Tin>::value) {
+  if constexpr (std::is_same<T, Tin>::value && !seq_fields<T>()) {
     if (g.pipe) {
       const size_t ps = pipe_smem(g);
       if (mode == CG_PLAIN)
@@ -2688,28 +2753,30 @@ void col_div(const Geo<T>& g0, int mode, const cx<T>* Qx, const cx<T>* Qy, const
   const Geo<T> g = g0.pipe ? col_narrow(g0) : g0;
   const int nb = g.H >> g.ltc, nt = col_threads(g);
   const size_t sm = col_smem(g, 2);
-  if (g.pipe) {
-    const size_t ps = pipe_smem(g);
-    switch (mode) {
-      case CD_PLAIN:
-        kp_col_div<T, CD_PLAIN><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
-        break;
-      case CD_CG:
-        kp_col_div<T, CD_CG><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
-        break;
-      case CD_RESID:
-        kp_col_div<T, CD_RESID><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
-        break;
-      case CD_RESID_FIRST:
-        if constexpr (std::is_same<T, float>::value)
-          kp_col_div<T, CD_RESID_FIRST><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
-        break;
+  if constexpr (!seq_fields<T>()) {
+    if (g.pipe) {
+      const size_t ps = pipe_smem(g);
+      switch (mode) {
+        case CD_PLAIN:
+          kp_col_div<T, CD_PLAIN><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
+          break;
+        case CD_CG:
+          kp_col_div<T, CD_CG><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
+          break;
+        case CD_RESID:
+          kp_col_div<T, CD_RESID><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
+          break;
+        case CD_RESID_FIRST:
+          if constexpr (std::is_same<T, float>::value)
+            kp_col_div<T, CD_RESID_FIRST><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
+          break;
 
-      default:
-        kp_col_div<T, CD_RESID_REFINE><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
-        break;
+        default:
+          kp_col_div<T, CD_RESID_REFINE><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
+          break;
+      }
+      return;
     }
-    return;
   }
   switch (mode) {
     case CD_PLAIN:
@@ -2726,6 +2793,10 @@ void col_div(const Geo<T>& g0, int mode, const cx<T>* Qx, const cx<T>* Qy, const
         k_col_div<T, CD_RESID_FIRST><<<nb, nt, sm, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
       break;
 
+    case CD_DECIDE:
+      if constexpr (seq_fields<T>())
+        k_col_div<T, CD_DECIDE><<<nb, nt, sm, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
+      break;
     default:
       k_col_div<T, CD_RESID_REFINE><<<nb, nt, sm, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
       break;
@@ -2737,9 +2808,11 @@ void col_heat(const Geo<T>& g0, cx<T>* Mx, cx<T>* My, SolveState* st, cudaStream
     if (g0.fx) return col_heat<fx64>(as_fx(g0), fxp(Mx), fxp(My), st, s);
   // the whole tile (one slab); the persistent pass at most 512 threads
   const Geo<T> g = g0.pipe ? col_narrow(g0) : g0;
-  if (g.pipe) {
-    kp_col_heat<T><<<g.pgrid, col_threads(g), pipe_smem(g), s>>>(g, Mx, My, st);
-    return;
+  if constexpr (!seq_fields<T>()) {
+    if (g.pipe) {
+      kp_col_heat<T><<<g.pgrid, col_threads(g), pipe_smem(g), s>>>(g, Mx, My, st);
+      return;
+    }
   }
   k_col_heat<T><<<g.H >> g.ltc, col_threads(g), col_smem(g, 1), s>>>(g, Mx, My, st);
 }
@@ -2847,14 +2920,16 @@ void set_smem_limits_t() {
     allow_smem(k_col_div<T, CD_RESID_FIRST>);
     allow_smem(kp_col_div<T, CD_RESID_FIRST>);
   }
-  allow_smem(kp_col_div<T, CD_PLAIN>);
-  allow_smem(kp_col_div<T, CD_CG>);
-  allow_smem(kp_col_div<T, CD_RESID>);
-  allow_smem(kp_col_div<T, CD_RESID_REFINE>);
-  allow_smem(kp_col_heat<T>);
-  allow_smem(kp_col_grad<T, CG_PLAIN>);
-  allow_smem(kp_col_grad<T, CG_DUPDATE>);
-  allow_smem(kp_col_grad<T, CG_ADDDELTA>);
+  if constexpr (!seq_fields<T>()) {
+    allow_smem(kp_col_div<T, CD_PLAIN>);
+    allow_smem(kp_col_div<T, CD_CG>);
+    allow_smem(kp_col_div<T, CD_RESID>);
+    allow_smem(kp_col_div<T, CD_RESID_REFINE>);
+    allow_smem(kp_col_heat<T>);
+    allow_smem(kp_col_grad<T, CG_PLAIN>);
+    allow_smem(kp_col_grad<T, CG_DUPDATE>);
+    allow_smem(kp_col_grad<T, CG_ADDDELTA>);
+  }
   allow_smem(k_row_adj_point<T>);
   allow_smem(k_row_adj_press<T>);
   allow_smem(k_col_lap_dot<T>);
@@ -2873,6 +2948,9 @@ extern template void row_c2r<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<f
                               fx64*, SolveState*, int, cudaStream_t);
 extern template void row_apply<fx64, fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*,
                                         const fx64*, const fx64*, const fx64*, cx<fx64>*,
+                                        cx<fx64>*, SolveState*, cudaStream_t);
+extern template void row_apply<fx64, float>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*,
+                                        const float*, const float*, const float*, cx<fx64>*,
                                         cx<fx64>*, SolveState*, cudaStream_t);
 extern template void row_split<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, const fx64*,
                                const fx64*, const fx64*, cx<fx64>*, cx<fx64>*, SplitCoef, SolveState*,

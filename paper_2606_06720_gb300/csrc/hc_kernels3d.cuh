@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(cta_bound<T>(256)) k3_zgrad(Geo<T> g, cx<Tin>*
     beta = st_beta<T>(st);
     pc = pc_of<T>(st);
   }
-  if (MODE == CG_ADDDELTA) add_delta = st->sweeps > 0;
+  if (MODE == CG_ADDDELTA) add_delta = st->sweeps > 0 && !st->delta_added;
   if constexpr (seq_fields<T>()) {
 #pragma unroll 1
     for (int q = 0; q < 3; ++q) {
@@ -390,6 +390,9 @@ __global__ void __launch_bounds__(cta_bound<T>(256)) k3_zdiv(Geo<T> g, Tri<cx<T>
       const double r2 = (double)rv.x * (double)rv.x + (double)rv.y * (double)rv.y;
       acc[0] += w * r2;
       acc[1] += w * r2 * (double)pinv3(g, kx, ky, kz, pc);
+    } else if constexpr (MODE == CD_DECIDE) {
+      const cx<T> rv = csub(bvec[idx], q);  // the norm only
+      acc[0] += w * ((double)rv.x * (double)rv.x + (double)rv.y * (double)rv.y);
     } else if constexpr (MODE == CD_RESID_FIRST) {
       const cx<float> rf = ccast<float>(csub(bvec[idx], q));
       r32[idx] = rf;
@@ -417,7 +420,11 @@ __global__ void __launch_bounds__(cta_bound<T>(256)) k3_zdiv(Geo<T> g, Tri<cx<T>
   }
   if constexpr (MODE == CD_PLAIN || MODE == CD_CG) return;
   double tot[3];
-  if constexpr (MODE == CD_RESID) {
+  if constexpr (MODE == CD_DECIDE) {
+    double a1[1] = {acc[0]}, t1[1];
+    if (last_cta_sum<1>(a1, g.partials, &st->ticket[TK_RESID], t1) && threadIdx.x == 0)
+      resid_decide(st, t1[0]);
+  } else if constexpr (MODE == CD_RESID) {
     double a2[2] = {acc[0], acc[1]}, t2[2];
     if (last_cta_sum<2>(a2, g.partials, &st->ticket[TK_RESID], t2) && threadIdx.x == 0)
       resid_init(st, t2[0], t2[1]);
@@ -792,6 +799,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k3_cg_update(Geo<
       st->done = 1;
       st->status = HC_ENOCONV;
     }
+    if (st->done) predict_residual(st);
     if (st->graph_mode) cudaGraphSetConditional(st->h_cur, st->done ? 0u : 1u);
   }
 }
@@ -896,6 +904,10 @@ void z_div(const Geo<T>& g, int mode, Tri<cx<T>*> Q, const cx<T>* d, const cx<T>
       if constexpr (std::is_same<T, float>::value)
         k3_zdiv<T, CD_RESID_FIRST><<<nb, nt, sm, s>>>(g, Q, d, b, out, r32, delta32, st);
       break;
+    case CD_DECIDE:
+      if constexpr (seq_fields<T>())
+        k3_zdiv<T, CD_DECIDE><<<nb, nt, sm, s>>>(g, Q, d, b, out, r32, delta32, st);
+      break;
     default:
       k3_zdiv<T, CD_RESID_REFINE><<<nb, nt, sm, s>>>(g, Q, d, b, out, r32, delta32, st);
       break;
@@ -904,6 +916,8 @@ void z_div(const Geo<T>& g, int mode, Tri<cx<T>*> Q, const cx<T>* d, const cx<T>
 template <typename T, typename Tm>
 void row_apply3(const Geo<T>& g, Tri<cx<T>*> G, Tri<const Tm*> m, const Tm* r, Tri<cx<T>*> Q,
                 SolveState* st, cudaStream_t s) {
+  if constexpr (std::is_same<T, double>::value && std::is_same<Tm, float>::value)
+    if (g.fx) return row_apply3<fx64, float>(as_fx(g), fxp(G), m, r, fxp(Q), st, s);
   if constexpr (std::is_same<T, double>::value && std::is_same<Tm, double>::value)
     if (g.fx)
       return row_apply3<fx64, fx64>(as_fx(g), fxp(G), fxp(m), fxp(r), fxp(Q), st, s);

@@ -35,7 +35,12 @@ void set_smem_limits_3d_fx(int refined) {
   }
   allow_smem(k3_axis_fft<fx64, -1, 1>);
   allow_smem(k3_axis_fft<fx64, +1, 1>);
+  allow_smem(k3_axis_fft<fx64, -1, 3>);
+  allow_smem(k3_axis_fft<fx64, +1, 3>);
   allow_smem(k3_zfwd_project<fx64>);
+  allow_smem(k3_zdiv<fx64, CD_DECIDE>);
+  allow_smem(k3_row_apply<fx64, float, false>);
+  set_smem_limits_zgrad<fx64, fx64>();
 }
 
 }  // namespace hc

@@ -96,6 +96,7 @@ __global__ void k_reset_accum(SolveState* st) {
   st->acc_first = 0;
   st->acc_mid = 0;
   st->acc_res_full = 0;
+  st->acc_again = 0;
   st->first_bad = 0;
   st->acc_iters = 0;
   st->acc_sweeps = 0;

@@ -12,6 +12,9 @@ template void row_c2r<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, 
 template void row_apply<fx64, fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*,
                                         const fx64*, const fx64*, const fx64*, cx<fx64>*,
                                         cx<fx64>*, SolveState*, cudaStream_t);
+template void row_apply<fx64, float>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*,
+                                        const float*, const float*, const float*, cx<fx64>*,
+                                        cx<fx64>*, SolveState*, cudaStream_t);
 template void row_split<fx64>(const Geo<fx64>&, const cx<fx64>*, const cx<fx64>*, const fx64*,
                                const fx64*, const fx64*, cx<fx64>*, cx<fx64>*, SplitCoef, SolveState*,
                                cudaStream_t);
@@ -55,7 +58,7 @@ void cert_resid(const Geo<double>& gd, const cx<double>* p, const float* mx, con
                                                           nullptr, sc);
 }
 
-// A refined context launches only the certification and p's transforms.
+// A refined context launches only the residuals and p's transforms.
 void set_smem_limits_fx(int refined) {
   if (!refined) {
     set_smem_limits_t<fx64>();
@@ -66,9 +69,10 @@ void set_smem_limits_fx(int refined) {
   allow_smem(k_col_fwd<fx64, 1>);
   allow_smem(k_col_inv<fx64>);
   allow_smem(k_row_c2r<fx64>);
-  allow_smem(k_col_grad<fx64, fx64, CG_PLAIN>);
+  set_smem_limits_grad<fx64, fx64>();
   allow_smem(k_row_apply<fx64, float, false, 1>);
   allow_smem(k_col_div<fx64, CD_CERT>);
+  allow_smem(k_col_div<fx64, CD_DECIDE>);
 }
 
 }  // namespace hc

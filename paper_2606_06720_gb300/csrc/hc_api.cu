@@ -438,17 +438,28 @@ void fill_geo(hc_ctx* c, hc::Geo<T>& g, const cx<T>* twx, const cx<T>* twy, cons
   // column CTA: tc packed columns x ny/8 threads: 1024 threads (FP32), 256
   // (FP64, double-float: at 128 registers two CTAs per SM, the same warps as
   // one of 512 in finer pieces; measured at 2048^2, the FP64 gradient and
-  // divergence passes take 674 us per step at 256 threads, 801 at 512)
+  // divergence passes take 674 us per step at 256 threads, 801 at 512), then
+  // narrower, to one warp, while fewer than 128 CTAs would run on the 152 SMs.  Measured (us
+  // per launch, wide tile / this rule): FP32 gradient and divergence 512^2 18.5 +
+  // 16.5 / 8.3 + 8.3, 1024^2 16.5 + 16.4 / 12.3 + 12.2; fx64 512^2 34.9 + 24.7 /
+  // 26.7 + 18.5, 64^2 30.8 + 20.6 / 20.6 + 14.4.  Narrower still loses: the rows
+  // of a narrow tile are partial sectors (1024^2 at 512 CTAs 17.1 + 12.3).
   int tc = (sizeof(T) == 4 ? hc::col_cta_max<T, true>() : 256) >> (g.lny - 3);
   if (tc < 1) tc = 1;
   if (tc > 32) tc = 32;
   if (tc > c->H) tc = c->H;
+  while (tc > 1 && c->H / tc < 128 && (tc >> 1) << (g.lny - 3) >= 32) tc >>= 1;
   g.tc = tc;
   g.ltc = ilog2(tc);
-  // row CTA: rpc rows x nx/8 threads, about 256 threads
-  int rpc = 256 >> (g.lnx - 3);
+  // row CTA: rpc rows x nx/8 threads, about 256 threads (FP32) or 128 (FP64,
+  // double-float: 1024^2 split row pass 127 us at 256 threads, 109 at 128), then
+  // fewer rows while the grid is small.  FP32 keeps two where it had more: its
+  // operator pass puts two rows on each thread (NV = 2) and sums them together.
+  int rpc = (sizeof(T) == 4 ? 256 : 128) >> (g.lnx - 3);
   if (rpc < 1) rpc = 1;
   if (rpc > c->ny) rpc = c->ny;
+  const int nv = sizeof(T) == 4 ? 2 : 1;  // rows per thread
+  while (rpc > nv && c->ny / rpc < 512 / nv && (rpc / 2 / nv) << (g.lnx - 3) >= 32) rpc >>= 1;
   g.rpc = rpc;
   g.lrpc = ilog2(rpc);
   g.twx = twx;

@@ -422,17 +422,18 @@ void hc_batch_destroy(hc_batch* batch);
  *   nx, ny: powers of two in [8, 4096] with nx*ny <= HC_NOALLOC_MAX_POINTS;
  *           anything else (or a null pointer) returns HC_EINVAL.
  *   stream: cudaStream_t (NULL: legacy default stream); the call only enqueues
- *           work on it and returns.  CUDA failures of its own launches return
+ *           work on it and returns (the first call on a device waits, see below).  CUDA failures of its own launches return
  *           HC_ECUDA; a non-sticky error left pending on the calling thread by
  *           earlier work is cleared on entry (cudaGetLastError), not reported.
  * Scratch lives in one fixed 640 KiB static device array of the library
  * (present on every GPU the process uses, until the process exits); the call
  * allocates nothing and calls no allocating routine.  All calls share that
- * array; each call rewrites it completely before reading it, so nothing from
- * an earlier call is reused, but calls whose GPU work overlaps (other streams
- * or threads at the same time) race on it and must be serialised by the
- * caller.  The first call on each device does a one-time set-up (it looks up
- * the array's device address and raises the kernels' shared-memory limit):
+ * array: its twiddle tables are constants, and of the rest each call rewrites
+ * what it reads, so no result of an earlier call is reused, but calls whose GPU
+ * work overlaps (other streams or threads at the same time) race on it and must
+ * be serialised by the caller.  The first call on each device does a one-time
+ * set-up (it looks up the array's device address, raises the kernels'
+ * shared-memory limit, fills the tables and waits for that on its stream):
  * make that first call before any stream capture. */
 int hc_spectrum_noalloc(const double* f, double* out, int nx, int ny, void* stream);
 

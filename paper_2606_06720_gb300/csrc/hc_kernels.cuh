@@ -770,6 +770,7 @@ template <typename T>
 __global__ void __launch_bounds__(cta_bound<T>(512)) k_row_r2c(Geo<T> g, const T* __restrict__ a,
                                                  const T* __restrict__ b, cx<T>* __restrict__ A,
                                                  cx<T>* __restrict__ B) {
+  if constexpr (seq_fields<T>()) cudaTriggerProgrammaticLaunchCompletion();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
   const int l8 = g.lnx - 3, N = g.nx, H = g.H, N8 = 1 << l8;
@@ -1848,9 +1849,12 @@ __global__ void __launch_bounds__(cta_bound<T>(col_cta_max<T, true>()), 1) k_col
 }
 
 template <typename T, int NV>
-__global__ void __launch_bounds__(512) k_col_fwd(Geo<T> g, const cx<T>* __restrict__ in0,
+__global__ void __launch_bounds__(cta_bound<T>(512)) k_col_fwd(Geo<T> g, const cx<T>* __restrict__ in0,
                                                  const cx<T>* __restrict__ in1, cx<T>* out0,
                                                  cx<T>* out1, int project, SolveState* st) {
+  // a launch that may overlap the kernel before it (hc_noalloc.cu) waits for its
+  // results here; otherwise this returns at once
+  if constexpr (seq_fields<T>()) cudaGridDependencySynchronize();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
   const ColIdx c = col_idx(g);

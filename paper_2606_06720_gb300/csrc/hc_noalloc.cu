@@ -27,25 +27,28 @@ using hc::FxTw;
 
 constexpr int kMaxDevices = 64;
 constexpr size_t kInterBytes = (size_t)HC_NOALLOC_MAX_POINTS / 2 * sizeof(cx<double>);
-constexpr size_t kTwBytes = 4096 * sizeof(cx<double>);
+constexpr int kTables = 2 * 4096;  // the table of length N starts at entry N
 
 // Row-transformed intermediate (ny * nx/2 complex doubles at most) followed by
-// the twiddle tables of the x and y lengths (4096 entries each at most).
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kInterBytes + 2 * kTwBytes];
+// the twiddle tables of every length (8 .. 4096).
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kInterBytes + kTables * sizeof(FxTw)];
 
 std::mutex g_mu;
-void* g_addr[kMaxDevices];  // device address of g_noalloc_scratch per device (set-up done)
+void* g_addr[kMaxDevices];    // device address of g_noalloc_scratch per device
+bool g_tables[kMaxDevices];   // its tables are filled
 
-// tw[m] = exp(-2 pi i m / N), m < N: Q62, or FP64 below the fixed-point lengths.
-__global__ void k_noalloc_twiddles(FxTw* tw, int N) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= N) return;
+// Table entry N + m = exp(-2 pi i m / N), m < N: Q62, or FP64 below the
+// fixed-point lengths.
+__global__ void k_noalloc_tables(FxTw* tab) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < 8 || i >= kTables) return;
+  const int N = 1 << (31 - __clz(i)), m = i - N;
   double s, c;
   sincospi(2.0 * (double)m / (double)N, &s, &c);
   if (N >= (1 << hc::kFxMinLog))
-    tw[m] = hc::fx_twiddle(__double2ll_rn(c * 0x1p62), __double2ll_rn(s * -0x1p62));
+    tab[i] = hc::fx_twiddle(__double2ll_rn(c * 0x1p62), __double2ll_rn(s * -0x1p62));
   else
-    reinterpret_cast<double2*>(tw)[m] = make_double2(c, -s);
+    reinterpret_cast<double2*>(tab)[i] = make_double2(c, -s);
 }
 
 int ilog2i(int v) {
@@ -57,9 +60,11 @@ int ilog2i(int v) {
 bool pow2_in(int v, int lo, int hi) { return v >= lo && v <= hi && (v & (v - 1)) == 0; }
 
 // One-time set-up per device: the device address of the static scratch (the
-// host-side symbol is only a stand-in) and the shared-memory opt-in of the
-// two kernels launched here.
-int setup_device(int dev, void** addr) {
+// host-side symbol is only a stand-in), the shared-memory opt-in of the two
+// kernels launched here, and the twiddle tables.  The tables are constants: they
+// are complete before the first call returns.  While s is being captured they
+// become part of the captured work instead, and a later call fills them for good.
+int setup_device(int dev, cudaStream_t s, void** addr) {
   std::lock_guard<std::mutex> lock(g_mu);
   if (dev < 0 || dev >= kMaxDevices) return HC_EINVAL;
   if (!g_addr[dev]) {
@@ -72,6 +77,18 @@ int setup_device(int dev, void** addr) {
     g_addr[dev] = p;
   }
   *addr = g_addr[dev];
+  if (!g_tables[dev]) {
+    cudaGetLastError();
+    k_noalloc_tables<<<kTables / 256, 256, 0, s>>>(
+        reinterpret_cast<FxTw*>(static_cast<unsigned char*>(*addr) + kInterBytes));
+    if (cudaGetLastError() != cudaSuccess) return HC_ECUDA;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) return HC_ECUDA;
+    if (cs == cudaStreamCaptureStatusNone) {
+      if (cudaStreamSynchronize(s) != cudaSuccess) return HC_ECUDA;
+      g_tables[dev] = true;
+    }
+  }
   return HC_OK;
 }
 
@@ -84,17 +101,16 @@ extern "C" int hc_spectrum_noalloc(const double* f, double* out, int nx, int ny,
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return HC_ECUDA;
   void* base = nullptr;
-  int rc = setup_device(dev, &base);
-  if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
+  int rc = setup_device(dev, s, &base);
+  if (rc) return rc;
   // A non-sticky error left pending on this thread by earlier work (the
   // caller's or another library's) is consumed here, so that the check after
   // the launches reports only this call's own launches.
   cudaGetLastError();
   unsigned char* b = static_cast<unsigned char*>(base);
   cx<fx64>* inter = reinterpret_cast<cx<fx64>*>(b);
-  FxTw* twx = reinterpret_cast<FxTw*>(b + kInterBytes);
-  FxTw* twy = reinterpret_cast<FxTw*>(b + kInterBytes + kTwBytes);
+  const FxTw* tab = reinterpret_cast<const FxTw*>(b + kInterBytes);
 
   hc::Geo<fx64> g = {};
   g.nx = nx;
@@ -103,28 +119,44 @@ extern "C" int hc_spectrum_noalloc(const double* f, double* out, int nx, int ny,
   g.lnx = ilog2i(nx);
   g.lny = ilog2i(ny);
   g.lH = ilog2i(nx / 2);
-  int tc = 512 >> (g.lny - 3);
+  // 256-thread column CTAs and 128-thread row CTAs, narrower (to one warp) until
+  // there are enough of them for the chip, as a context's default shapes
+  int tc = 256 >> (g.lny - 3);
   tc = tc < 1 ? 1 : (tc > 32 ? 32 : tc);
   if (tc > g.H) tc = g.H;
+  while (tc > 1 && g.H / tc < 128 && (tc >> 1) << (g.lny - 3) >= 32) tc >>= 1;
   g.tc = tc;
   g.ltc = ilog2i(tc);
-  int rpc = 256 >> (g.lnx - 3);
+  int rpc = 128 >> (g.lnx - 3);
   rpc = rpc < 1 ? 1 : rpc;
   if (rpc > ny) rpc = ny;
+  while (rpc > 1 && ny / rpc < 512 && (rpc >> 1) << (g.lnx - 3) >= 32) rpc >>= 1;
   g.rpc = rpc;
   g.lrpc = ilog2i(rpc);
-  g.twx = reinterpret_cast<const cx<fx64>*>(twx);
-  g.twy = reinterpret_cast<const cx<fx64>*>(twy);
+  g.twx = reinterpret_cast<const cx<fx64>*>(tab + nx);
+  g.twy = reinterpret_cast<const cx<fx64>*>(tab + ny);
 
-  // Every call rewrites the tables and the whole intermediate before reading
-  // them, so nothing carried over from an earlier call is used.
-  k_noalloc_twiddles<<<(nx + 255) / 256, 256, 0, s>>>(twx, nx);
-  k_noalloc_twiddles<<<(ny + 255) / 256, 256, 0, s>>>(twy, ny);
+  // Every call rewrites the part of the intermediate that it reads, so nothing
+  // carried over from an earlier call is used.  The column pass may start while
+  // the row pass drains (it waits before its first read): with the tables kept
+  // and the narrower CTAs a 256^2 call takes 25 us where four launches in 8 and
+  // 32 CTAs took 39 (67 with FP64 passes).  What is left is the latency of one
+  // warp's instructions: each thread carries 8 points through three passes.
   hc::k_row_r2c<fx64><<<ny >> g.lrpc, rpc << (g.lnx - 3), (size_t)rpc * nx * sizeof(cx<double>), s>>>(
       g, hc::fxp(f), nullptr, inter, nullptr);
-  hc::k_col_fwd<fx64, 1><<<g.H >> g.ltc, tc << (g.lny - 3),
-                             (size_t)(ny + (ny >> 3)) * tc * sizeof(cx<double>), s>>>(
-      g, inter, nullptr, reinterpret_cast<cx<fx64>*>(out), nullptr, 0, nullptr);
+  cudaLaunchAttribute early = {};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g.H >> g.ltc);
+  cfg.blockDim = dim3(tc << (g.lny - 3));
+  cfg.dynamicSmemBytes = (size_t)(ny + (ny >> 3)) * tc * sizeof(cx<double>);
+  cfg.stream = s;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, hc::k_col_fwd<fx64, 1>, g, (const cx<fx64>*)inter, (const cx<fx64>*)nullptr,
+                     reinterpret_cast<cx<fx64>*>(out), (cx<fx64>*)nullptr, 0,
+                     (hc::SolveState*)nullptr);
   if (cudaGetLastError() != cudaSuccess) return HC_ECUDA;
   return HC_OK;
 }

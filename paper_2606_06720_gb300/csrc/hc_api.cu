@@ -144,7 +144,9 @@ struct hc_ctx {
   cx<double>* b64;          // source spectrum (projected)
   cx<double>* r64;          // residual (FP64)
   cx<double>* d64;          // CG direction (plain mode)
-  cx<double>* q64;          // A d (plain mode)
+  cx<double>* q64;          // A d (plain mode, 3D and component calls)
+  double* pinv64;           // plain mode, 2D: the running step's preconditioner symbol
+  double* dots;             // plain mode, 2D: the row pass's per-CTA sums of <d, A d>
   cx<double>* G64;          // dim spectra: gradient / flux / m scratch (FP64)
   cx<float>* b32;           // refined: FP32 copy of the projected source spectrum
   cx<df64>* bq;             // HC_FP32_REFINED: double-float copy of it (mid-step residual)
@@ -247,33 +249,41 @@ void twiddles(int N, std::vector<double>& re, std::vector<double>& im) {
   }
 }
 
-// Twiddle table of the fx64 kernels.  Fixed-point lengths: exp(-2 pi i m / N) in
-// Q62, the first octant from the long double functions, the others by symmetry;
-// shorter lengths: the FP64 values.
-std::vector<hc::FxTw> twiddles_fx(int N) {
-  std::vector<hc::FxTw> out(N);
-  if (N < (1 << hc::kFxMinLog)) {
-    std::vector<double> re, im;
-    twiddles(N, re, im);
-    for (int m = 0; m < N; ++m) {
-      const double v[2] = {re[m], im[m]};
-      std::memcpy(&out[m], v, sizeof(v));
-    }
-    return out;
-  }
-  // (long double is slow in software on some hosts: N/8 + 1 evaluations only)
-  const int E = N / 8, Q = N / 4;
+// exp(-2 pi i m / N), m < N, in Q62: the first octant (of N a multiple of 8; else
+// the first half turn) from the long double functions, the rest by symmetry.
+// (long double is slow in software on some hosts.)
+std::vector<hc::FxTw> twiddles_q62(int N) {
+  const long double two_pi = 6.28318530717958647692528676655900577L;
+  const int E = N % 8 == 0 ? N / 8 : N / 2;
   std::vector<long long> co(E + 1), si(E + 1);
   for (int r = 0; r <= E; ++r) {
-    const long double phi = 1.57079632679489661923132169163975144L * (long double)r / Q;
+    const long double phi = two_pi * (long double)r / N;
     co[r] = std::llroundl(std::ldexp(std::cos(phi), 62));
     si[r] = std::llroundl(std::ldexp(std::sin(phi), 62));
   }
+  std::vector<hc::FxTw> out(N);
   for (int m = 0; m < N; ++m) {
-    const int q = m / Q, r = m - q * Q;  // angle = (pi/2) (q + r/Q)
-    const long long c = r <= E ? co[r] : si[Q - r], s = r <= E ? si[r] : co[Q - r];
-    const long long re[4] = {c, -s, -c, s}, im[4] = {s, c, -s, -c};
-    out[m] = hc::fx_twiddle(re[q], -im[q]);
+    if (N % 8 == 0) {
+      const int Q = N / 4, q = m / Q, r = m - q * Q;  // angle = (pi/2) (q + r/Q)
+      const long long c = r <= E ? co[r] : si[Q - r], s = r <= E ? si[r] : co[Q - r];
+      const long long re[4] = {c, -s, -c, s}, im[4] = {s, c, -s, -c};
+      out[m] = hc::fx_twiddle(re[q], -im[q]);
+    } else {
+      out[m] = 2 * m <= N ? hc::fx_twiddle(co[m], -si[m]) : hc::fx_twiddle(co[N - m], si[N - m]);
+    }
+  }
+  return out;
+}
+// Twiddle table of the fx64 kernels: Q62, or the FP64 values of a length that
+// they transform in FP64.
+std::vector<hc::FxTw> twiddles_fx(int N) {
+  if (N >= (1 << hc::kFxMinLog)) return twiddles_q62(N);
+  std::vector<hc::FxTw> out(N);
+  std::vector<double> re, im;
+  twiddles(N, re, im);
+  for (int m = 0; m < N; ++m) {
+    const double v[2] = {re[m], im[m]};
+    std::memcpy(&out[m], v, sizeof(v));
   }
   return out;
 }
@@ -308,10 +318,12 @@ void layout_generic(hc_ctx* c, Layout& L) {
   c->d64 = L.take<cx<double>>(S64);
   c->q64 = L.take<cx<double>>(S64);
   c->G64 = L.take<cx<double>>(2 * S64);
+  c->pinv64 = L.take<double>(sizeof(double) * c->ns);
+  c->dots = L.take<double>(sizeof(double) * c->ny);
   for (int k = 0; k < 2; ++k) c->m[k] = L.take<double>(sizeof(double) * n);
   c->rf = L.take<double>(sizeof(double) * n);
-  c->twx_d = L.take<cx<double>>(sizeof(cx<double>) * c->nx);
-  c->twy_d = L.take<cx<double>>(sizeof(cx<double>) * c->ny);
+  c->twx_x = L.take<hc::FxTw>(sizeof(hc::FxTw) * c->nx);
+  c->twy_x = L.take<hc::FxTw>(sizeof(hc::FxTw) * c->ny);
   c->kxd_d = L.take<double>(sizeof(double) * c->H);
   c->kyd_d = L.take<double>(sizeof(double) * c->ny);
   c->hx_d = L.take<double>(sizeof(double) * c->H);
@@ -338,6 +350,10 @@ void layout(hc_ctx* c, Layout& L) {
   if (!c->refined) {
     c->d64 = L.take<cx<double>>(S64);
     c->q64 = L.take<cx<double>>(S64);
+    if (d == 2) {
+      c->pinv64 = L.take<double>(sizeof(double) * c->ns);
+      c->dots = L.take<double>(sizeof(double) * c->ny);
+    }
     c->b32 = c->r32 = c->d32 = c->q32 = c->x32 = c->G32 = nullptr;
     c->bq = nullptr;
     for (int k = 0; k < d; ++k) c->m[k] = L.take<double>(sizeof(double) * n);
@@ -605,20 +621,9 @@ int scan_zones(cudaStream_t s, const char* base, const Zones& z, int* bad) {
 // multipliers (Nyquist entry 0, reading R1) of the Hh = nx/2 + 1 columns and
 // the ny rows.
 int upload_tables_generic(hc_ctx* c) {
-  std::vector<double> re, im;
-  auto put_tw = [&](int N, cx<double>* dd) -> int {
-    twiddles(N, re, im);
-    std::vector<cx<double>> hd(N);
-    for (int m = 0; m < N; ++m) {
-      hd[m].x = re[m];
-      hd[m].y = im[m];
-    }
-    CU(cudaMemcpy(dd, hd.data(), sizeof(cx<double>) * N, cudaMemcpyHostToDevice));
-    return HC_OK;
-  };
-  int rc = put_tw(c->nx, c->twx_d);
-  if (!rc) rc = put_tw(c->ny, c->twy_d);
-  if (rc) return rc;
+  const std::vector<hc::FxTw> qx = twiddles_q62(c->nx), qy = twiddles_q62(c->ny);
+  CU(cudaMemcpy(c->twx_x, qx.data(), sizeof(hc::FxTw) * c->nx, cudaMemcpyHostToDevice));
+  CU(cudaMemcpy(c->twy_x, qy.data(), sizeof(hc::FxTw) * c->ny, cudaMemcpyHostToDevice));
   std::vector<double> kx(c->H), ky(c->ny);
   for (int k = 0; k < c->H; ++k) kx[k] = xid(k, c->nx, c->grid.L[0]);
   for (int k = 0; k < c->ny; ++k) ky[k] = xid(k, c->ny, c->grid.L[1]);
@@ -635,13 +640,15 @@ void fill_generic_geo(hc_ctx* c) {
   g.Hh = c->H;
   g.nrx = radices(c->nx, g.rx);
   g.nry = radices(c->ny, g.ry);
-  g.twx = c->twx_d;
-  g.twy = c->twy_d;
+  g.qx = c->twx_x;
+  g.qy = c->twy_x;
   g.kxd = c->kxd_d;
   g.kyd = c->kyd_d;
   g.hx = c->hx_d;
   g.hy = c->hy_d;
   g.partials = c->partials;
+  g.dots = c->dots;
+  g.pinv = c->pinv64;
   // the grid-wide sums (hc::msum) take only nx, ny and the partials
   c->gd = hc::Geo<double>{};
   c->gd.nx = c->nx;
@@ -876,7 +883,8 @@ void plain_init(hc_ctx* c) {
     hc::gen_row_apply(c->gg, Gx, Gy, (const double*)c->m[0], (const double*)c->m[1],
                       (const double*)c->rf, Gx, Gy, nullptr, c->stream);
     hc::gen_col_div(c->gg, hc::CD_RESID, Gx, Gy, c->b64, c->r64, c->st, c->stream);
-    c->launches += 3;
+    hc::gen_pinv_table(c->gg, c->st, c->stream);
+    c->launches += 4;
     return;
   }
   if (c->dim == 3) {
@@ -895,7 +903,8 @@ void plain_init(hc_ctx* c) {
                                 (const double*)c->rf, Gx, Gy, nullptr, c->stream);
   hc::col_div<double>(g, hc::CD_RESID, Gx, Gy, nullptr, c->b64, c->r64, nullptr, nullptr, c->st,
                       c->stream);
-  c->launches += 3;
+  hc::pinv_table(g, c->st, c->stream);
+  c->launches += 4;
 }
 
 void plain_iter(hc_ctx* c) {
@@ -905,9 +914,8 @@ void plain_iter(hc_ctx* c) {
     hc::gen_col_grad(c->gg, hc::CG_DUPDATE, nullptr, c->r64, c->d64, Gx, Gy, c->st, 1, c->stream);
     hc::gen_row_apply(c->gg, Gx, Gy, (const double*)c->m[0], (const double*)c->m[1],
                       (const double*)c->rf, Gx, Gy, c->st, c->stream);
-    hc::gen_col_div(c->gg, hc::CD_CG, Gx, Gy, nullptr, c->q64, c->st, c->stream);
-    hc::gen_cg_update(c->gg, c->p64, c->r64, c->d64, c->q64, c->st, c->stream);
-    c->launches += 4;
+    hc::gen_col_div_upd(c->gg, Gx, Gy, c->d64, c->p64, c->r64, c->st, c->stream);
+    c->launches += 3;
     return;
   }
   if (c->dim == 3) {
@@ -926,10 +934,8 @@ void plain_iter(hc_ctx* c) {
                                Gy, c->st, 1, c->stream);
   hc::row_apply<double, double>(g, Gx, Gy, (const double*)c->m[0], (const double*)c->m[1],
                                 (const double*)c->rf, Gx, Gy, c->st, c->stream);
-  hc::col_div<double>(g, hc::CD_CG, Gx, Gy, c->d64, nullptr, c->q64, nullptr, nullptr, c->st,
-                      c->stream);
-  hc::cg_update<double>(g, c->p64, c->r64, c->d64, c->q64, c->st, c->stream);
-  c->launches += 4;
+  hc::col_div_upd(g, Gx, Gy, c->d64, c->p64, c->r64, c->st, c->stream);
+  c->launches += 3;
 }
 
 // Refined modes: S - A p^k in FP32 from the warm start, the first inner
@@ -1445,8 +1451,9 @@ void abort_capture(cudaStream_t s) {
 // iteration, one FP64 refinement residual.
 void set_node_counts(hc_ctx* c) {
   const int split = c->dim == 3 ? 5 : 4, resid = c->dim == 3 ? 5 : 3;
-  c->graph_nodes_fixed = 1 + resid + split + 1;
-  c->graph_nodes_body = c->dim == 3 ? 6 : 4;
+  const int table = c->dim == 2 && !c->refined ? 1 : 0;  // the preconditioner symbol
+  c->graph_nodes_fixed = 1 + resid + table + split + 1;
+  c->graph_nodes_body = c->dim == 3 ? 6 : (c->refined ? 4 : 3);
   c->graph_nodes_outer = resid;
 }
 
@@ -1972,6 +1979,8 @@ int hc_create(hc_ctx** out, const hc_grid* grid, const hc_params* params, void* 
     c->gq.tc = c->gd.tc;
     c->gq.ltc = c->gd.ltc;
     c->gd.fx = c->refined ? 0 : 1;
+    c->gd.dots = c->dots;
+    c->gd.pinv = c->pinv64;
     c->gd.qx = c->twx_x;
     c->gd.qy = c->twy_x;
     c->gd.qz = c->twz_x;

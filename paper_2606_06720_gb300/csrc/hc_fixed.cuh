@@ -113,14 +113,15 @@ __device__ __forceinline__ long long fquarter1(long long v) {
 }
 __device__ __forceinline__ fxc fquarter(fxc v) { return fxc{fquarter1(v.x), fquarter1(v.y)}; }
 
-// t / sqrt(2): 2^63 / sqrt(2) = 2^32 * 0x5A82799A - 0x0310CDBE.
+// t / sqrt(2): 2^63 / sqrt(2) = 2^32 * 0x5A82799A - 0x0310CDBE; the rounding
+// constant holds the mean of the dropped low product as well.
 __device__ __forceinline__ long long fhalf_sqrt(long long t) {
   const int th = (int)(t >> 32);
   const unsigned tl = (unsigned)t;
   long long cross;
   asm("mad.wide.u32 %0, %1, %2, %3;"
       : "=l"(cross)
-      : "r"(tl), "r"(0x5A82799Au), "l"(0x40000000LL));
+      : "r"(tl), "r"(0x5A82799Au), "l"(0x40000000LL - 0x018866DF));
   cross = mad32(th, -0x0310CDBE, cross);
   return (mul32(th, 0x5A82799A) << 1) + (cross >> 31);
 }
@@ -201,6 +202,30 @@ __device__ __forceinline__ double fx_to(long long v, int eb) {
   return __hiloint2double(hi | (s & (int)0x80000000), (int)(unsigned)m);
 }
 
+// acc + (x 2^(1023 - E))^2 with off20 = (E - 127) 2^20, |x| 2^(1023 - E) < 2.
+__device__ __forceinline__ float fx_sumsq(float acc, double x, int off20) {
+  const int t = max((__double2hiint(x) & 0x7fffffff) - off20, 0);
+  const float f = __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)t, 3));
+  return fmaf(f, f, acc);
+}
+// Merge a partial (largest upper word, sum of squares relative to its exponent).
+__device__ __forceinline__ void fx_merge(int& em, float& a, int2 p) {
+  const int d = (em >> 20) - (p.x >> 20);  // bring both sums to the larger exponent
+  const float f = __int_as_float(max(127 - 2 * abs(d), 0) << 23);
+  a = d < 0 ? a * f + __int_as_float(p.y) : a + __int_as_float(p.y) * f;
+  em = max(em, p.x);
+}
+// S < 2^(k+1), k its exponent, so ||x|| < 2^(E - 1023 + (k + 2) / 2); the factor
+// covers the float sum's rounding.
+__device__ __forceinline__ FxScale fx_scale_of(int em, float a) {
+  const int k = (__float_as_int(a * 1.001f) >> 23) - 127, e = em >> 20;
+  FxScale sc;
+  sc.bad = e == 2047;
+  sc.small = e < 160;
+  sc.e = em == 0 ? 0 : e - 1023 + ((k + 2) >> 1) + (sc.small ? 512 : 0);
+  return sc;
+}
+
 // The scales of NV transforms: one per lane group.  Lanes of a transform are
 // `ks` apart within a warp, min(32 / ks, N/8) of them, and its warps follow one
 // another; the warps' partial maxima and sums meet in the transform's slab.
@@ -223,15 +248,10 @@ __device__ __forceinline__ void fx_scales(const cx<fx64> (&v)[NV][8], cx<fx64>* 
     E[q] = e;
     const int off20 = ((e >> 20) - 127) << 20;
     float a = 0.0f;
-    auto add = [&](double x) {  // (x 2^(1023 - E))^2, |x| 2^(1023 - E) < 2
-      const int t = max((__double2hiint(x) & 0x7fffffff) - off20, 0);
-      const float f = __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)t, 3));
-      a = fmaf(f, f, a);
-    };
 #pragma unroll
     for (int s = 0; s < 8; ++s) {
-      add(v[q][s].x.v);
-      add(v[q][s].y.v);
+      a = fx_sumsq(a, v[q][s].x.v, off20);
+      a = fx_sumsq(a, v[q][s].y.v, off20);
     }
     for (int off = ks; off < top; off <<= 1) a += __shfl_xor_sync(mask, a, off);
     S[q] = a;
@@ -251,26 +271,14 @@ __device__ __forceinline__ void fx_scales(const cx<fx64> (&v)[NV][8], cx<fx64>* 
     for (int q = 0; q < NV; ++q) {
       int em = 0;
       float a = 0.0f;
-      for (int i = 0; i < nw; ++i) {
-        const int2 p = *reinterpret_cast<const int2*>(sl[q] + (size_t)i * ks);
-        const int d = (em >> 20) - (p.x >> 20);  // bring both sums to the larger exponent
-        const float f = __int_as_float(max(127 - 2 * abs(d), 0) << 23);
-        a = d < 0 ? a * f + __int_as_float(p.y) : a + __int_as_float(p.y) * f;
-        em = max(em, p.x);
-      }
+      for (int i = 0; i < nw; ++i)
+        fx_merge(em, a, *reinterpret_cast<const int2*>(sl[q] + (size_t)i * ks));
       E[q] = em;
       S[q] = a;
     }
   }
 #pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    // S < 2^(k+1), k its exponent, so ||x|| < 2^(E - 1023 + (k + 2) / 2); the
-    // factor covers the float sum's rounding
-    const int k = (__float_as_int(S[q] * 1.001f) >> 23) - 127, e = E[q] >> 20;
-    sc[q].bad = e == 2047;
-    sc[q].small = e < 160;
-    sc[q].e = E[q] == 0 ? 0 : e - 1023 + ((k + 2) >> 1) + (sc[q].small ? 512 : 0);
-  }
+  for (int q = 0; q < NV; ++q) sc[q] = fx_scale_of(E[q], S[q]);
 }
 
 // ------------------------------------------------------------------ the passes
@@ -378,9 +386,10 @@ struct FxOut {
   double f1, f2;
 };
 __device__ __forceinline__ double fx_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-__device__ __forceinline__ FxOut fx_out(const FxScale& sc, int lN, int half) {
+// Integers v stand for v 2^(eb - 1085).
+__device__ __forceinline__ FxOut fx_out_at(const FxScale& sc, int eb) {
   FxOut o;
-  o.eb = 1024 + sc.e + 2 * (lN > 9 ? 3 : (lN > 6 ? 2 : 1)) - half;
+  o.eb = eb;
   o.plain = !sc.bad && !sc.small && o.eb <= 2045;
   o.f1 = o.f2 = 1.0;
   if (!o.plain) {
@@ -390,6 +399,9 @@ __device__ __forceinline__ FxOut fx_out(const FxScale& sc, int lN, int half) {
     o.f2 = fx_pow2(ex - ex / 2);
   }
   return o;
+}
+__device__ __forceinline__ FxOut fx_out(const FxScale& sc, int lN, int half) {
+  return fx_out_at(sc, 1024 + sc.e + 2 * (lN > 9 ? 3 : (lN > 6 ? 2 : 1)) - half);
 }
 
 // fft_canon for FP64 data of length 2^lN, lN >= kFxMinLog.

@@ -2,16 +2,22 @@
 // N = 2^a 3^b 5^c per axis, among them the paper's N = 50 2^k grids of its
 // grid-convergence study (Section 4, Tables 1-3).  FP64 throughout.
 //
-// Transforms are mixed-radix Stockham FFTs (radix 2, 3, 4, 5 passes) on one
-// transform per CTA, held in shared memory, with the CTA's threads sharing
-// each pass's butterflies.  The spectral state is the unpacked half spectrum:
+// Transforms are mixed-radix Stockham FFTs (radix 2, 3, 4, 5 passes) of one row,
+// or of a column's two fields together, held in a CTA's shared memory, with the
+// CTA's threads sharing each pass's butterflies.  Their arithmetic is the 64-bit
+// block fixed point of hc_fixed.cuh, because the FP64 pipe is narrow: with FP64
+// passes one transform at a time the four CG kernels of 400 x 400 took 108 us,
+// now 44.  Passes divide by 2: from an L2 norm of 2^61 the largest
+// growth up to 4096 points, 5^5, leaves every input of a pass below 2^61.7 and,
+// with a factor of at most sqrt(5) inside it, every value below 2^62.9.
+// The spectral state is the unpacked half spectrum:
 // ny rows of Hh = nx/2 + 1 values (kx = 0 .. nx/2), row-major, unnormalised
 // DFTs.  A step makes the same passes as the power-of-two path, each fused
 // with the same pointwise work:
 //   column gradient   d = M^-1 r + beta d (CG) or p, times i xi / n, inverse along y
 //   row apply         inverse along x, q = (m.g) m + r g, <d, A d> by parts, forward along x
 //   column divergence forward along y, -i xi . q^ (CG output or the residual S - A p)
-//   CG update         x += alpha d, r -= alpha A d, the two dot products
+//                     (CG: with x += alpha d, r -= alpha A d, the two dot products)
 //   split step        gradient, row pass with activation + relaxation, column
 //                     pass with the heat factor exp(-D^2 |xi|^2 dt), row back-transform
 // and the same one-thread solve bookkeeping (SolveState), so CG, its stopping
@@ -23,97 +29,181 @@ namespace hc {
 namespace {
 
 // ------------------------------------------------------------------ small DFTs
-// Kernel exp(S 2 pi i j k / R), natural order in and out.  The radix-3 and
-// radix-5 constants are the closed forms cos(2 pi/3) = -1/2,
-// sin(2 pi/3) = sqrt(3)/2, cos(2 pi/5) = (sqrt 5 - 1)/4,
-// cos(4 pi/5) = -(sqrt 5 + 1)/4, sin(2 pi/5) = sqrt(10 + 2 sqrt 5)/4,
-// sin(4 pi/5) = sqrt(10 - 2 sqrt 5)/4.
+// t c for a constant 0 < c < 1 with 2^62 c = 2^32 H + L, L signed; |t| <= 2^62.5.
+// The dropped product of the low limbs is L/2^31 on average: it joins the
+// rounding constant.
+template <int H, int L>
+__device__ __forceinline__ long long fmul_const(long long t) {
+  const int th = (int)(t >> 32);
+  long long cross;
+  asm("mad.wide.u32 %0, %1, %2, %3;"
+      : "=l"(cross)
+      : "r"((unsigned)t), "r"((unsigned)H), "l"(0x20000000LL + L / 2));
+  cross = mad32(th, L, cross);
+  return (mul32(th, H) << 2) + (cross >> 30);
+}
+// v w / 2 (fmul without half of its shift) and v / 2, rounded as fmul rounds.
+__device__ __forceinline__ fxc fmul2(fxc v, const FxW& w) {
+  const int vxl = (int)v.x, vyl = (int)v.y;
+  const unsigned bx = (unsigned)vxl >> 31, by = (unsigned)vyl >> 31;
+  const int vxh = (int)(v.x >> 32) + (int)bx;
+  const int vyh = (int)(v.y >> 32) + (int)by;
+  const long long cr = mad32(vyl, w.nh, mad32(vyh, w.nl, mad32(vxl, w.xh, mul32(vxh, w.xl))));
+  const long long ci = mad32(vyl, w.xh, mad32(vyh, w.xl, mad32(vxl, w.ph, mul32(vxh, w.pl))));
+  fxc r;
+  r.x = (mad32(vyh, w.nh, mul32(vxh, w.xh)) << 1) + ((cr + (long long)(0x3fffffffu + bx)) >> 31);
+  r.y = (mad32(vyh, w.xh, mul32(vxh, w.ph)) << 1) + ((ci + (long long)(0x3fffffffu + by)) >> 31);
+  return r;
+}
+__device__ __forceinline__ long long fhalf1(long long v) {
+  return (v + (long long)((unsigned)v >> 31)) >> 1;
+}
+
+// Kernel exp(S 2 pi i j k / R), natural order in and out.  Radix 3: cos(2 pi/3) =
+// -1/2, sin(2 pi/3) = sqrt(3)/2.  Radix 5: with c1, c2 = cos(2 pi/5), cos(4 pi/5),
+// c1 + c2 = -1/2 and c1 - c2 = sqrt(5)/2; s1, s2 = sin(2 pi/5), sin(4 pi/5) =
+// sqrt(10 +- 2 sqrt 5)/4, and s1 b1 + s2 b2, s2 b1 - s1 b2 share s2 (b1 + b2).
 template <int S>
-__device__ __forceinline__ void gdft3(cx<double>* v) {
-  const double h = 0.86602540378443864676;
-  const cx<double> a = cadd(v[1], v[2]), b = csub(v[1], v[2]);
-  const cx<double> t = cmk<double>(v[0].x - 0.5 * a.x, v[0].y - 0.5 * a.y);
-  const cx<double> u = cmul_si<S>(cmk<double>(h * b.x, h * b.y));
-  v[0] = cadd(v[0], a);
-  v[1] = cadd(t, u);
-  v[2] = csub(t, u);
+__device__ __forceinline__ void gdft3(fxc* v) {
+  const fxc a = fadd(v[1], v[2]), b = fsub(v[1], v[2]);
+  const fxc t = fxc{v[0].x - fhalf1(a.x), v[0].y - fhalf1(a.y)};
+  const fxc u = fmul_si<S>(fxc{fmul_const<929887697, -1332128537>(b.x),
+                               fmul_const<929887697, -1332128537>(b.y)});  // sqrt(3)/2
+  v[0] = fadd(v[0], a);
+  v[1] = fadd(t, u);
+  v[2] = fsub(t, u);
 }
 
 template <int S>
-__device__ __forceinline__ void gdft5(cx<double>* v) {
-  const double c1 = 0.30901699437494742410, c2 = -0.80901699437494742410;
-  const double s1 = 0.95105651629515357212, s2 = 0.58778525229247312917;
-  const cx<double> a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]);
-  const cx<double> a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
-  const cx<double> t1 = cmk<double>(v[0].x + c1 * a1.x + c2 * a2.x, v[0].y + c1 * a1.y + c2 * a2.y);
-  const cx<double> t2 = cmk<double>(v[0].x + c2 * a1.x + c1 * a2.x, v[0].y + c2 * a1.y + c1 * a2.y);
-  const cx<double> u1 =
-      cmul_si<S>(cmk<double>(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y));
-  const cx<double> u2 =
-      cmul_si<S>(cmk<double>(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y));
-  v[0] = cmk<double>(v[0].x + a1.x + a2.x, v[0].y + a1.y + a2.y);
-  v[1] = cadd(t1, u1);
-  v[4] = csub(t1, u1);
-  v[2] = cadd(t2, u2);
-  v[3] = csub(t2, u2);
+__device__ __forceinline__ void gdft5(fxc* v) {
+  const fxc a1 = fadd(v[1], v[4]), b1 = fsub(v[1], v[4]);
+  const fxc a2 = fadd(v[2], v[3]), b2 = fsub(v[2], v[3]);
+  const fxc a = fadd(a1, a2), d = fsub(a1, a2), e = fadd(b1, b2);
+  const fxc t = fxc{v[0].x - fquarter1(a.x), v[0].y - fquarter1(a.y)};
+  const fxc m = fxc{fmul_const<600239927, 803819395>(d.x), fmul_const<600239927, 803819395>(d.y)};  // sqrt(5)/4
+  const fxc p = fxc{fmul_const<631129609, -357254181>(e.x), fmul_const<631129609, -357254181>(e.y)};    // s2
+  const fxc q1 = fxc{fmul_const<390059550, -1644870943>(b1.x), fmul_const<390059550, -1644870943>(b1.y)};  // s1 - s2
+  const fxc q2 = fxc{b2.x + fmul_const<578576943, 1935587992>(b2.x), b2.y + fmul_const<578576943, 1935587992>(b2.y)};  // s1 + s2
+  const fxc u1 = fmul_si<S>(fadd(p, q1)), u2 = fmul_si<S>(fsub(p, q2));
+  const fxc t1 = fadd(t, m), t2 = fsub(t, m);
+  v[0] = fadd(v[0], a);
+  v[1] = fadd(t1, u1);
+  v[4] = fsub(t1, u1);
+  v[2] = fadd(t2, u2);
+  v[3] = fsub(t2, u2);
 }
 
-// One radix-R pass of a length-N Stockham FFT, by all threads of the CTA:
+// One radix-R pass of NB length-N Stockham FFTs, by all threads of the CTA:
 // butterfly j < N/R takes src[j + r N/R], r < R, twiddles element r by
 // w^(r k), k = j mod Ns, w = exp(S 2 pi i / (Ns R)) (a table entry
 // tw[m] = exp(-2 pi i m / N), conjugated for S = +1), and writes
 // dst[(j / Ns) Ns R + k + r Ns].
-template <int S, int R>
-__device__ __forceinline__ void gpass(const cx<double>* __restrict__ src, cx<double>* __restrict__ dst,
-                                      int N, int Ns, const cx<double>* __restrict__ tw) {
-  const int nb = N / R, step = N / (Ns * R);
-  for (int j = threadIdx.x; j < nb; j += blockDim.x) {
-    const int k = j % Ns;
-    cx<double> v[R];
+template <int S, int R, int NB>
+__device__ __forceinline__ void gpass(const fxc* __restrict__ src, fxc* __restrict__ dst, int N, int Ns,
+                                      const FxTw* __restrict__ tw) {
+  const int nb = N / R, step = nb / Ns;
+  const float inv = 1.0f / (float)Ns;
+  for (int i = threadIdx.x; i < NB * nb; i += blockDim.x) {
+    const int o = (NB > 1 && i >= nb) ? N : 0, j = o ? i - nb : i;
+    const int k = j - Ns * (int)(((float)j + 0.5f) * inv);  // j mod Ns
+    fxc v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = src[j + r * nb];
+    for (int r = 0; r < R; ++r) v[r] = src[o + j + r * nb];
     if (Ns > 1) {
+      v[0] = fxc{fhalf1(v[0].x), fhalf1(v[0].y)};
 #pragma unroll
-      for (int r = 1; r < R; ++r) {
-        cx<double> w = ldg(&tw[r * k * step]);
-        if (S > 0) w.y = -w.y;
-        v[r] = cmul(v[r], w);
-      }
+      for (int r = 1; r < R; ++r) v[r] = fmul2(v[r], fx_w<S>(tw, r * k * step));
     }
-    if constexpr (R == 2) dft2<S>(v[0], v[1]);
+    if constexpr (R == 2) {
+      const fxc t = v[0];
+      v[0] = fadd(t, v[1]);
+      v[1] = fsub(t, v[1]);
+    }
     if constexpr (R == 3) gdft3<S>(v);
-    if constexpr (R == 4) dft4<S>(v[0], v[1], v[2], v[3]);
+    if constexpr (R == 4) fdft4<S>(v[0], v[1], v[2], v[3]);
     if constexpr (R == 5) gdft5<S>(v);
-    const int base = (j / Ns) * Ns * R + k;
+    const int base = o + (j - k) * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) dst[base + r * Ns] = v[r];
   }
 }
 
-// Length-N transform of the values in a (scratch b), S = -1 forward, +1
-// inverse (unnormalised).  The caller synchronises after filling a; returns
-// the buffer that holds the result, synchronised.
-template <int S>
-__device__ cx<double>* gfft(cx<double>* a, cx<double>* b, int N, const int* rad, int np,
-                            const cx<double>* __restrict__ tw) {
+// NB length-N transforms of the values at a, a + N (scratch b, as long), S = -1
+// forward, +1 inverse (unnormalised).  The caller synchronises after filling a;
+// returns the buffer that holds the results, synchronised.
+template <int S, int NB = 1>
+__device__ cx<double>* gfft(cx<double>* ad, cx<double>* bd, int N, const int* rad, int np,
+                            const FxTw* __restrict__ tw) {
+  // scales (fx_scales): per warp first, relative to the warp's largest exponent
+  __shared__ int2 s_part[8 * NB];
+  FxScale sc[NB];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+  for (int t = 0; t < NB; ++t) {
+    const cx<double>* x = ad + t * N;
+    int e = 0;
+    for (int k = threadIdx.x; k < N; k += blockDim.x)
+      e = max(e, max(__double2hiint(x[k].x) & 0x7fffffff, __double2hiint(x[k].y) & 0x7fffffff));
+    e = __reduce_max_sync(0xffffffffu, e);
+    const int off20 = ((e >> 20) - 127) << 20;
+    float f2 = 0.0f;
+    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+      f2 = fx_sumsq(f2, x[k].x, off20);
+      f2 = fx_sumsq(f2, x[k].y, off20);
+    }
+    for (int off = 16; off > 0; off >>= 1) f2 += __shfl_xor_sync(0xffffffffu, f2, off);
+    if (lane == 0) s_part[t * 8 + warp] = make_int2(e, __float_as_int(f2));
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < NB; ++t) {
+    int em = 0;
+    float f2 = 0.0f;
+    for (int w = 0; w < nw; ++w) fx_merge(em, f2, s_part[t * 8 + w]);
+    sc[t] = fx_scale_of(em, f2);
+  }
+  fxc *a = reinterpret_cast<fxc*>(ad), *b = reinterpret_cast<fxc*>(bd);
+#pragma unroll
+  for (int t = 0; t < NB; ++t) {
+    const int b20 = ((1024 + sc[t].e) << 20) + 0xfffff;  // 2^61
+    const double up = sc[t].small ? 0x1p512 : 1.0;
+    for (int k = t * N + threadIdx.x; k < (t + 1) * N; k += blockDim.x) {
+      const cx<double> v = ad[k];
+      if (sc[t].small) a[k] = fxc{fx_from(v.x * up, b20), fx_from(v.y * up, b20)};
+      else a[k] = fxc{fx_from(v.x, b20), fx_from(v.y, b20)};
+    }
+  }
+  __syncthreads();
   int Ns = 1;
   for (int p = 0; p < np; ++p) {
     const int R = rad[p];
     if (R == 2)
-      gpass<S, 2>(a, b, N, Ns, tw);
+      gpass<S, 2, NB>(a, b, N, Ns, tw);
     else if (R == 3)
-      gpass<S, 3>(a, b, N, Ns, tw);
+      gpass<S, 3, NB>(a, b, N, Ns, tw);
     else if (R == 4)
-      gpass<S, 4>(a, b, N, Ns, tw);
+      gpass<S, 4, NB>(a, b, N, Ns, tw);
     else
-      gpass<S, 5>(a, b, N, Ns, tw);
+      gpass<S, 5, NB>(a, b, N, Ns, tw);
     __syncthreads();
-    cx<double>* t = a;
+    fxc* t = a;
     a = b;
     b = t;
     Ns *= R;
   }
-  return a;
+  cx<double>* rd = reinterpret_cast<cx<double>*>(a);
+#pragma unroll
+  for (int t = 0; t < NB; ++t) {
+    const FxOut o = fx_out_at(sc[t], 1024 + sc[t].e + np - 1);
+    for (int k = t * N + threadIdx.x; k < (t + 1) * N; k += blockDim.x) {
+      const fxc v = a[k];
+      cx<double> d = cmk<double>(fx_to(v.x, o.eb), fx_to(v.y, o.eb));
+      if (!o.plain) d = cmk<double>(d.x * o.f1 * o.f2, d.y * o.f1 * o.f2);
+      rd[k] = d;
+    }
+  }
+  __syncthreads();
+  return rd;
 }
 
 // Parseval weight of half-spectrum column kx: 1 for kx = 0 and (even nx) the
@@ -151,7 +241,9 @@ __device__ __forceinline__ void gstore_pair(const GenGeo& g, const cx<double>* Z
 }  // namespace
 
 // ------------------------------------------------------------------ column gradient
-template <int MODE>
+// NB = 2: both fields' transforms together; 1: one after the other (columns too
+// long for four buffers in shared memory).
+template <int MODE, int NB>
 __global__ void __launch_bounds__(256) gk_col_grad(GenGeo g, const cx<double>* __restrict__ in,
                                                    const cx<double>* __restrict__ rvec,
                                                    cx<double>* dio, cx<double>* __restrict__ Gx,
@@ -160,9 +252,8 @@ __global__ void __launch_bounds__(256) gk_col_grad(GenGeo g, const cx<double>* _
   if (check_done && st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int ny = g.ny, H = g.Hh, kx = blockIdx.x;
-  cx<double>* P = reinterpret_cast<cx<double>*>(smem_raw);
-  cx<double>* A = P + ny;
-  cx<double>* B = A + ny;
+  cx<double>* A = reinterpret_cast<cx<double>*>(smem_raw);
+  cx<double>* B = A + NB * ny;
   const double invn = 1.0 / ((double)g.nx * (double)ny);
   const double kxv = g.kxd[kx];
   bool first = false;
@@ -173,36 +264,38 @@ __global__ void __launch_bounds__(256) gk_col_grad(GenGeo g, const cx<double>* _
     beta = st->beta;
     pc = pc_of<double>(st);
   }
-  for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
-    const size_t idx = (size_t)ky * H + kx;
-    cx<double> v;
-    if constexpr (MODE == CG_DUPDATE) {
-      const cx<double> z = cscale(rvec[idx], pinv_ab(kxv, g.kyd[ky], pc));
-      v = first ? z : cadd(z, cscale(dio[idx], beta));
-      dio[idx] = v;
-    } else {
-      v = in[idx];
+  for (int q = 0; q < 2; q += NB) {
+    for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
+      const size_t idx = (size_t)ky * H + kx;
+      const double kyv = g.kyd[ky];
+      cx<double> v;
+      if (MODE != CG_DUPDATE) {
+        v = in[idx];
+      } else if (q > 0) {  // updated by this thread
+        v = dio[idx];
+      } else {
+        const cx<double> z = cscale(rvec[idx], g.pinv[idx]);
+        v = first ? z : cadd(z, cscale(dio[idx], beta));
+        dio[idx] = v;
+      }
+      const double a = kxv * invn, b = kyv * invn;
+      const cx<double> vx = cmk<double>(-a * v.y, a * v.x), vy = cmk<double>(-b * v.y, b * v.x);
+      A[ky] = q == 0 ? vx : vy;  // i (xi / n) P
+      if (NB > 1) A[ny + ky] = vy;
     }
-    P[ky] = v;
-    const double a = kxv * invn;
-    A[ky] = cmk<double>(-a * v.y, a * v.x);  // i (xi_x / n) P
+    __syncthreads();
+    const cx<double>* R = gfft<+1, NB>(A, B, ny, g.ry, g.nry, g.qy);
+    for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
+      (q == 0 ? Gx : Gy)[(size_t)ky * H + kx] = R[ky];
+      if (NB > 1) Gy[(size_t)ky * H + kx] = R[ny + ky];
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  cx<double>* R = gfft<+1>(A, B, ny, g.ry, g.nry, g.twy);
-  for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) Gx[(size_t)ky * H + kx] = R[ky];
-  __syncthreads();
-  for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
-    const double a = g.kyd[ky] * invn;
-    A[ky] = cmk<double>(-a * P[ky].y, a * P[ky].x);  // i (xi_y / n) P
-  }
-  __syncthreads();
-  R = gfft<+1>(A, B, ny, g.ry, g.nry, g.twy);
-  for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) Gy[(size_t)ky * H + kx] = R[ky];
 }
 
 // ------------------------------------------------------------------ row apply
-// DOT: the CG variant; alpha = rho / <d, A d> with <d, A d> = n sum g . K g
-// (summation by parts), as in the power-of-two row pass.
+// DOT: the CG variant; <d, A d> = n sum g . K g (summation by parts), as in the
+// power-of-two row pass, one partial per row.
 template <bool DOT>
 __global__ void __launch_bounds__(256) gk_row_apply(GenGeo g, const cx<double>* Gx,
                                                     const cx<double>* Gy,
@@ -217,7 +310,7 @@ __global__ void __launch_bounds__(256) gk_row_apply(GenGeo g, const cx<double>* 
   cx<double>* B = A + N;
   gload_pair(g, Gx + (size_t)y * H, Gy + (size_t)y * H, A);
   __syncthreads();
-  cx<double>* R = gfft<+1>(A, B, N, g.rx, g.nrx, g.twx);
+  cx<double>* R = gfft<+1>(A, B, N, g.rx, g.nrx, g.qx);
   double gkg = 0.0;
   const size_t ro = (size_t)y * N;
   for (int x = threadIdx.x; x < N; x += blockDim.x) {
@@ -228,39 +321,58 @@ __global__ void __launch_bounds__(256) gk_row_apply(GenGeo g, const cx<double>* 
     R[x] = cmk<double>(ax * mg + r * gx, ay * mg + r * gy);
   }
   __syncthreads();
-  cx<double>* R2 = gfft<-1>(R, R == A ? B : A, N, g.rx, g.nrx, g.twx);
+  cx<double>* R2 = gfft<-1>(R, R == A ? B : A, N, g.rx, g.nrx, g.qx);
   gstore_pair(g, R2, Qx + (size_t)y * H, Qy + (size_t)y * H);
   if (DOT) {
-    double a1[1] = {gkg}, t1[1];
-    if (last_cta_sum<1>(a1, g.partials, &st->ticket[TK_DIV], t1) && threadIdx.x == 0)
-      cg_alpha_from(st, t1[0], (double)g.nx * (double)g.ny);
+    double a1[1] = {gkg};  // the CTA's partial: gk_col_div_upd forms alpha
+    block_sum<1>(a1);
+    if (threadIdx.x == 0) g.dots[blockIdx.x] = a1[0];
   }
 }
 
 // ------------------------------------------------------------------ column divergence
-// -i (xi_x Qx^ + xi_y Qy^) after the forward transforms along y.  CD_PLAIN:
-// written to out; CD_CG: the CG's A d (alpha came from the row pass);
-// CD_RESID: out = b - A p and the CG start (plain solve).
-template <int MODE>
+// The forward transforms along y of a column's two fields, in shared memory.
+template <int NB>
+__device__ __forceinline__ void gdiv_fields(const GenGeo& g, const cx<double>* __restrict__ Qx,
+                                            const cx<double>* __restrict__ Qy, const cx<double>*& Rx,
+                                            const cx<double>*& Ry) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int ny = g.ny, H = g.Hh, kx = blockIdx.x;
+  cx<double>* A = reinterpret_cast<cx<double>*>(smem_raw);
+  cx<double>* B = A + NB * ny;
+  for (int q = 0; q < 2; q += NB) {
+    for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
+      const size_t idx = (size_t)ky * H + kx;
+      A[ky] = (q == 0 ? Qx : Qy)[idx];
+      if (NB > 1) A[ny + ky] = Qy[idx];
+    }
+    __syncthreads();
+    const cx<double>* R = gfft<-1, NB>(A, B, ny, g.ry, g.nry, g.qy);
+    if (NB > 1) {
+      Rx = R;
+      Ry = R + ny;
+    } else if (q == 0) {  // waits in a third buffer
+      cx<double>* T = B + ny;
+      for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) T[ky] = R[ky];
+      Rx = T;
+      __syncthreads();
+    } else {
+      Ry = R;
+    }
+  }
+}
+
+// -i (xi_x Qx^ + xi_y Qy^) after those.  CD_PLAIN: written to out; CD_RESID: out =
+// b - A p and the CG start.
+template <int MODE, int NB>
 __global__ void __launch_bounds__(256) gk_col_div(GenGeo g, const cx<double>* __restrict__ Qx,
                                                   const cx<double>* __restrict__ Qy,
                                                   const cx<double>* __restrict__ bvec,
                                                   cx<double>* __restrict__ out, SolveState* st) {
-  if (MODE == CD_CG && st->done) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   const int ny = g.ny, H = g.Hh, kx = blockIdx.x;
-  cx<double>* T = reinterpret_cast<cx<double>*>(smem_raw);
-  cx<double>* A = T + ny;
-  cx<double>* B = A + ny;
   const double kxv = g.kxd[kx];
-  for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) A[ky] = Qx[(size_t)ky * H + kx];
-  __syncthreads();
-  cx<double>* R = gfft<-1>(A, B, ny, g.ry, g.nry, g.twy);
-  for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) T[ky] = cscale(R[ky], kxv);
-  __syncthreads();
-  for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) A[ky] = Qy[(size_t)ky * H + kx];
-  __syncthreads();
-  R = gfft<-1>(A, B, ny, g.ry, g.nry, g.twy);
+  const cx<double>*Rx, *R;
+  gdiv_fields<NB>(g, Qx, Qy, Rx, R);
   const double w = gweight(g, kx);
   double acc[2] = {0.0, 0.0};
   Pc<double> pc{};
@@ -268,7 +380,7 @@ __global__ void __launch_bounds__(256) gk_col_div(GenGeo g, const cx<double>* __
   for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
     const size_t idx = (size_t)ky * H + kx;
     const double b = g.kyd[ky];
-    const cx<double> t = cmk<double>(T[ky].x + b * R[ky].x, T[ky].y + b * R[ky].y);
+    const cx<double> t = cmk<double>(kxv * Rx[ky].x + b * R[ky].x, kxv * Rx[ky].y + b * R[ky].y);
     const cx<double> q = cmk<double>(t.y, -t.x);
     if constexpr (MODE == CD_RESID) {
       const cx<double> rv = csub(bvec[idx], q);
@@ -288,35 +400,58 @@ __global__ void __launch_bounds__(256) gk_col_div(GenGeo g, const cx<double>* __
 }
 
 // ------------------------------------------------------------------ CG update
-__global__ void __launch_bounds__(256) gk_cg_update(GenGeo g, cx<double>* __restrict__ x,
-                                                    cx<double>* __restrict__ r,
-                                                    const cx<double>* __restrict__ d,
-                                                    const cx<double>* __restrict__ q,
-                                                    SolveState* st) {
+// The preconditioner symbol of the running step (k_pinv_table).
+__global__ void __launch_bounds__(256) gk_pinv_table(GenGeo g, const SolveState* st) {
+  const Pc<double> pc = pc_of<double>(st);
+  const size_t total = (size_t)g.ny * g.Hh;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+       i += (size_t)gridDim.x * blockDim.x)
+    g.pinv[i] = pinv_ab(g.kxd[i % (size_t)g.Hh], g.kyd[i / (size_t)g.Hh], pc);
+}
+
+// Divergence pass and CG update in one (k_col_div_upd): with alpha from the row
+// pass's partials, x += alpha d, r -= alpha A d and the sums for beta.
+template <int NB>
+__global__ void __launch_bounds__(256) gk_col_div_upd(GenGeo g, const cx<double>* __restrict__ Qx,
+                                                      const cx<double>* __restrict__ Qy,
+                                                      const cx<double>* __restrict__ d,
+                                                      cx<double>* __restrict__ x,
+                                                      cx<double>* __restrict__ r, SolveState* st) {
   if (st->done) {
     if (st->graph_mode && blockIdx.x == 0 && threadIdx.x == 0)
       cudaGraphSetConditional(st->h_cur, 0u);
     return;
   }
-  const double alpha = st->alpha;
-  const Pc<double> pc = pc_of<double>(st);
-  const int H = g.Hh;
-  const size_t total = (size_t)g.ny * H;
-  double rr = 0.0, rz = 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int kx = (int)(i % (size_t)H), ky = (int)(i / (size_t)H);
-    const cx<double> dv = d[i], qv = q[i];
-    x[i] = cmk<double>(x[i].x + alpha * dv.x, x[i].y + alpha * dv.y);
-    const cx<double> rv = cmk<double>(r[i].x - alpha * qv.x, r[i].y - alpha * qv.y);
-    r[i] = rv;
-    const double w = gweight(g, kx), r2 = rv.x * rv.x + rv.y * rv.y;
-    rr += w * r2;
-    rz += w * r2 * pinv_ab(g.kxd[kx], g.kyd[ky], pc);
-  }
-  double acc[2] = {rr, rz}, tot[2];
+  const double rho = st->rho, n = (double)g.nx * (double)g.ny;
+  const double share = dots_share(g.dots, g.ny);
+  const cx<double>*Rx, *Ry;
+  gdiv_fields<NB>(g, Qx, Qy, Rx, Ry);
+  const double gkg = dots_total(share), dq = gkg * n;
+  const bool ok = dq > 0 && isfinite(dq);
+  const double alpha = ok ? rho / dq : 0.0;
+  const int H = g.Hh, kx = blockIdx.x;
+  const double w = gweight(g, kx), kxv = g.kxd[kx];
+  double acc[2] = {0.0, 0.0};
+  if (ok)
+    for (int ky = threadIdx.x; ky < g.ny; ky += blockDim.x) {
+      const size_t i = (size_t)ky * H + kx;
+      const double b = g.kyd[ky];
+      // A d = (t.y, -t.x)
+      const cx<double> t = cmk<double>(kxv * Rx[ky].x + b * Ry[ky].x, kxv * Rx[ky].y + b * Ry[ky].y);
+      const cx<double> dv = d[i], xv = x[i];
+      cx<double> rv = r[i];
+      x[i] = cmk<double>(xv.x + alpha * dv.x, xv.y + alpha * dv.y);
+      rv = cmk<double>(rv.x - alpha * t.y, rv.y + alpha * t.x);
+      r[i] = rv;
+      const double r2 = rv.x * rv.x + rv.y * rv.y;
+      acc[0] += r2;
+      acc[1] += r2 * g.pinv[i];
+    }
+  acc[0] *= w;
+  acc[1] *= w;
+  double tot[2];
   if (last_cta_sum<2>(acc, g.partials, &st->ticket[TK_UPDATE], tot) && threadIdx.x == 0)
-    cg_step_finish(st, tot[0], tot[1]);
+    cg_fused_finish(st, gkg, n, tot[0], tot[1]);
 }
 
 // ------------------------------------------------------------------ split step
@@ -335,7 +470,7 @@ __global__ void __launch_bounds__(256) gk_row_split(GenGeo g, cx<double>* Gx, cx
   cx<double>* B = A + N;
   gload_pair(g, Gx + (size_t)y * H, Gy + (size_t)y * H, A);
   __syncthreads();
-  cx<double>* R = gfft<+1>(A, B, N, g.rx, g.nrx, g.twx);
+  cx<double>* R = gfft<+1>(A, B, N, g.rx, g.nrx, g.qx);
   const size_t ro = (size_t)y * N;
   const bool diag = st->diag != 0;
   bool finite = true;
@@ -351,36 +486,41 @@ __global__ void __launch_bounds__(256) gk_row_split(GenGeo g, cx<double>* Gx, cx
   if (!finite) st->nonfinite = 1;
   if (diag) en.finish(g.partials, st);
   __syncthreads();
-  cx<double>* R2 = gfft<-1>(R, R == A ? B : A, N, g.rx, g.nrx, g.twx);
+  cx<double>* R2 = gfft<-1>(R, R == A ? B : A, N, g.rx, g.nrx, g.qx);
   gstore_pair(g, R2, Gx + (size_t)y * H, Gy + (size_t)y * H);
 }
 
 // Column pass of the diffusion, in place: forward along y, times
 // exp(-D^2 |xi|^2 dt) / n (eq. diffusion_space_discrete), inverse along y.
 // With diagnostics, sum |grad m_new|^2 = n sum w |xi~|^2 |v|^2 (v = F(m_new)/n).
+template <int NB>
 __global__ void __launch_bounds__(256) gk_col_heat(GenGeo g, cx<double>* Mx, cx<double>* My,
                                                    SolveState* st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int ny = g.ny, H = g.Hh, kx = blockIdx.x;
   cx<double>* A = reinterpret_cast<cx<double>*>(smem_raw);
-  cx<double>* B = A + ny;
+  cx<double>* B = A + NB * ny;
   const double invn = 1.0 / ((double)g.nx * (double)ny);
   const double w = gweight(g, kx), a = g.kxd[kx];
   double gm = 0.0;
-  for (int f = 0; f < 2; ++f) {
-    cx<double>* M = f == 0 ? Mx : My;
-    for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) A[ky] = M[(size_t)ky * H + kx];
+  for (int f = 0; f < 2; f += NB) {
+    for (int t = 0; t < NB; ++t)
+      for (int ky = threadIdx.x; ky < ny; ky += blockDim.x)
+        A[t * ny + ky] = (f + t == 0 ? Mx : My)[(size_t)ky * H + kx];
     __syncthreads();
-    cx<double>* R = gfft<-1>(A, B, ny, g.ry, g.nry, g.twy);
-    for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
-      const cx<double> v = cscale(R[ky], g.hx[kx] * g.hy[ky] * invn);
-      R[ky] = v;
-      const double b = g.kyd[ky];
-      gm += w * (a * a + b * b) * (v.x * v.x + v.y * v.y);
-    }
+    cx<double>* R = gfft<-1, NB>(A, B, ny, g.ry, g.nry, g.qy);
+    for (int t = 0; t < NB; ++t)
+      for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
+        const cx<double> v = cscale(R[t * ny + ky], g.hx[kx] * g.hy[ky] * invn);
+        R[t * ny + ky] = v;
+        const double b = g.kyd[ky];
+        gm += w * (a * a + b * b) * (v.x * v.x + v.y * v.y);
+      }
     __syncthreads();
-    cx<double>* R2 = gfft<+1>(R, R == A ? B : A, ny, g.ry, g.nry, g.twy);
-    for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) M[(size_t)ky * H + kx] = R2[ky];
+    cx<double>* R2 = gfft<+1, NB>(R, R == A ? B : A, ny, g.ry, g.nry, g.qy);
+    for (int t = 0; t < NB; ++t)
+      for (int ky = threadIdx.x; ky < ny; ky += blockDim.x)
+        (f + t == 0 ? Mx : My)[(size_t)ky * H + kx] = R2[t * ny + ky];
     __syncthreads();
   }
   if (st && st->diag) gradnorm_finish(gm, (double)g.nx * (double)ny, g.partials, st, 1);
@@ -398,7 +538,7 @@ __global__ void __launch_bounds__(256) gk_row_c2r(GenGeo g, const cx<double>* A,
   cx<double>* W = Z + N;
   gload_pair(g, A + (size_t)y * H, B ? B + (size_t)y * H : nullptr, Z);
   __syncthreads();
-  cx<double>* R = gfft<+1>(Z, W, N, g.rx, g.nrx, g.twx);
+  cx<double>* R = gfft<+1>(Z, W, N, g.rx, g.nrx, g.qx);
   const size_t ro = (size_t)y * N;
   const bool diag = kappa_update && st->diag;
   double mxx = 0, myy = 0, mxy = 0, d2 = 0;
@@ -441,7 +581,7 @@ __global__ void __launch_bounds__(256) gk_row_fwd(GenGeo g, const double* __rest
   for (int x = threadIdx.x; x < N; x += blockDim.x)
     Z[x] = cmk<double>(a[ro + x], b ? b[ro + x] : 0.0);
   __syncthreads();
-  cx<double>* R = gfft<-1>(Z, W, N, g.rx, g.nrx, g.twx);
+  cx<double>* R = gfft<-1>(Z, W, N, g.rx, g.nrx, g.qx);
   gstore_pair(g, R, A + (size_t)y * H, B ? B + (size_t)y * H : nullptr);
 }
 
@@ -465,7 +605,7 @@ __global__ void __launch_bounds__(256) gk_col_fwd(GenGeo g, const cx<double>* in
     cx<double>* out = f == 0 ? out0 : out1;
     for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) A[ky] = in[(size_t)ky * H + kx];
     __syncthreads();
-    cx<double>* R = gfft<-1>(A, B, ny, g.ry, g.nry, g.twy);
+    cx<double>* R = gfft<-1>(A, B, ny, g.ry, g.nry, g.qy);
     for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
       cx<double> v = R[ky];
       if (project && f == 0 && gnull(g, kx, ky)) v = czero<double>();
@@ -498,7 +638,7 @@ __global__ void __launch_bounds__(256) gk_col_inv(GenGeo g, const cx<double>* in
   cx<double>* B = A + ny;
   for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) A[ky] = in[(size_t)ky * H + kx];
   __syncthreads();
-  cx<double>* R = gfft<+1>(A, B, ny, g.ry, g.nry, g.twy);
+  cx<double>* R = gfft<+1>(A, B, ny, g.ry, g.nry, g.qy);
   for (int ky = threadIdx.x; ky < ny; ky += blockDim.x)
     out[(size_t)ky * H + kx] = cscale(R[ky], scale);
 }
@@ -508,6 +648,15 @@ namespace {
 constexpr int kGenThreads = 256;
 size_t gcol_smem(const GenGeo& g, int bufs) { return (size_t)bufs * g.ny * sizeof(cx<double>); }
 size_t grow_smem(const GenGeo& g) { return (size_t)2 * g.nx * sizeof(cx<double>); }
+// Columns whose two fields fit shared memory together (two buffers each).
+bool gpair(const GenGeo& g) { return g.ny <= 3000; }
+// Threads for `points` of a CTA's transforms: two points each (the passes of a
+// radix-4 butterfly leave half of them idle, but the conversions and pointwise
+// loops are longer: 400^2 row pass 30 us at four points a thread, 22 at two).
+int gthreads(int points) {
+  const int t = (points / 2 + 31) / 32 * 32;
+  return t < 64 ? 64 : (t > kGenThreads ? kGenThreads : t);
+}
 int gupd_blocks(const GenGeo& g) {
   const size_t b = ((size_t)g.ny * g.Hh + kGenThreads - 1) / kGenThreads;
   return (int)(b < 608 ? b : 608);
@@ -517,70 +666,77 @@ int gupd_blocks(const GenGeo& g) {
 void gen_col_grad(const GenGeo& g, int mode, const cx<double>* in, const cx<double>* rvec,
                   cx<double>* dio, cx<double>* Gx, cx<double>* Gy, SolveState* st, int check_done,
                   cudaStream_t s) {
-  if (mode == CG_DUPDATE)
-    gk_col_grad<CG_DUPDATE><<<g.Hh, kGenThreads, gcol_smem(g, 3), s>>>(g, in, rvec, dio, Gx, Gy, st,
-                                                                       check_done);
-  else
-    gk_col_grad<CG_PLAIN><<<g.Hh, kGenThreads, gcol_smem(g, 3), s>>>(g, in, rvec, dio, Gx, Gy, st,
+  const auto k = mode == CG_DUPDATE
+                     ? (gpair(g) ? gk_col_grad<CG_DUPDATE, 2> : gk_col_grad<CG_DUPDATE, 1>)
+                     : (gpair(g) ? gk_col_grad<CG_PLAIN, 2> : gk_col_grad<CG_PLAIN, 1>);
+  k<<<g.Hh, gthreads(2 * g.ny), gcol_smem(g, gpair(g) ? 4 : 2), s>>>(g, in, rvec, dio, Gx, Gy, st,
                                                                      check_done);
 }
 void gen_row_apply(const GenGeo& g, const cx<double>* Gx, const cx<double>* Gy, const double* mx,
                    const double* my, const double* r, cx<double>* Qx, cx<double>* Qy,
                    SolveState* st, cudaStream_t s) {
   if (st)
-    gk_row_apply<true><<<g.ny, kGenThreads, grow_smem(g), s>>>(g, Gx, Gy, mx, my, r, Qx, Qy, st);
+    gk_row_apply<true><<<g.ny, gthreads(g.nx), grow_smem(g), s>>>(g, Gx, Gy, mx, my, r, Qx, Qy, st);
   else
-    gk_row_apply<false><<<g.ny, kGenThreads, grow_smem(g), s>>>(g, Gx, Gy, mx, my, r, Qx, Qy, st);
+    gk_row_apply<false><<<g.ny, gthreads(g.nx), grow_smem(g), s>>>(g, Gx, Gy, mx, my, r, Qx, Qy, st);
 }
 void gen_col_div(const GenGeo& g, int mode, const cx<double>* Qx, const cx<double>* Qy,
                  const cx<double>* b, cx<double>* out, SolveState* st, cudaStream_t s) {
-  if (mode == CD_RESID)
-    gk_col_div<CD_RESID><<<g.Hh, kGenThreads, gcol_smem(g, 3), s>>>(g, Qx, Qy, b, out, st);
-  else if (mode == CD_CG)
-    gk_col_div<CD_CG><<<g.Hh, kGenThreads, gcol_smem(g, 3), s>>>(g, Qx, Qy, b, out, st);
-  else
-    gk_col_div<CD_PLAIN><<<g.Hh, kGenThreads, gcol_smem(g, 3), s>>>(g, Qx, Qy, b, out, st);
+  const auto k = mode == CD_RESID ? (gpair(g) ? gk_col_div<CD_RESID, 2> : gk_col_div<CD_RESID, 1>)
+                                  : (gpair(g) ? gk_col_div<CD_PLAIN, 2> : gk_col_div<CD_PLAIN, 1>);
+  k<<<g.Hh, gthreads(2 * g.ny), gcol_smem(g, gpair(g) ? 4 : 3), s>>>(g, Qx, Qy, b, out, st);
 }
-void gen_cg_update(const GenGeo& g, cx<double>* x, cx<double>* r, const cx<double>* d,
-                   const cx<double>* q, SolveState* st, cudaStream_t s) {
-  gk_cg_update<<<gupd_blocks(g), kGenThreads, 0, s>>>(g, x, r, d, q, st);
+void gen_pinv_table(const GenGeo& g, const SolveState* st, cudaStream_t s) {
+  gk_pinv_table<<<gupd_blocks(g), kGenThreads, 0, s>>>(g, st);
+}
+void gen_col_div_upd(const GenGeo& g, const cx<double>* Qx, const cx<double>* Qy, const cx<double>* d,
+                     cx<double>* x, cx<double>* r, SolveState* st, cudaStream_t s) {
+  const auto k = gpair(g) ? gk_col_div_upd<2> : gk_col_div_upd<1>;
+  k<<<g.Hh, gthreads(2 * g.ny), gcol_smem(g, gpair(g) ? 4 : 3), s>>>(g, Qx, Qy, d, x, r, st);
 }
 void gen_row_split(const GenGeo& g, cx<double>* Gx, cx<double>* Gy, const double* mx,
                    const double* my, const double* r, SplitCoef cf, SolveState* st,
                    cudaStream_t s) {
-  gk_row_split<<<g.ny, kGenThreads, grow_smem(g), s>>>(g, Gx, Gy, mx, my, r, cf, st);
+  gk_row_split<<<g.ny, gthreads(g.nx), grow_smem(g), s>>>(g, Gx, Gy, mx, my, r, cf, st);
 }
 void gen_col_heat(const GenGeo& g, cx<double>* Mx, cx<double>* My, SolveState* st, cudaStream_t s) {
-  gk_col_heat<<<g.Hh, kGenThreads, gcol_smem(g, 2), s>>>(g, Mx, My, st);
+  const auto k = gpair(g) ? gk_col_heat<2> : gk_col_heat<1>;
+  k<<<g.Hh, gthreads(2 * g.ny), gcol_smem(g, gpair(g) ? 4 : 2), s>>>(g, Mx, My, st);
 }
 void gen_row_c2r(const GenGeo& g, const cx<double>* A, const cx<double>* B, double* a, double* b,
                  SolveState* st, int kappa_update, cudaStream_t s) {
-  gk_row_c2r<<<g.ny, kGenThreads, grow_smem(g), s>>>(g, A, B, a, b, st, kappa_update);
+  gk_row_c2r<<<g.ny, gthreads(g.nx), grow_smem(g), s>>>(g, A, B, a, b, st, kappa_update);
 }
 void gen_row_fwd(const GenGeo& g, const double* a, const double* b, cx<double>* A, cx<double>* B,
                  cudaStream_t s) {
-  gk_row_fwd<<<g.ny, kGenThreads, grow_smem(g), s>>>(g, a, b, A, B);
+  gk_row_fwd<<<g.ny, gthreads(g.nx), grow_smem(g), s>>>(g, a, b, A, B);
 }
 void gen_col_fwd(const GenGeo& g, const cx<double>* in0, const cx<double>* in1, cx<double>* out0,
                  cx<double>* out1, int project, int gradnorm, SolveState* st, cudaStream_t s) {
-  gk_col_fwd<<<g.Hh, kGenThreads, gcol_smem(g, 2), s>>>(g, in0, in1, out0, out1, project, gradnorm,
+  gk_col_fwd<<<g.Hh, gthreads(g.ny), gcol_smem(g, 2), s>>>(g, in0, in1, out0, out1, project, gradnorm,
                                                         st);
 }
 void gen_col_inv(const GenGeo& g, const cx<double>* in, cx<double>* out, double scale,
                  cudaStream_t s) {
-  gk_col_inv<<<g.Hh, kGenThreads, gcol_smem(g, 2), s>>>(g, in, out, scale);
+  gk_col_inv<<<g.Hh, gthreads(g.ny), gcol_smem(g, 2), s>>>(g, in, out, scale);
 }
 
 void set_smem_limits_gen() {
-  allow_smem(gk_col_grad<CG_PLAIN>);
-  allow_smem(gk_col_grad<CG_DUPDATE>);
+  allow_smem(gk_col_grad<CG_PLAIN, 1>);
+  allow_smem(gk_col_grad<CG_PLAIN, 2>);
+  allow_smem(gk_col_grad<CG_DUPDATE, 1>);
+  allow_smem(gk_col_grad<CG_DUPDATE, 2>);
   allow_smem(gk_row_apply<true>);
   allow_smem(gk_row_apply<false>);
-  allow_smem(gk_col_div<CD_PLAIN>);
-  allow_smem(gk_col_div<CD_CG>);
-  allow_smem(gk_col_div<CD_RESID>);
+  allow_smem(gk_col_div<CD_PLAIN, 1>);
+  allow_smem(gk_col_div<CD_PLAIN, 2>);
+  allow_smem(gk_col_div_upd<1>);
+  allow_smem(gk_col_div_upd<2>);
+  allow_smem(gk_col_div<CD_RESID, 1>);
+  allow_smem(gk_col_div<CD_RESID, 2>);
   allow_smem(gk_row_split);
-  allow_smem(gk_col_heat);
+  allow_smem(gk_col_heat<1>);
+  allow_smem(gk_col_heat<2>);
   allow_smem(gk_row_c2r);
   allow_smem(gk_row_fwd);
   allow_smem(gk_col_fwd);

@@ -292,6 +292,8 @@ struct Geo {
   int pipe;                  // 1: column passes run persistent with cp.async double buffering
   int pgrid;                 // CTAs of a persistent column pass (<= SMs, <= tiles)
   int fx;                    // Geo<double>: launch the fx64 kernels (as_fx)
+  double* dots;              // plain FP64 CG: the row pass's per-CTA sums of <d, A d>
+  double* pinv;              // plain FP64 CG: the running step's preconditioner symbol, as the spectra
   const FxTw* qx;            // Geo<double>: twiddle tables of the fx64 kernels
   const FxTw* qy;
   const FxTw* qz;
@@ -340,13 +342,15 @@ struct GenGeo {
   int nx, ny, Hh;
   int rx[kGenMaxPasses], nrx;  // radices (2, 3, 4, 5) of the x transform, product nx
   int ry[kGenMaxPasses], nry;  // the same along y
-  const cx<double>* twx;       // exp(-2 pi i m / nx), m < nx
-  const cx<double>* twy;       // exp(-2 pi i m / ny), m < ny
+  const FxTw* qx;              // exp(-2 pi i m / nx), m < nx, in Q62
+  const FxTw* qy;              // exp(-2 pi i m / ny), m < ny
   const double* kxd;           // first-derivative multipliers, kx < Hh (0 at the Nyquist index)
   const double* kyd;           // the same, ky < ny
   const double* hx;            // heat factor exp(-D^2 xi_x^2 dt), kx < Hh
   const double* hy;            // exp(-D^2 xi_y^2 dt), ky < ny
   double* partials;            // per-CTA FP64 partial sums
+  double* dots;                // the row pass's per-CTA sums of <d, A d>
+  double* pinv;                // the running step's preconditioner symbol, as the spectra
 };
 
 // One member of a batched size class of the parameter sweep (2D grids of one
@@ -588,6 +592,11 @@ void set_smem_limits_3d_df();
 // Opt every kernel of one precision in to the full shared memory per block.
 void set_smem_limits_f32();
 void set_smem_limits_f64();
+// Plain FP64 CG (2D, fx64): the step's preconditioner table, and the divergence
+// pass with the CG update.
+void pinv_table(const Geo<double>& g, const SolveState* st, cudaStream_t s);
+void col_div_upd(const Geo<double>& g, const cx<double>* Qx, const cx<double>* Qy, const cx<double>* d,
+                 cx<double>* x, cx<double>* r, SolveState* st, cudaStream_t s);
 void set_smem_limits_fx(int refined);
 // Lagged certification (2D refined steps): the FP64 certifying residual of
 // pressure p with the FP32 m, r it was solved with (sc: the certifying state,
@@ -640,8 +649,9 @@ void gen_row_apply(const GenGeo& g, const cx<double>* Gx, const cx<double>* Gy, 
                    SolveState* st, cudaStream_t s);
 void gen_col_div(const GenGeo& g, int mode, const cx<double>* Qx, const cx<double>* Qy,
                  const cx<double>* b, cx<double>* out, SolveState* st, cudaStream_t s);
-void gen_cg_update(const GenGeo& g, cx<double>* x, cx<double>* r, const cx<double>* d,
-                   const cx<double>* q, SolveState* st, cudaStream_t s);
+void gen_pinv_table(const GenGeo& g, const SolveState* st, cudaStream_t s);
+void gen_col_div_upd(const GenGeo& g, const cx<double>* Qx, const cx<double>* Qy, const cx<double>* d,
+                     cx<double>* x, cx<double>* r, SolveState* st, cudaStream_t s);
 void gen_row_split(const GenGeo& g, cx<double>* Gx, cx<double>* Gy, const double* mx,
                    const double* my, const double* r, SplitCoef cf, SolveState* st, cudaStream_t s);
 void gen_col_heat(const GenGeo& g, cx<double>* Mx, cx<double>* My, SolveState* st, cudaStream_t s);

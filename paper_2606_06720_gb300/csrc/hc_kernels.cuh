@@ -974,6 +974,11 @@ __device__ __forceinline__ void row_apply_body(Geo<T> g, const cx<T>* Gx, const 
       // FP32: the CTA's partial only; the divergence pass forms alpha
       // (cg_alpha_finish), so this pass ends without a fence or ticket
       cta_pair_partial(gkg, 0.0f, g.partials, blockIdx.x);
+    } else if constexpr (std::is_same<T, fx64>::value) {
+      // the CTA's partial only, as FP32: every CTA of k_col_div_upd forms alpha
+      double a1[1] = {(double)gkg};
+      block_sum<1>(a1);
+      if (threadIdx.x == 0) g.dots[blockIdx.x] = a1[0];
     } else {
       double a1[1] = {(double)gkg}, t1[1];
       if (last_cta_sum<1>(a1, g.partials, &st->ticket[TK_DIV], t1) && threadIdx.x == 0)
@@ -1540,7 +1545,7 @@ __device__ __forceinline__ void col_grad_body(Geo<T> g, cx<Tin>* in, const cx<T>
         } else if constexpr (MODE == CG_PLAIN) {
           P = ccast<T>(in[idx]);
         } else if constexpr (MODE == CG_DUPDATE) {
-          const cx<T> z = cscale(rvec[idx], pinv_sym(g, c.kx, ky, pc));
+          const cx<T> z = cscale(rvec[idx], T(g.pinv[idx]));
           P = first ? z : cadd(z, cscale(dio[idx], beta));
           dio[idx] = P;
         } else {
@@ -1754,6 +1759,43 @@ __global__ void __launch_bounds__(cta_bound<T>(col_cta_max<T, true>()), 1) k_col
                                                  cx<float>* __restrict__ delta32, SolveState* st) {
   col_div_body<T, MODE>(g, Qx, Qy, d, bvec, out, r32, delta32, st);
 }
+
+// ------------------------------------------------------------------ plain FP64 CG
+// The preconditioner symbol of the running step as a table: its division is a
+// dozen FP64 instructions, twice per value and iteration, against 8 bytes read.
+__global__ void __launch_bounds__(256) k_pinv_table(Geo<double> g, const SolveState* st);
+
+// The step length from the row pass's per-CTA sums, in every CTA alike: this
+// thread's share (loaded early, before the transforms), then the sum.
+__device__ __forceinline__ double dots_share(const double* dots, int np) {
+  double a = 0.0;
+  for (int i = threadIdx.x; i < np; i += blockDim.x) a += __ldcg(&dots[i]);
+  return a;
+}
+__device__ __forceinline__ double dots_total(double share) {
+  __shared__ double s_dot;
+  double a[1] = {share};
+  block_sum<1>(a);
+  if (threadIdx.x == 0) s_dot = a[0];
+  __syncthreads();
+  return s_dot;
+}
+// End of an iteration in the fused pass (the last CTA's first thread): the step
+// length is recorded, or its breakdown ends the solve (x and r untouched then).
+__device__ __forceinline__ void cg_fused_finish(SolveState* st, double gkg, double n, double rr,
+                                                double rz) {
+  cg_alpha_from(st, gkg, n);
+  if (!st->done) cg_step_finish(st, rr, rz);
+  else if (st->graph_mode) cudaGraphSetConditional(st->h_cur, 0u);
+}
+
+// Divergence pass and CG update of a plain FP64 iteration in one (fx64): A d
+// stays in the CTA, x += alpha d, r -= alpha A d, and the sums for beta.  Against
+// the two kernels it saves a launch, and writing and reading A d.
+__global__ void __launch_bounds__(cta_bound<fx64>(512)) k_col_div_upd(
+    Geo<fx64> g, const cx<fx64>* __restrict__ Qx, const cx<fx64>* __restrict__ Qy,
+    const cx<double>* __restrict__ d, cx<double>* __restrict__ x, cx<double>* __restrict__ r,
+    SolveState* st);
 
 // sum over one thread's spectral values of w |xi~|^2 (|v0|^2 + |v1|^2) (w the
 // Parseval weight of the packed column kx, xi~ the R1 derivative multipliers;

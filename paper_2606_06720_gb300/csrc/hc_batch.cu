@@ -218,7 +218,7 @@ void batch_cg_iter(const BInst* bi, const BShape& sh, cudaStream_t s) {
   else
     kb_cg_apply<1><<<row_grid(g, sh.nb), row_threads(g), sm, s>>>(bi);
   kb_cg_div<<<col_grid(g, sh.nb), col_threads(g), col_smem(g, 2), s>>>(bi);
-  kb_cg_update<<<dim3(upd_blocks((size_t)g.ny * g.H), sh.nb), 256, 0, s>>>(bi);
+  kb_cg_update<<<dim3(cg_blocks((size_t)g.ny * g.H), sh.nb), 256, 0, s>>>(bi);
 }
 
 void batch_mid_resid(const BInst* bi, const BShape& sh, cudaStream_t s) {

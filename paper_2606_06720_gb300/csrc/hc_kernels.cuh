@@ -435,13 +435,14 @@ __device__ __forceinline__ bool last_cta_sum(double (&v)[K], double* partials,
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < K; ++k) partials[blockIdx.x * kPartialStride + k] = v[k];
-    __threadfence();
-    unsigned int t = atomicAdd(ticket, 1u);
+    // the ticket releases this thread's partials and, in the last CTA, acquires
+    // the others' (the barrier passes that on to its threads)
+    unsigned int t;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
     s_last = (t == gridDim.x - 1) ? 1u : 0u;
   }
   __syncthreads();
   if (!s_last) return false;
-  __threadfence();
   // every thread of the last CTA sums a fixed strided subset of the partials,
   // then a fixed-order block reduction: deterministic for a given grid
   double w[K];
@@ -888,11 +889,16 @@ __device__ __forceinline__ void cg_alpha_from(SolveState* st, double gkg, double
 // Step length of an FP32 CG iteration from the row pass's per-CTA partials of
 // <d, A d> (cta_pair_partial): run by one CTA of the divergence pass that
 // follows it, which sums them in fixed order and calls cg_alpha_from.  The
-// update kernel after that pass reads alpha.
-__device__ __forceinline__ void cg_alpha_finish(const Geo<float>& g, SolveState* st) {
+// update kernel after that pass reads alpha.  Each thread loads its share before
+// the pass's transforms; the sum comes after them.
+__device__ __forceinline__ double cg_alpha_share(const Geo<float>& g) {
   const int np = g.rpipe ? g.rgrid : (g.ny >> g.lrpc);  // CTAs of the row pass
-  double a[1] = {0.0};
-  for (int i = threadIdx.x; i < np; i += blockDim.x) a[0] += g.partials[(size_t)i * kPartialStride];
+  double a = 0.0;
+  for (int i = threadIdx.x; i < np; i += blockDim.x) a += g.partials[(size_t)i * kPartialStride];
+  return a;
+}
+__device__ __forceinline__ void cg_alpha_finish(const Geo<float>& g, SolveState* st, double share) {
+  double a[1] = {share};
   block_sum<1>(a);
   if (threadIdx.x == 0) cg_alpha_from(st, a[0], (double)g.nx * (double)g.ny);
   __syncthreads();  // the block_sum scratch is reused by the caller
@@ -1609,8 +1615,9 @@ __device__ __forceinline__ void col_div_body(Geo<T> g, const cx<T>* __restrict__
                                                  cx<T>* __restrict__ out, cx<float>* __restrict__ r32,
                                                  cx<float>* __restrict__ delta32, SolveState* st) {
   if ((MODE == CD_CG || MODE == CD_CERT) && st->done) return;
+  double alpha_share = 0.0;
   if constexpr (MODE == CD_CG && std::is_same<T, float>::value)
-    if (blockIdx.x == 0) cg_alpha_finish(g, st);
+    if (blockIdx.x == 0) alpha_share = cg_alpha_share(g);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
   const ColIdx c = col_idx(g);
@@ -1715,6 +1722,8 @@ __device__ __forceinline__ void col_div_body(Geo<T> g, const cx<T>* __restrict__
       rzacc.add_prod(wpf * rf.y, rf.y);
     }
   }
+  if constexpr (MODE == CD_CG && std::is_same<T, float>::value)
+    if (blockIdx.x == 0) cg_alpha_finish(g, st, alpha_share);
   if constexpr (MODE == CD_PLAIN || MODE == CD_CG) return;
   double tot[3];
   if constexpr (MODE == CD_DECIDE) {
@@ -2085,7 +2094,7 @@ __global__ void __launch_bounds__(512) kp_col_div(Geo<T> g, const cx<T>* __restr
                                                   cx<float>* __restrict__ delta32, SolveState* st) {
   if (MODE == CD_CG && st->done) return;
   if constexpr (MODE == CD_CG && std::is_same<T, float>::value)
-    if (blockIdx.x == 0) cg_alpha_finish(g, st);
+    if (blockIdx.x == 0) cg_alpha_finish(g, st, cg_alpha_share(g));
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
   const int H = g.H, se = slab_elems(g), ntiles = g.H >> g.ltc;
@@ -2664,6 +2673,13 @@ static inline int upd_blocks(size_t total) {
   return (int)(b < 608 ? b : 608);  // 4 CTAs of 256 threads per SM on 152 SMs
 }
 
+// CTAs of the CG update: four values a thread, so that a small grid's sums meet
+// over few tickets (512^2: 10.0 us in 512 CTAs of one value a thread).
+static inline int cg_blocks(size_t total) {
+  const size_t b = (total + 1023) / 1024;
+  return (int)(b < 608 ? b : 608);
+}
+
 template <typename T>
 void row_r2c(const Geo<T>& g, const T* a, const T* b, cx<T>* A, cx<T>* B, cudaStream_t s) {
   if constexpr (std::is_same<T, double>::value)
@@ -2874,7 +2890,7 @@ void col_gradnorm(const Geo<T>& g0, const cx<T>* Mx, const cx<T>* My, SolveState
 template <typename T>
 void cg_update(const Geo<T>& g, cx<T>* x, cx<T>* r, const cx<T>* d, const cx<T>* q, SolveState* st,
                cudaStream_t s) {
-  k_cg_update<T><<<upd_blocks((size_t)g.ny * g.H), 256, 0, s>>>(g, x, r, d, q, st);
+  k_cg_update<T><<<cg_blocks((size_t)g.ny * g.H), 256, 0, s>>>(g, x, r, d, q, st);
 }
 template <typename Ti>
 void to_cm(const Geo<float>& g, const cx<Ti>* in, cx<float>* out, cudaStream_t s) {

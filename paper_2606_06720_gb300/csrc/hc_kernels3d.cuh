@@ -957,7 +957,7 @@ void z_gradnorm(const Geo<T>& g, Tri<cx<T>*> G, SolveState* st, int into_next, c
 template <typename T>
 void cg_update3(const Geo<T>& g, cx<T>* x, cx<T>* r, const cx<T>* d, const cx<T>* q,
                 SolveState* st, cudaStream_t s) {
-  k3_cg_update<T><<<upd_blocks((size_t)g.nz * g.ny * g.H), 256, 0, s>>>(g, x, r, d, q, st);
+  k3_cg_update<T><<<cg_blocks((size_t)g.nz * g.ny * g.H), 256, 0, s>>>(g, x, r, d, q, st);
 }
 template <typename T>
 void msum3(const Geo<T>& g, Tri<const T*> m, SolveState* st, cudaStream_t s) {

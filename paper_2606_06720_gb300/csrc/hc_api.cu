@@ -146,7 +146,7 @@ struct hc_ctx {
   cx<double>* d64;          // CG direction (plain mode)
   cx<double>* q64;          // A d (plain mode, 3D and component calls)
   double* pinv64;           // plain mode, 2D: the running step's preconditioner symbol
-  double* dots;             // plain mode, 2D: the row pass's per-CTA sums of <d, A d>
+  double* dots;             // 2D: per-CTA sums of <d, A d> (plain mode, loop kernels)
   cx<double>* G64;          // dim spectra: gradient / flux / m scratch (FP64)
   cx<float>* b32;           // refined: FP32 copy of the projected source spectrum
   cx<df64>* bq;             // HC_FP32_REFINED: double-float copy of it (mid-step residual)
@@ -213,6 +213,7 @@ struct hc_ctx {
   cudaStream_t cap_hi, cap_lo;          // capture streams of the lagged graph's two branches
   cudaStream_t io_stream;               // hc_set_state / hc_get_state: copies beside p's transform
   cudaEvent_t io_ev[2 + 4];             // entry, copies done, and one per row chunk of p
+  int loop_nt;  // CTA size of the CG loop kernel, 0: an iteration's kernels apart
   int graph_nodes_fixed, graph_nodes_body, graph_nodes_outer;
 };
 
@@ -347,13 +348,12 @@ void layout(hc_ctx* c, Layout& L) {
   c->b64 = L.take<cx<double>>(S64);
   c->r64 = L.take<cx<double>>(S64);
   c->G64 = L.take<cx<double>>(d * S64);
+  // row CTAs of an iteration, or CTAs of the loop kernel
+  if (d == 2) c->dots = L.take<double>(sizeof(double) * std::max(c->ny, 128));
   if (!c->refined) {
     c->d64 = L.take<cx<double>>(S64);
     c->q64 = L.take<cx<double>>(S64);
-    if (d == 2) {
-      c->pinv64 = L.take<double>(sizeof(double) * c->ns);
-      c->dots = L.take<double>(sizeof(double) * c->ny);
-    }
+    if (d == 2) c->pinv64 = L.take<double>(sizeof(double) * c->ns);
     c->b32 = c->r32 = c->d32 = c->q32 = c->x32 = c->G32 = nullptr;
     c->bq = nullptr;
     for (int k = 0; k < d; ++k) c->m[k] = L.take<double>(sizeof(double) * n);
@@ -1239,11 +1239,25 @@ void split_step(hc_ctx* c) {
 int read_state(hc_ctx* c) {
   CU(cudaMemcpyAsync(c->st_host, c->st, sizeof(hc::SolveState), cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
-  return HC_OK;
+  return c->st_host->loop_timeout ? HC_ETIMEOUT : HC_OK;
+}
+
+// The whole CG loop of an inner solve in one launch (loop_nt > 0).
+void refined_loop(hc_ctx* c) {
+  hc::cg_loop_f32(c->gf, c->loop_nt, c->x32, c->r32, c->G32, c->G32 + (size_t)c->ny * c->H,
+                  (const float*)c->m[0], (const float*)c->m[1], (const float*)c->rf, c->st, c->stream);
 }
 
 // Launch CG iterations in chunks until the device says done.
 int run_cg_host(hc_ctx* c, bool refined_inner) {
+  if (c->loop_nt) {
+    refined_loop(c);
+    CU(cudaGetLastError());
+    int rc = read_state(c);
+    if (rc) return rc;
+    c->launches += (long long)c->graph_nodes_body * c->st_host->it;
+    return HC_OK;
+  }
   for (int guard = 0; guard < 1000000; guard += kChunk) {
     for (int k = 0; k < kChunk; ++k) {
       if (refined_inner)
@@ -1354,7 +1368,9 @@ int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h) {
   auto capture_iter = [&](cudaGraph_t body) -> int {
     CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0,
                                      cudaStreamCaptureModeThreadLocal));
-    if (c->refined)
+    if (c->loop_nt)
+      refined_loop(c);
+    else if (c->refined)
       refined_iter(c);
     else
       plain_iter(c);
@@ -1664,7 +1680,10 @@ int build_pipe_graph(hc_ctx* c) {
     };
     auto capture_iter = [&](cudaGraph_t body) -> int {
       CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-      refined_iter(c);
+      if (c->loop_nt)
+        refined_loop(c);
+      else
+        refined_iter(c);
       return end_capture(s, body, nullptr);
     };
     // gate, IF(not halted)
@@ -1979,7 +1998,7 @@ int hc_create(hc_ctx** out, const hc_grid* grid, const hc_params* params, void* 
     c->gq.tc = c->gd.tc;
     c->gq.ltc = c->gd.ltc;
     c->gd.fx = c->refined ? 0 : 1;
-    c->gd.dots = c->dots;
+    c->gd.dots = c->gf.dots = c->dots;
     c->gd.pinv = c->pinv64;
     c->gd.qx = c->twx_x;
     c->gd.qy = c->twy_x;
@@ -1988,6 +2007,10 @@ int hc_create(hc_ctx** out, const hc_grid* grid, const hc_params* params, void* 
       fill_geo3<float>(c, c->gf, c->rowf, c->twz_f, c->kzd_f, c->hz_f);
       fill_geo3<double>(c, c->gd, c->rowd, c->twz_d, c->kzd_d, c->hz_d);
       fill_geo3<df64>(c, c->gq, c->rowq, c->twz_q, c->kzd_q, nullptr);
+    }
+    if (c->dim == 2 && c->refined) {
+      const int nt = hc::cg_loop_threads(c->nx, c->ny);
+      if (nt && hc::cg_loop_fits_f32(c->nx, c->ny, nt)) c->loop_nt = nt;
     }
     hc::set_smem_limits_fx(c->refined);
     if (c->dim == 3) hc::set_smem_limits_3d_fx(c->refined);
@@ -3375,6 +3398,7 @@ int hc_batch_step(hc_batch* b, int nsteps, hc_step_stats* stats) {
     if (b->cls_of[i] < 0) c->launches += graph_kernel_count(c, h);
     if (stats) fill_stats(c, &stats[i]);
     if (!first_bad && h.first_bad) first_bad = h.first_bad;
+    if (h.loop_timeout) first_bad = HC_ETIMEOUT;
     int rc = set_graph_mode(c, 0);
     if (rc) return rc;
   }

@@ -1,0 +1,352 @@
+// hc_cgloop.cu -- the CG loop of a 2D solve as one cooperative kernel.
+//
+// On grids up to about 10^6 points an iteration's launches (three or four kernels and the
+// loop node's turn) cost as much as their work: at 512^2 an iteration took 40 us, of which
+// the kernels ran 29, each of them mostly the latency of its start, its loads and its last
+// CTA's sums.  Here one launch runs the whole loop.  Every CTA keeps the same column tile
+// and the same rows throughout, so x, r and d never leave it (registers and shared memory),
+// m and r of the coefficient are staged once, and only the transposed fields Gx, Gy and
+// three sums an iteration pass between CTAs, across three grid barriers.  Each CTA forms
+// alpha, beta and the stop test from the CTAs' partial sums, all in the same order, so all
+// leave the loop together and none waits for a last CTA.
+#include "hc_kernels.cuh"
+
+namespace hc {
+
+// Polls of a grid barrier before it gives up, about a second.
+constexpr unsigned kBarrierPolls = 1u << 20;
+
+// Grid barrier number `target / gridDim.x`.  The launch is cooperative, so every CTA is
+// resident and arrives.  False in every thread of a CTA whose wait ran out.  What any CTA
+// wrote before it is visible to every thread after it.
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    int ok = 0;
+    for (unsigned i = 0; i < kBarrierPolls; ++i) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (v >= target) {
+        ok = 1;
+        break;
+      }
+    }
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// The scalars of a solve, kept by every thread alike.
+struct LoopCg {
+  double rho, rnorm2, alpha, beta;
+  int it, done, status;
+};
+
+// After the row pass: the step length, as cg_alpha_from.
+__device__ __forceinline__ bool loop_alpha(LoopCg& k, double gkg, double n, int refined,
+                                           double thresh2) {
+  const double dq = gkg * n;
+  if (dq > 0 && isfinite(dq)) {
+    k.alpha = k.rho / dq;
+    return true;
+  }
+  k.alpha = 0.0;
+  k.done = 1;
+  if (!isfinite(dq)) k.status = HC_ENONFINITE;
+  else if (!refined && k.rnorm2 > thresh2) k.status = HC_ENOCONV;
+  return false;
+}
+// After the update: beta and the stop test, as cg_step_finish.
+__device__ __forceinline__ void loop_beta(LoopCg& k, double rr, double rz, double thresh2,
+                                          int maxit) {
+  k.rnorm2 = rr;
+  k.beta = k.rho > 0 ? rz / k.rho : 0.0;
+  k.rho = rz;
+  k.it += 1;
+  if (!isfinite(rr)) {
+    k.status = HC_ENONFINITE;
+    k.done = 1;
+  } else if (rr <= thresh2) {
+    k.done = 1;
+  } else if (k.it >= maxit) {
+    k.done = 1;
+    k.status = HC_ENOCONV;
+  }
+}
+// The end of the loop, one thread of the grid: the solve state as the kernels of an
+// iteration would have left it.
+__device__ __forceinline__ void loop_finish(SolveState* st, const LoopCg& k, int its, bool timeout) {
+  st->rnorm2 = k.rnorm2;
+  st->alpha = k.alpha;
+  st->alpha_f = (float)k.alpha;
+  st->beta = k.beta;
+  st->beta_f = (float)k.beta;
+  st->rho = k.rho;
+  st->it = k.it;
+  st->total_it += its;
+  if (k.status) st->status = k.status;
+  if (timeout) st->loop_timeout = 1;
+  st->first = 0;
+  st->done = 1;
+  predict_residual(st);
+  if (st->graph_mode) cudaGraphSetConditional(st->h_cur, 0u);
+}
+// The last CTA to leave re-arms the barrier.
+__device__ __forceinline__ void loop_leave(SolveState* st) {
+  if (threadIdx.x == 0) {
+    unsigned t;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(&st->loop_exit) : "memory");
+    if (t == gridDim.x - 1) {
+      st->loop_exit = 0u;
+      st->loop_bar = 0u;
+    }
+  }
+}
+
+// Sum over the CTAs of K values (K doubles each at p[cta * stride]), in every thread.
+template <int K>
+__device__ __forceinline__ void grid_total(const double* p, int stride, double (&tot)[K]) {
+  __shared__ double s_tot[K];
+  double w[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) w[k] = 0.0;
+  for (unsigned c = threadIdx.x; c < gridDim.x; c += blockDim.x)
+#pragma unroll
+    for (int k = 0; k < K; ++k) w[k] += __ldcg(&p[c * stride + k]);
+  block_sum<K>(w);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int k = 0; k < K; ++k) s_tot[k] = w[k];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < K; ++k) tot[k] = s_tot[k];
+}
+
+// FP32 inner solve (x, r column-major).  g's tile (tc, rpc) is the loop's: blockDim.x threads
+// carry two fields of 8 values of a column, or 8 values of two rows.  The arithmetic is the
+// separate kernels' to the bit, roundings written out; only the order of the sums differs.
+// row_sums: a row's share of <d, A d> is summed by itself, as where those kernels put one row
+// on a thread.
+// MAXT: 512 threads at 128 registers (some spills), or 256 without.
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>* x,
+                                                        const cx<float>* r, cx<float>* Gx,
+                                                        cx<float>* Gy, const float* mx,
+                                                        const float* my, const float* rf,
+                                                        SolveState* st, int row_sums) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (st->done) return;  // nothing writes it before every CTA has passed a barrier
+  using C = cx<float>;
+  C* sm = reinterpret_cast<C*>(smem_raw);
+  const int nt = blockDim.x, t = threadIdx.x, H = g.H;
+  const ColIdx c = col_idx(g);
+  const int se = slab_elems(g);
+  C* const csl[2] = {sm + c.b, sm + se + c.b};
+  // rows
+  const int l8 = g.lnx - 3, N = g.nx, N8 = 1 << l8;
+  const int rj = t & (N8 - 1), r0 = (t >> l8) * 2, y0 = (blockIdx.x << g.lrpc) + r0;
+  C* const rsl[2] = {sm + (size_t)r0 * N, sm + (size_t)(r0 + 1) * N};
+  C* const Ra[2] = {Gx + (size_t)y0 * H, Gx + (size_t)(y0 + 1) * H};
+  C* const Rb[2] = {Gy + (size_t)y0 * H, Gy + (size_t)(y0 + 1) * H};
+  // behind the slabs: this CTA's rows of mx, my, r, then x (slot s of thread t at s nt + t)
+  float* sf = reinterpret_cast<float*>(sm + 18 * nt);
+  C* xs = reinterpret_cast<C*>(sf + 3 * (size_t)g.rpc * N) + t;
+  {
+    const size_t row0 = ((size_t)blockIdx.x << g.lrpc) * N;
+    const int per = (int)(((size_t)g.rpc * N * sizeof(float)) >> 4);
+    const float* const src[3] = {mx + row0, my + row0, rf + row0};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      char* dst = reinterpret_cast<char*>(sf + (size_t)q * g.rpc * N);
+      const char* from = reinterpret_cast<const char*>(src[q]);
+      for (int i = t; i < per; i += nt) cp_async16(dst + 16 * i, from + 16 * i);
+    }
+    cp_async_commit();
+  }
+  const double n = (double)g.nx * (double)g.ny, thresh2 = st->thresh2;
+  const int maxit = st->maxit;
+  const Pc<float> pc = pc_of<float>(st);
+  LoopCg k{st->rho, st->rnorm2, 0.0, 0.0, st->it, 0, 0};
+  const int it0 = k.it;
+  unsigned* const bar = &st->loop_bar;
+  unsigned target = 0;
+  const float invn = exp2_neg<float>(g.lnx + g.lny), kx = g.kxd[c.kx];
+  const float ax = kx * invn;
+  const float wt = c.kx == 0 ? 1.0f : 2.0f;  // Parseval weight of a packed column
+  float pv[8];  // the preconditioner symbol
+  C rv[8], dv[8];
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {
+    const int ky = c.j + s * c.NY8;
+    const float b = g.kyd[ky];
+    const float xa = __fmul_rn(pc.xx, kx), xb = __fmul_rn(__fmul_rn(2.0f, pc.xy), kx);
+    const float yb = __fmul_rn(pc.yy, b);
+    const float s2 = __fmaf_rn(yb, b, __fmaf_rn(xa, kx, __fmul_rn(xb, b)));
+    pv[s] = s2 > 0.0f ? 1.0f / s2 : 0.0f;
+    const size_t i = cmi(g, ky, c.kx);
+    rv[s] = r[i];
+    dv[s] = czero<float>();
+    xs[(size_t)s * nt] = x[i];
+  }
+  cp_async_wait_all();
+  bool live = true;  // no wait has run out
+  while (true) {
+    // gradient of d = M^-1 r + beta d
+    const bool first = k.it == it0;
+    const float beta = (float)k.beta;
+    C v[2][8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const C z = cmk<float>(__fmul_rn(rv[s].x, pv[s]), __fmul_rn(rv[s].y, pv[s]));
+      const C P = first ? z : cmk<float>(__fmaf_rn(dv[s].x, beta, z.x), __fmaf_rn(dv[s].y, beta, z.y));
+      dv[s] = P;
+      const float ay = g.kyd[c.j + s * c.NY8] * invn;
+      v[0][s] = cmk<float>(__fmul_rn(-ax, P.y), __fmul_rn(ax, P.x));
+      v[1][s] = cmk<float>(__fmul_rn(-ay, P.y), __fmul_rn(ay, P.x));
+    }
+    fft_canon<+1, 2>(v, csl, g.tc, c.j, g.lny, g.twy);
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const size_t idx = (size_t)(c.j + s * c.NY8) * H + c.kx;
+      Gx[idx] = v[0][s];
+      Gy[idx] = v[1][s];
+    }
+    live = grid_barrier(bar, target += gridDim.x);
+    if (!live) break;
+    // (m m + r I) grad d along the rows, in place
+    load_rows_c2r<2>(v, (const C* const*)Ra, (const C* const*)Rb, rj, N8);
+    fft_canon<+1, 2, true>(v, rsl, 1, rj, g.lnx, g.twx);
+    float gk = 0.0f, gk0 = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float* smx = sf + (size_t)(r0 + q) * N;
+      const float* smy = smx + (size_t)g.rpc * N;
+      const float* srr = smy + (size_t)g.rpc * N;
+      if (q == 1 && row_sums) {
+        gk0 = gk;
+        gk = 0.0f;
+      }
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const int xp = rj + s * N8;
+        const float gx = v[q][s].x, gy = v[q][s].y;
+        const float a = smx[xp], b = smy[xp], rr = srr[xp];
+        const float mg = __fmaf_rn(a, gx, __fmul_rn(b, gy));
+        const float g2 = __fmaf_rn(gx, gx, __fmul_rn(gy, gy));
+        gk = __fadd_rn(gk, __fmaf_rn(rr, g2, __fmul_rn(mg, mg)));
+        v[q][s] = cmk<float>(__fmaf_rn(rr, gx, __fmul_rn(a, mg)), __fmaf_rn(rr, gy, __fmul_rn(b, mg)));
+      }
+    }
+    fft_rows_r2c<2>(v, rsl, rj, g.lnx, g.twx, Ra, Rb);
+    {
+      float h[1] = {gk}, l[1] = {0.0f};
+      pair_add(h[0], l[0], gk0, 0.0f);
+      double p[1];
+      cta_pair_sums<1>(h, l, p);
+      if (t == 0) g.dots[blockIdx.x] = p[0];
+    }
+    live = grid_barrier(bar, target += gridDim.x);
+    if (!live) break;
+    // A d = -div; x += alpha d, r -= alpha A d
+    const double share = t < (int)gridDim.x ? __ldcg(&g.dots[t]) : 0.0;
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const size_t idx = (size_t)(c.j + s * c.NY8) * H + c.kx;
+      v[0][s] = Gx[idx];
+      v[1][s] = Gy[idx];
+    }
+    fft_canon<-1, 2>(v, csl, g.tc, c.j, g.lny, g.twy);
+    double w = share;
+    for (int i = t + nt; i < (int)gridDim.x; i += nt) w += __ldcg(&g.dots[i]);
+    const double gkg = dots_total(w);
+    if (!loop_alpha(k, gkg, n, 1, thresh2)) break;
+    const float alpha = (float)k.alpha;
+    DotAcc<float> rr, rz;
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const float ay = g.kyd[c.j + s * c.NY8];
+      const C q = cmk<float>(__fmaf_rn(kx, v[0][s].y, __fmul_rn(ay, v[1][s].y)),
+                             -__fmaf_rn(kx, v[0][s].x, __fmul_rn(ay, v[1][s].x)));
+      const C xv = xs[(size_t)s * nt];
+      xs[(size_t)s * nt] = cmk<float>(__fmaf_rn(alpha, dv[s].x, xv.x), __fmaf_rn(alpha, dv[s].y, xv.y));
+      rv[s] = cmk<float>(__fmaf_rn(-alpha, q.x, rv[s].x), __fmaf_rn(-alpha, q.y, rv[s].y));
+      rr.add_prod(wt * rv[s].x, rv[s].x);
+      rr.add_prod(wt * rv[s].y, rv[s].y);
+      const float wp = wt * pv[s];
+      rz.add_prod(wp * rv[s].x, rv[s].x);
+      rz.add_prod(wp * rv[s].y, rv[s].y);
+    }
+    {
+      float h[2] = {rr.hi, rz.hi}, l[2] = {rr.lo, rz.lo};
+      double p[2];
+      cta_pair_sums<2>(h, l, p);
+      if (t == 0) {
+        g.partials[(size_t)blockIdx.x * kPartialStride] = p[0];
+        g.partials[(size_t)blockIdx.x * kPartialStride + 1] = p[1];
+      }
+    }
+    live = grid_barrier(bar, target += gridDim.x);
+    if (!live) break;
+    double tot[2];
+    grid_total<2>(g.partials, kPartialStride, tot);
+    loop_beta(k, tot[0], tot[1], thresh2, maxit);
+    if (k.done) break;
+  }
+  if (live) {
+#pragma unroll
+    for (int s = 0; s < 8; ++s) x[cmi(g, c.j + s * c.NY8, c.kx)] = xs[(size_t)s * nt];
+  }
+  if (blockIdx.x == 0 && t == 0) loop_finish(st, k, k.it - it0, !live);
+  loop_leave(st);
+}
+
+static inline size_t loop_smem(int nt, int rpc, int nx) {
+  return (size_t)18 * nt * sizeof(cx<float>) + (size_t)3 * rpc * nx * sizeof(float) +
+         (size_t)8 * nt * sizeof(cx<float>);
+}
+
+// Threads of a CTA: 16 values each in either pass, enough of them for a column and for two
+// rows, at most 128 CTAs, so that all are resident at one a SM.
+int cg_loop_threads(int nx, int ny) {
+  const long long n = (long long)nx * ny;
+  int nt = 32;
+  while (nt < ny / 8 || nt < nx / 8 || n / (16 * nt) > 128) nt *= 2;
+  if (nt > 512 || n < 16 * nt) return 0;
+  if (8 * nt / ny > 32 || 8 * nt / ny > nx / 2) return 0;
+  return nt;
+}
+
+bool cg_loop_fits_f32(int nx, int ny, int nt) {
+  const int grid = (int)((long long)nx * ny / (16 * nt)), rpc = 16 * nt / nx;
+  const auto kernel = nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>;
+  allow_smem(kernel);
+  int dev = 0, sms = 0, coop = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, nt, loop_smem(nt, rpc, nx)) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return coop && (long long)per * sms >= grid;
+}
+
+void cg_loop_f32(const Geo<float>& g0, int nt, cx<float>* x, const cx<float>* r, cx<float>* Gx,
+                 cx<float>* Gy, const float* mx, const float* my, const float* rf, SolveState* st,
+                 cudaStream_t s) {
+  Geo<float> g = g0;
+  int row_sums = g0.rpc < 2;
+  g.tc = 8 * nt / g.ny;
+  g.rpc = 16 * nt / g.nx;
+  for (g.ltc = 0; (1 << g.ltc) < g.tc;) ++g.ltc;
+  for (g.lrpc = 0; (1 << g.lrpc) < g.rpc;) ++g.lrpc;
+  void* args[] = {&g, &x, &r, &Gx, &Gy, &mx, &my, &rf, &st, &row_sums};
+  cudaLaunchCooperativeKernel((const void*)(nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>), dim3(g.H >> g.ltc), dim3(nt), args,
+                              loop_smem(nt, g.rpc, g.nx), s);
+}
+
+}  // namespace hc

@@ -201,6 +201,9 @@ struct SolveState {
   int delta_added;           // the fx64 residual has added the pending correction to p64
   int acc_again;             // fx64 residuals that missed, summed over the steps since the last reset
   unsigned int ticket[8];    // last-CTA tickets, one per reduction site
+  unsigned int loop_bar;     // CG loop kernel: arrivals at its grid barriers (0 between launches)
+  unsigned int loop_exit;    // CTAs that have left it
+  int loop_timeout;          // a barrier's bounded wait ran out (sticky)
   // Diagnostics of Section 2.5, accumulated by the split step when diag != 0.
   // A step solves p[m^k] and so evaluates E_h(m^k) with its own pressure.
   double dsum[3];            // running step: sum r|g|^2, sum (m.g)^2, sum |m|^(2 gamma) (gamma = 0: sum ln|m|); m = m^k, g = grad p[m^k]
@@ -292,7 +295,7 @@ struct Geo {
   int pipe;                  // 1: column passes run persistent with cp.async double buffering
   int pgrid;                 // CTAs of a persistent column pass (<= SMs, <= tiles)
   int fx;                    // Geo<double>: launch the fx64 kernels (as_fx)
-  double* dots;              // plain FP64 CG: the row pass's per-CTA sums of <d, A d>
+  double* dots;              // the row pass's per-CTA sums of <d, A d> (plain FP64 CG, the loop kernels)
   double* pinv;              // plain FP64 CG: the running step's preconditioner symbol, as the spectra
   const FxTw* qx;            // Geo<double>: twiddle tables of the fx64 kernels
   const FxTw* qy;
@@ -598,6 +601,14 @@ void pinv_table(const Geo<double>& g, const SolveState* st, cudaStream_t s);
 void col_div_upd(const Geo<double>& g, const cx<double>* Qx, const cx<double>* Qy, const cx<double>* d,
                  cx<double>* x, cx<double>* r, SolveState* st, cudaStream_t s);
 void set_smem_limits_fx(int refined);
+// The CG loop of a 2D solve as one cooperative kernel (hc_cgloop.cu).  cg_loop_threads: its
+// CTA size for a grid, 0 where the separate kernels are the better ones; ..._fits: this device
+// keeps all its CTAs resident.
+int cg_loop_threads(int nx, int ny);
+bool cg_loop_fits_f32(int nx, int ny, int nt);
+void cg_loop_f32(const Geo<float>& g, int nt, cx<float>* x, const cx<float>* r, cx<float>* Gx,
+                 cx<float>* Gy, const float* mx, const float* my, const float* rf, SolveState* st,
+                 cudaStream_t s);
 // Lagged certification (2D refined steps): the FP64 certifying residual of
 // pressure p with the FP32 m, r it was solved with (sc: the certifying state,
 // skipped when nothing is pending); the commit after a lagged step (copies

@@ -335,7 +335,9 @@ enum {
 int hc_time_kernel(hc_ctx* ctx, int kernel, int reps, double* ms_per_launch);
 
 /* Number of this library's kernel launches issued by the context so far
- * (graph launches count every kernel node). */
+ * (graph launches count every kernel node).  Where the CG loop runs as one
+ * kernel (2D, up to about 10^6 points) its iterations still count as the
+ * kernels that each stands for, so that counts compare between grids. */
 int hc_launch_count(const hc_ctx* ctx, long long* count);
 
 /* Measured FP64 FMA throughput of the current device in TFLOP/s (an FMA counts

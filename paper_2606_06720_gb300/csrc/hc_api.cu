@@ -1242,16 +1242,20 @@ int read_state(hc_ctx* c) {
   return c->st_host->loop_timeout ? HC_ETIMEOUT : HC_OK;
 }
 
-// The whole CG loop of an inner solve in one launch (loop_nt > 0).
-void refined_loop(hc_ctx* c) {
-  hc::cg_loop_f32(c->gf, c->loop_nt, c->x32, c->r32, c->G32, c->G32 + (size_t)c->ny * c->H,
-                  (const float*)c->m[0], (const float*)c->m[1], (const float*)c->rf, c->st, c->stream);
+// The whole CG loop of a solve in one launch (loop_nt > 0).
+void cg_loop(hc_ctx* c) {
+  if (c->refined)
+    hc::cg_loop_f32(c->gf, c->loop_nt, c->x32, c->r32, c->G32, c->G32 + c->ns, (const float*)c->m[0],
+                    (const float*)c->m[1], (const float*)c->rf, c->st, c->stream);
+  else
+    hc::cg_loop_fx(c->gd, c->loop_nt, c->p64, c->r64, c->G64, c->G64 + c->ns, (const double*)c->m[0],
+                   (const double*)c->m[1], (const double*)c->rf, c->st, c->stream);
 }
 
 // Launch CG iterations in chunks until the device says done.
 int run_cg_host(hc_ctx* c, bool refined_inner) {
   if (c->loop_nt) {
-    refined_loop(c);
+    cg_loop(c);
     CU(cudaGetLastError());
     int rc = read_state(c);
     if (rc) return rc;
@@ -1369,7 +1373,7 @@ int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h) {
     CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0,
                                      cudaStreamCaptureModeThreadLocal));
     if (c->loop_nt)
-      refined_loop(c);
+      cg_loop(c);
     else if (c->refined)
       refined_iter(c);
     else
@@ -1681,7 +1685,7 @@ int build_pipe_graph(hc_ctx* c) {
     auto capture_iter = [&](cudaGraph_t body) -> int {
       CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
       if (c->loop_nt)
-        refined_loop(c);
+        cg_loop(c);
       else
         refined_iter(c);
       return end_capture(s, body, nullptr);
@@ -2008,10 +2012,8 @@ int hc_create(hc_ctx** out, const hc_grid* grid, const hc_params* params, void* 
       fill_geo3<double>(c, c->gd, c->rowd, c->twz_d, c->kzd_d, c->hz_d);
       fill_geo3<df64>(c, c->gq, c->rowq, c->twz_q, c->kzd_q, nullptr);
     }
-    if (c->dim == 2 && c->refined) {
-      const int nt = hc::cg_loop_threads(c->nx, c->ny);
-      if (nt && hc::cg_loop_fits_f32(c->nx, c->ny, nt)) c->loop_nt = nt;
-    }
+    if (c->dim == 2)
+      c->loop_nt = c->refined ? hc::cg_loop_threads_f32(c->nx, c->ny) : hc::cg_loop_threads_fx(c->nx, c->ny);
     hc::set_smem_limits_fx(c->refined);
     if (c->dim == 3) hc::set_smem_limits_3d_fx(c->refined);
     if (c->refined) {  // a plain FP64 context runs the fx64 kernels alone

@@ -9,6 +9,12 @@
 // three sums an iteration pass between CTAs, across three grid barriers.  Each CTA forms
 // alpha, beta and the stop test from the CTAs' partial sums, all in the same order, so all
 // leave the loop together and none waits for a last CTA.
+//
+// Measured (us an iteration, separate kernels -> loop; several hundred iterations): FP32 512^2
+// 40 -> 20; FP64 32^2 60 -> 40, 64^2 58 -> 33, 256^2 76 -> 43, 512^2 82 -> 62, 1024x512 (512
+// threads at 128 registers) 108 -> 108, so FP64 stops at 256 threads.  What is left: FP32, the
+// three barriers and the L2 latency of Gx and Gy around them; FP64, a warp's own instructions.
+// Beyond 512 threads a CTA (2^20 points) x, r and d no longer fit on the chip.
 #include "hc_kernels.cuh"
 
 namespace hc {
@@ -303,50 +309,278 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
   loop_leave(st);
 }
 
+// Plain FP64 solve (fx64 transforms, row-major x and r).  A warp's instructions are what
+// bounds a small grid here (64^2: one warp on each of 16 SMs, 8400 instructions an iteration),
+// a third of their time the fetch of code that a lone warp runs through once.  So a thread
+// carries one transform of 8 values at a time, and the iteration's four transforms are four
+// turns of a loop around one copy of the code: forward ones all, an inverse one with real and
+// imaginary parts exchanged before and after.  The two halves of the CTA take the two fields
+// of the same columns, and share out the columns' values for everything else (half h owns
+// slots 4 h .. 4 h + 3), which cross between them through ex.
+__global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* x,
+                                                        const cx<double>* r, cx<fx64>* Gx,
+                                                        cx<fx64>* Gy, const fx64* mx,
+                                                        const fx64* my, const fx64* rf,
+                                                        SolveState* st) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (st->done) return;  // nothing writes it before every CTA has passed a barrier
+  using C = cx<fx64>;
+  C* sm = reinterpret_cast<C*>(smem_raw);
+  const int nt = blockDim.x, hn = nt >> 1, t = threadIdx.x, H = g.H;
+  const int f = t >= hn ? 1 : 0, u = t - f * hn;  // field, thread within the half
+  const int b = u & (g.tc - 1), j = u >> g.ltc, col = (blockIdx.x << g.ltc) + b;
+  const int NY8 = 1 << (g.lny - 3), se = slab_elems(g);
+  C* const cslab = sm + f * se + b;
+  C* const G = f == 0 ? Gx : Gy;
+  const int l8 = g.lnx - 3, N = g.nx, N8 = 1 << l8;
+  const int rj = t & (N8 - 1), r0 = t >> l8;
+  const size_t y0 = ((size_t)blockIdx.x << g.lrpc) + r0;
+  C* const rslab = sm + (size_t)r0 * (N + N8);
+  C* const Ra[1] = {Gx + y0 * H};
+  C* const Rb[1] = {Gy + y0 * H};
+  // behind the slabs (9 nt values): ex (slot s of thread u at s hn + u), then this CTA's rows
+  // of mx, my, r
+  C* const ex = sm + 9 * nt + u;
+  fx64* sf = reinterpret_cast<fx64*>(sm + 13 * nt);
+  {
+    const size_t row0 = ((size_t)blockIdx.x << g.lrpc) * N;
+    const int per = (int)(((size_t)g.rpc * N * sizeof(fx64)) >> 4);
+    const fx64* const src[3] = {mx + row0, my + row0, rf + row0};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      char* dst = reinterpret_cast<char*>(sf + (size_t)q * g.rpc * N);
+      const char* from = reinterpret_cast<const char*>(src[q]);
+      for (int i = t; i < per; i += nt) cp_async16(dst + 16 * i, from + 16 * i);
+    }
+    cp_async_commit();
+  }
+  const double n = (double)g.nx * (double)g.ny, invn = 1.0 / n, thresh2 = st->thresh2;
+  const int maxit = st->maxit;
+  LoopCg k{st->rho, st->rnorm2, 0.0, 0.0, st->it, 0, 0};
+  const int it0 = k.it;
+  unsigned* const bar = &st->loop_bar;
+  unsigned target = 0;
+  const double kx = g.kxd[col].v;
+  const double w = col == 0 ? 1.0 : 2.0;  // Parseval weight of a packed column
+  cx<double> xv[4], rv[4], dv[4];
+  double pv[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const size_t e = (size_t)(j + (4 * f + i) * NY8) * H + col;
+    xv[i] = x[e];
+    rv[i] = r[e];
+    dv[i] = cmk<double>(0.0, 0.0);
+    pv[i] = g.pinv[e];
+  }
+  cp_async_wait_all();
+  bool live = true;  // no wait has run out
+  C v[1][8];
+  int phase = 0;  // columns inverse, rows inverse, rows forward, columns forward
+#pragma unroll 1
+  while (true) {
+    if (phase == 0) {
+      // gradient of d = M^-1 r + beta d
+      const bool first = k.it == it0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const cx<double> z = cmk<double>(rv[i].x * pv[i], rv[i].y * pv[i]);
+        dv[i] = first ? z : cmk<double>(z.x + k.beta * dv[i].x, z.y + k.beta * dv[i].y);
+        ex[(4 * f + i) * hn] = cmk<fx64>(dv[i].x, dv[i].y);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const C P = ex[s * hn];
+        const fx64 a = (f == 0 ? kx : g.kyd[j + s * NY8].v) * invn;
+        v[0][s] = cmk<fx64>(a * P.x, -a * P.y);  // i (k/n) P, exchanged
+      }
+    } else if (phase == 1) {
+      load_rows_c2r<1>(v, (const C* const*)Ra, (const C* const*)Rb, rj, N8);
+#pragma unroll
+      for (int s = 0; s < 8; ++s) v[0][s] = cmk<fx64>(v[0][s].y, v[0][s].x);
+    } else if (phase == 3) {
+#pragma unroll
+      for (int s = 0; s < 8; ++s) v[0][s] = G[(size_t)(j + s * NY8) * H + col];
+    }
+    const bool cols = phase == 0 || phase == 3;
+    C* const sl[1] = {cols ? cslab : rslab};
+    const int ks = cols ? 1 << g.ltc : 1, jt = cols ? j : rj, lN = cols ? g.lny : g.lnx;
+    const C* const tw = cols ? g.twy : g.twx;
+    const double share = phase == 3 ? dots_share(g.dots, gridDim.x) : 0.0;
+    fxc fi[1][8];
+    FxScale sc[1];
+    if (lN >= kFxMinLog) {
+      fx_run<-1, 1, false>(v, fi, sl, ks, jt, lN, tw, sc);
+      if (phase != 2) {
+        const FxOut o = fx_out(sc[0], lN, 0);
+#pragma unroll
+        for (int s = 0; s < 8; ++s) v[0][s] = cmk<fx64>(fx_to(fi[0][s].x, o.eb), fx_to(fi[0][s].y, o.eb));
+        if (!o.plain) {
+#pragma unroll
+          for (int s = 0; s < 8; ++s)
+            v[0][s] = cmk<fx64>(v[0][s].x.v * o.f1 * o.f2, v[0][s].y.v * o.f1 * o.f2);
+        }
+      }
+    } else {
+      fft_rt<-1, 1, false>(v, sl, ks, jt, lN, tw);
+    }
+    if (phase == 0) {
+#pragma unroll
+      for (int s = 0; s < 8; ++s)
+        G[(size_t)(j + s * NY8) * H + col] = cmk<fx64>(v[0][s].y, v[0][s].x);
+      live = grid_barrier(bar, target += gridDim.x);
+      if (!live) break;
+      phase = 1;
+    } else if (phase == 1) {
+      // (m m + r I) grad d along the rows
+      double gkg = 0.0;
+      const fx64* smx = sf + (size_t)r0 * N;
+      const fx64* smy = smx + (size_t)g.rpc * N;
+      const fx64* srr = smy + (size_t)g.rpc * N;
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const int xp = rj + s * N8;
+        const fx64 gx = v[0][s].y, gy = v[0][s].x;
+        const fx64 ax = smx[xp], ay = smy[xp], rr = srr[xp];
+        const fx64 mg = ax * gx + ay * gy;
+        gkg += (mg * mg + rr * (gx * gx + gy * gy)).v;
+        v[0][s] = cmk<fx64>(ax * mg + rr * gx, ay * mg + rr * gy);
+      }
+      double a1[1] = {gkg};
+      block_sum<1>(a1);
+      if (t == 0) g.dots[blockIdx.x] = a1[0];
+      phase = 2;
+    } else if (phase == 2) {
+      if (lN >= kFxMinLog) fx_store_r2c<1>(fi, sc, sl, rj, lN, Ra, Rb);
+      else store_rows_r2c<1>(v, sl, rj, N, H, Ra, Rb);
+      live = grid_barrier(bar, target += gridDim.x);
+      if (!live) break;
+      phase = 3;
+    } else {
+      // A d = -div; x += alpha d, r -= alpha A d
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {  // the other half's slots go to it
+        const fx64 a = f == 0 ? kx : g.kyd[j + s * NY8].v;
+        v[0][s] = cscale(v[0][s], a);
+        if ((s >= 4) != (f == 1)) ex[s * hn] = v[0][s];
+      }
+      const double gkg = dots_total(share);  // its barriers also order ex
+      if (!loop_alpha(k, gkg, n, 0, thresh2)) break;
+      double acc[2] = {0.0, 0.0};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const C o = ex[(4 * f + i) * hn];
+        const C own = f == 0 ? v[0][i] : v[0][4 + i];
+        const double tx = own.x.v + o.x.v, ty = own.y.v + o.y.v;  // A d = (ty, -tx)
+        xv[i] = cmk<double>(xv[i].x + k.alpha * dv[i].x, xv[i].y + k.alpha * dv[i].y);
+        rv[i] = cmk<double>(rv[i].x - k.alpha * ty, rv[i].y + k.alpha * tx);
+        const double r2 = rv[i].x * rv[i].x + rv[i].y * rv[i].y;
+        acc[0] += r2;
+        acc[1] += r2 * pv[i];
+      }
+      acc[0] *= w;
+      acc[1] *= w;
+      block_sum<2>(acc);
+      if (t == 0) {
+        g.partials[(size_t)blockIdx.x * kPartialStride] = acc[0];
+        g.partials[(size_t)blockIdx.x * kPartialStride + 1] = acc[1];
+      }
+      live = grid_barrier(bar, target += gridDim.x);
+      if (!live) break;
+      double tot[2];
+      grid_total<2>(g.partials, kPartialStride, tot);
+      loop_beta(k, tot[0], tot[1], thresh2, maxit);
+      if (k.done) break;
+      phase = 0;
+    }
+  }
+  if (live) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[(size_t)(j + (4 * f + i) * NY8) * H + col] = xv[i];
+  }
+  if (blockIdx.x == 0 && t == 0) loop_finish(st, k, k.it - it0, !live);
+  loop_leave(st);
+}
+
 static inline size_t loop_smem(int nt, int rpc, int nx) {
   return (size_t)18 * nt * sizeof(cx<float>) + (size_t)3 * rpc * nx * sizeof(float) +
          (size_t)8 * nt * sizeof(cx<float>);
 }
 
-// Threads of a CTA: 16 values each in either pass, enough of them for a column and for two
-// rows, at most 128 CTAs, so that all are resident at one a SM.
-int cg_loop_threads(int nx, int ny) {
-  const long long n = (long long)nx * ny;
-  int nt = 32;
-  while (nt < ny / 8 || nt < nx / 8 || n / (16 * nt) > 128) nt *= 2;
-  if (nt > 512 || n < 16 * nt) return 0;
-  if (8 * nt / ny > 32 || 8 * nt / ny > nx / 2) return 0;
-  return nt;
+static inline size_t loop_smem_fx(int nt) {
+  return (size_t)13 * nt * sizeof(cx<fx64>) + (size_t)24 * nt * sizeof(fx64);
 }
 
-bool cg_loop_fits_f32(int nx, int ny, int nt) {
-  const int grid = (int)((long long)nx * ny / (16 * nt)), rpc = 16 * nt / nx;
-  const auto kernel = nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>;
+// Threads of a CTA: `per` values each in either pass (FP32: 16, two fields or two rows; fx64:
+// 8), enough of them for a column and for a row group, at most 128 CTAs, so that all are
+// resident at one a SM.
+static int loop_threads(int nx, int ny, int per) {
+  const long long n = (long long)nx * ny;
+  int nt = 32;
+  while (nt < 2 * ny / per || nt < nx / 8 || n / (per * nt) > 128) nt *= 2;
+  if (nt > 512 || n < (long long)per * nt) return 0;
+  const int tc = per * nt / (2 * ny);
+  return tc > 32 || tc > nx / 2 ? 0 : nt;
+}
+
+// All CTAs of the loop kernel resident at once on this device.
+template <typename K>
+static bool loop_fits(K kernel, int nt, size_t smem, long long grid) {
   allow_smem(kernel);
   int dev = 0, sms = 0, coop = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, nt, loop_smem(nt, rpc, nx)) !=
-          cudaSuccess) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, nt, smem) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   return coop && (long long)per * sms >= grid;
 }
 
+// Geometry of the loop's passes: per values a thread.
+template <typename T>
+static Geo<T> loop_geo(const Geo<T>& g0, int nt, int per) {
+  Geo<T> g = g0;
+  g.tc = per * nt / (2 * g.ny);
+  g.rpc = per * nt / g.nx;
+  for (g.ltc = 0; (1 << g.ltc) < g.tc;) ++g.ltc;
+  for (g.lrpc = 0; (1 << g.lrpc) < g.rpc;) ++g.lrpc;
+  return g;
+}
+
+int cg_loop_threads_f32(int nx, int ny) {
+  const int nt = loop_threads(nx, ny, 16);
+  if (!nt) return 0;
+  const long long grid = (long long)nx * ny / (16 * nt);
+  const size_t smem = loop_smem(nt, 16 * nt / nx, nx);
+  return loop_fits(nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>, nt, smem, grid) ? nt : 0;
+}
+int cg_loop_threads_fx(int nx, int ny) {
+  const int nt = loop_threads(nx, ny, 8);
+  // 512 threads would have to fit 128 registers: 1024x512 108 us an iteration either way,
+  // 32x2048 (16 CTAs) 110 -> 129
+  if (!nt || nt > 256) return 0;
+  const long long grid = (long long)nx * ny / (8 * nt);
+  return loop_fits(k_cg_loop_fx, nt, loop_smem_fx(nt), grid) ? nt : 0;
+}
+
 void cg_loop_f32(const Geo<float>& g0, int nt, cx<float>* x, const cx<float>* r, cx<float>* Gx,
                  cx<float>* Gy, const float* mx, const float* my, const float* rf, SolveState* st,
                  cudaStream_t s) {
-  Geo<float> g = g0;
+  Geo<float> g = loop_geo(g0, nt, 16);
   int row_sums = g0.rpc < 2;
-  g.tc = 8 * nt / g.ny;
-  g.rpc = 16 * nt / g.nx;
-  for (g.ltc = 0; (1 << g.ltc) < g.tc;) ++g.ltc;
-  for (g.lrpc = 0; (1 << g.lrpc) < g.rpc;) ++g.lrpc;
   void* args[] = {&g, &x, &r, &Gx, &Gy, &mx, &my, &rf, &st, &row_sums};
-  cudaLaunchCooperativeKernel((const void*)(nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>), dim3(g.H >> g.ltc), dim3(nt), args,
-                              loop_smem(nt, g.rpc, g.nx), s);
+  cudaLaunchCooperativeKernel((const void*)(nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>),
+                              dim3(g.H >> g.ltc), dim3(nt), args, loop_smem(nt, g.rpc, g.nx), s);
+}
+void cg_loop_fx(const Geo<double>& g0, int nt, cx<double>* x, const cx<double>* r, cx<double>* Gx,
+                cx<double>* Gy, const double* mx, const double* my, const double* rf,
+                SolveState* st, cudaStream_t s) {
+  Geo<fx64> g = loop_geo(as_fx(g0), nt, 8);
+  void* args[] = {&g, &x, &r, &Gx, &Gy, &mx, &my, &rf, &st};
+  cudaLaunchCooperativeKernel((const void*)k_cg_loop_fx,
+                              dim3(g.H >> g.ltc), dim3(nt), args, loop_smem_fx(nt), s);
 }
 
 }  // namespace hc

@@ -430,12 +430,9 @@ __device__ __forceinline__ void fft_fixed(cx<fx64> (&v)[NV][8], cx<fx64>* const*
 // exponent and the sums stay off the FP64 pipe.  (Two outputs of one transform
 // have a joint modulus within the vector's norm, so their sum fits as well.)
 template <int NV>
-__device__ __forceinline__ void fft_fixed_r2c(cx<fx64> (&v)[NV][8], cx<fx64>* const* sl, int j,
-                                              int lN, const cx<fx64>* __restrict__ tw,
-                                              cx<fx64>* const* A, cx<fx64>* const* B) {
-  FxScale sc[NV];
-  fxc f[NV][8];
-  fx_run<-1, NV, true>(v, f, sl, 1, j, lN, tw, sc);
+__device__ __forceinline__ void fx_store_r2c(const fxc (&f)[NV][8], const FxScale (&sc)[NV],
+                                             cx<fx64>* const* sl, int j, int lN, cx<fx64>* const* A,
+                                             cx<fx64>* const* B) {
   const int N = 1 << lN, N8 = N >> 3, H = N >> 1;
   __syncthreads();
 #pragma unroll
@@ -469,6 +466,15 @@ __device__ __forceinline__ void fft_fixed_r2c(cx<fx64> (&v)[NV][8], cx<fx64>* co
       if (B[q]) B[q][k] = bd;
     }
   }
+}
+template <int NV>
+__device__ __forceinline__ void fft_fixed_r2c(cx<fx64> (&v)[NV][8], cx<fx64>* const* sl, int j,
+                                              int lN, const cx<fx64>* __restrict__ tw,
+                                              cx<fx64>* const* A, cx<fx64>* const* B) {
+  FxScale sc[NV];
+  fxc f[NV][8];
+  fx_run<-1, NV, true>(v, f, sl, 1, j, lN, tw, sc);
+  fx_store_r2c<NV>(f, sc, sl, j, lN, A, B);
 }
 
 }  // namespace hc

@@ -601,11 +601,14 @@ void pinv_table(const Geo<double>& g, const SolveState* st, cudaStream_t s);
 void col_div_upd(const Geo<double>& g, const cx<double>* Qx, const cx<double>* Qy, const cx<double>* d,
                  cx<double>* x, cx<double>* r, SolveState* st, cudaStream_t s);
 void set_smem_limits_fx(int refined);
-// The CG loop of a 2D solve as one cooperative kernel (hc_cgloop.cu).  cg_loop_threads: its
-// CTA size for a grid, 0 where the separate kernels are the better ones; ..._fits: this device
-// keeps all its CTAs resident.
-int cg_loop_threads(int nx, int ny);
-bool cg_loop_fits_f32(int nx, int ny, int nt);
+// The CG loop of a 2D solve as one cooperative kernel (hc_cgloop.cu): FP32 inner solves and
+// plain FP64 ones (fx64).  cg_loop_threads_*: its CTA size for a grid, 0 where the separate
+// kernels are the better ones or this device does not keep all its CTAs resident.
+int cg_loop_threads_f32(int nx, int ny);
+int cg_loop_threads_fx(int nx, int ny);
+void cg_loop_fx(const Geo<double>& g, int nt, cx<double>* x, const cx<double>* r, cx<double>* Gx,
+                cx<double>* Gy, const double* mx, const double* my, const double* rf,
+                SolveState* st, cudaStream_t s);
 void cg_loop_f32(const Geo<float>& g, int nt, cx<float>* x, const cx<float>* r, cx<float>* Gx,
                  cx<float>* Gy, const float* mx, const float* my, const float* rf, SolveState* st,
                  cudaStream_t s);

@@ -213,6 +213,7 @@ struct hc_ctx {
   cudaStream_t cap_hi, cap_lo;          // capture streams of the lagged graph's two branches
   cudaStream_t io_stream;               // hc_set_state / hc_get_state: copies beside p's transform
   cudaEvent_t io_ev[2 + 4];             // entry, copies done, and one per row chunk of p
+  bool tuned;   // launch shapes set by hc_set_tuning
   int loop_nt;  // CTA size of the CG loop kernel, 0: an iteration's kernels apart
   int graph_nodes_fixed, graph_nodes_body, graph_nodes_outer;
 };
@@ -3109,13 +3110,27 @@ hc::Geo<T> class_geo(const hc::Geo<T>& own, const hc::Geo<T>& rep) {
   return g;
 }
 
-hc::BInst member_record(const hc_ctx* c, const hc_ctx* rep) {
+// Column tile of a class: a context's default narrows until one grid alone has CTAs enough for
+// the chip, and the rows of such a tile are partial 32-byte sectors.  nb grids need less, so the
+// tile widens to whole sectors while 256 CTAs remain.  Three steps of 16 members: 512^2 (tile 2 ->
+// 4) 22.5 -> 21.3 ms, 256^2 (1 -> 4) 9.1 -> 8.0; at 64 bytes 22.4 and 8.3, at 128 25.3 and 8.3.
+template <typename T>
+void class_widen(hc::Geo<T>& g, int nb, int max_threads) {
+  while (g.tc * (int)sizeof(cx<T>) < 32 && 2 * g.tc <= std::min(32, g.H) &&
+         (2 * g.tc) << (g.lny - 3) <= max_threads && (long long)nb * (g.H / (2 * g.tc)) >= 256) {
+    g.tc *= 2;
+    g.ltc += 1;
+  }
+}
+
+hc::BInst member_record(const hc_ctx* c, const hc::Geo<float>& gf, const hc::Geo<double>& gd,
+                        const hc::Geo<df64>& gq) {
   hc::BInst b{};
-  b.gf = class_geo(c->gf, rep->gf);
+  b.gf = class_geo(c->gf, gf);
   b.gfn = hc::col_narrow(b.gf);
-  b.gd = class_geo(c->gd, rep->gd);
+  b.gd = class_geo(c->gd, gd);
   b.gx = hc::as_fx(b.gd);
-  b.gq = class_geo(c->gq, rep->gq);
+  b.gq = class_geo(c->gq, gq);
   b.st = c->st;
   b.p64 = c->p64;
   b.b64 = c->b64;
@@ -3301,7 +3316,16 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
       bc.d_inst = reinterpret_cast<hc::BInst*>(p + 256);
       p += 256 + bc.members.size() * sizeof(hc::BInst);
       std::vector<hc::BInst> recs;
-      for (int k : bc.members) recs.push_back(member_record(b->ctx[k], rep));
+      hc::Geo<float> gf = rep->gf;
+      hc::Geo<double> gd = rep->gd;
+      hc::Geo<df64> gq = rep->gq;
+      if (!rep->tuned) {
+        const int nb = (int)bc.members.size();
+        class_widen(gf, nb, 1024);
+        class_widen(gd, nb, 256);
+        class_widen(gq, nb, 256);
+      }
+      for (int k : bc.members) recs.push_back(member_record(b->ctx[k], gf, gd, gq));
       if (cudaMemcpy(bc.d_inst, recs.data(), recs.size() * sizeof(hc::BInst),
                      cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(HC_ECUDA);
@@ -3487,6 +3511,7 @@ int hc_set_tuning(hc_ctx* c, const hc_tuning* t) {
   c->gf.lrpc = ilog2(t->row_rows[0]);
   c->gd.rpc = t->row_rows[1];
   c->gd.lrpc = ilog2(t->row_rows[1]);
+  c->tuned = true;
   c->gf.pipe = t->col_pipe[0];
   c->gd.pipe = t->col_pipe[1];
   c->gf.rpipe = t->row_pipe[0];

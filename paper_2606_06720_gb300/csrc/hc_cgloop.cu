@@ -19,12 +19,15 @@
 
 namespace hc {
 
-// Polls of a grid barrier before it gives up, about a second.
-constexpr unsigned kBarrierPolls = 1u << 20;
+// Polls of a grid barrier before it gives up, several seconds: another stream's kernel may
+// hold an SM that one of the CTAs waits for.
+constexpr unsigned kBarrierPolls = 1u << 23;
 
 // Grid barrier number `target / gridDim.x`.  The launch is cooperative, so every CTA is
 // resident and arrives.  False in every thread of a CTA whose wait ran out.  What any CTA
 // wrote before it is visible to every thread after it.
+// (One counter, polled with acquires: a word per CTA that a warp polls took 2.4 us more a
+// barrier at 128 CTAs, relaxed polls and one fence 0.3 us more.)
 __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target) {
   __shared__ int s_ok;
   __syncthreads();

@@ -1243,6 +1243,18 @@ int read_state(hc_ctx* c) {
   return c->st_host->loop_timeout ? HC_ETIMEOUT : HC_OK;
 }
 
+// One loop kernel at a time on a device: the CTAs of two might each hold SMs that the other's
+// missing ones wait for.  Held by the calls that launch them until they have synchronised.
+std::mutex g_loop_mu[64];  // by device
+struct LoopGuard {
+  std::unique_lock<std::mutex> lk;
+  template <typename C>
+  explicit LoopGuard(const C* c) {
+    int dev = 0;
+    if (c->loop_nt && cudaGetDevice(&dev) == cudaSuccess) lk = std::unique_lock<std::mutex>(g_loop_mu[dev & 63]);
+  }
+};
+
 // The whole CG loop of a solve in one launch (loop_nt > 0).
 void cg_loop(hc_ctx* c) {
   if (c->refined)
@@ -1342,7 +1354,10 @@ int step_host(hc_ctx* c) {
 //            [HC_FP32_REFINED: IF(mid){double-float residual, WHILE(mid_inner){CG}}],
 //            WHILE(outer){IF(dec){fx64 residual}, IF(again){FP64 residual, WHILE(inner){CG}}} with the default
 //            residual switches, else WHILE(outer){FP64 residual, WHILE(inner){CG}}, split, step_end
-int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h) {
+// link: nodes that the chain follows, and then its own last ones (chains with loop kernels, of
+// which one at a time may run).
+int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h,
+                std::vector<cudaGraphNode_t>* link = nullptr) {
   cudaStream_t s = c->stream;
   Handles hh;
   cudaStreamCaptureStatus cs;
@@ -1384,7 +1399,8 @@ int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h) {
     return HC_OK;
   };
   std::vector<cudaGraphNode_t> tail;
-  CU(cudaStreamBeginCaptureToGraph(s, target, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+  CU(cudaStreamBeginCaptureToGraph(s, target, link ? link->data() : nullptr, nullptr,
+                                   link ? link->size() : 0, cudaStreamCaptureModeThreadLocal));
   hc::step_begin(c->st, (int)c->n, s);
   if (c->refined)
     first_resid32(c);
@@ -1452,8 +1468,9 @@ int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h) {
                                    cudaStreamCaptureModeThreadLocal));
   split_step(c);
   hc::step_end(c->st, c->refined, s);
-  cudaGraph_t same = target;
-  CU(cudaStreamEndCapture(s, &same));
+  rc = end_capture(target, tail);
+  if (rc) return rc;
+  if (link) *link = tail;
   *h = hh;
   return HC_OK;
 }
@@ -2450,6 +2467,7 @@ int hc_get_state(hc_ctx* c, double* m_out, size_t m_count, double* p_out, size_t
 int hc_step(hc_ctx* c, int nsteps, hc_step_stats* last) {
   if (!c || nsteps < 0) return HC_EINVAL;
   if (nsteps == 0) return HC_OK;
+  LoopGuard guard(c);
   hc::reset_accum(c->st, c->stream);
   c->launches += 1;
   if (pipe_on(c, nsteps)) {
@@ -2517,6 +2535,7 @@ static void gradient3(hc_ctx* c) {
 int hc_run(hc_ctx* c, int max_steps, double eps, int stop_on_energy, int* steps_done,
            hc_step_stats* last) {
   if (!c || max_steps < 0) return HC_EINVAL;
+  LoopGuard guard(c);
   if (steps_done) *steps_done = 0;
   const int forced = c->prm.diagnostics ? 0 : 1;
   if (forced) {
@@ -3022,6 +3041,7 @@ int hc_adjoint(hc_ctx* c, int nsteps, int every, const double* lamT, double* dc2
   if (!c || !lamT || nsteps < 0 || every < 1) return HC_EINVAL;
   if (c->df || c->dim != 2 || c->gen) return HC_ENOTSUP;
   if (workspace && (reinterpret_cast<uintptr_t>(workspace) % kAlign)) return HC_EINVAL;
+  LoopGuard guard(c);
   size_t need = 0;
   int rc = hc_adjoint_workspace_size(c, nsteps, every, &need);
   if (rc) return rc;
@@ -3083,6 +3103,7 @@ struct hc_batch {
   std::vector<Handles> h;     // per-context chains
   std::vector<int> cls_of;    // class of each context, -1: its own chain
   std::vector<BatchClass> cls;
+  int loop_nt = 0;            // some chain has loop kernels
   void* dmem;                 // device memory of the classes
   cudaStream_t stream;
   cudaStream_t cap;
@@ -3352,6 +3373,7 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
       return fail(rc);
     }
   }
+  std::vector<cudaGraphNode_t> link;
   for (int i = 0; i < count; ++i) {
     if (b->cls_of[i] >= 0) continue;
     hc_ctx* c = b->ctx[i];
@@ -3362,7 +3384,8 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
     cudaStream_t keep = c->stream;
     long long before = c->launches;
     c->stream = b->cap;
-    int rc = build_chain(c, graph, &b->h[i]);
+    int rc = build_chain(c, graph, &b->h[i], c->loop_nt ? &link : nullptr);
+    b->loop_nt = b->loop_nt ? b->loop_nt : c->loop_nt;
     c->stream = keep;
     c->launches = before;
     if (rc) {
@@ -3383,6 +3406,7 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
 
 int hc_batch_step(hc_batch* b, int nsteps, hc_step_stats* stats) {
   if (!b || nsteps < 0) return HC_EINVAL;
+  LoopGuard guard(b);
   if (nsteps == 0) return HC_OK;
   const int n = (int)b->ctx.size();
   for (int i = 0; i < n; ++i) {

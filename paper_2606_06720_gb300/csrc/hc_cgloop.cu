@@ -103,6 +103,15 @@ __device__ __forceinline__ void loop_finish(SolveState* st, const LoopCg& k, int
   predict_residual(st);
   if (st->graph_mode) cudaGraphSetConditional(st->h_cur, 0u);
 }
+// After a wait that ran out nothing is tried again: the solve ends here.
+__device__ __forceinline__ bool loop_gave_up(SolveState* st) {
+  if (!st->loop_timeout) return false;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->done = 1;
+    if (st->graph_mode) cudaGraphSetConditional(st->h_cur, 0u);
+  }
+  return true;
+}
 // The last CTA to leave re-arms the barrier.
 __device__ __forceinline__ void loop_leave(SolveState* st) {
   if (threadIdx.x == 0) {
@@ -148,6 +157,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
                                                         SolveState* st, int row_sums) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (st->done) return;  // nothing writes it before every CTA has passed a barrier
+  if (loop_gave_up(st)) return;
   using C = cx<float>;
   C* sm = reinterpret_cast<C*>(smem_raw);
   const int nt = blockDim.x, t = threadIdx.x, H = g.H;
@@ -327,6 +337,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
                                                         SolveState* st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (st->done) return;  // nothing writes it before every CTA has passed a barrier
+  if (loop_gave_up(st)) return;
   using C = cx<fx64>;
   C* sm = reinterpret_cast<C*>(smem_raw);
   const int nt = blockDim.x, hn = nt >> 1, t = threadIdx.x, H = g.H;

@@ -2464,10 +2464,8 @@ int hc_get_state(hc_ctx* c, double* m_out, size_t m_count, double* p_out, size_t
   return HC_OK;
 }
 
-int hc_step(hc_ctx* c, int nsteps, hc_step_stats* last) {
-  if (!c || nsteps < 0) return HC_EINVAL;
-  if (nsteps == 0) return HC_OK;
-  LoopGuard guard(c);
+// nsteps > 0 steps; the caller holds the LoopGuard (exported calls take it, bodies do not).
+static int step_body(hc_ctx* c, int nsteps, hc_step_stats* last) {
   hc::reset_accum(c->st, c->stream);
   c->launches += 1;
   if (pipe_on(c, nsteps)) {
@@ -2502,6 +2500,13 @@ int hc_step(hc_ctx* c, int nsteps, hc_step_stats* last) {
   if (rc) return rc;
   fill_stats(c, last);
   return c->st_host->first_bad;
+}
+
+int hc_step(hc_ctx* c, int nsteps, hc_step_stats* last) {
+  if (!c || nsteps < 0) return HC_EINVAL;
+  if (nsteps == 0) return HC_OK;
+  LoopGuard guard(c);
+  return step_body(c, nsteps, last);
 }
 
 static void gradient3(hc_ctx* c) {
@@ -2950,7 +2955,7 @@ int adjoint_t(hc_ctx* c, hc::Geo<T>& g, int nsteps, int every, const double* lam
                          a.cpk + kMsums * (k / every));
       if (rc) return rc;
     }
-    rc = hc_step(c, 1, nullptr);
+    rc = step_body(c, 1, nullptr);
     if (rc == HC_ENOCONV) status = status ? status : rc;
     else if (rc) return rc;
   }
@@ -2974,7 +2979,7 @@ int adjoint_t(hc_ctx* c, hc::Geo<T>& g, int nsteps, int every, const double* lam
     for (int k = k0; k < k1; ++k) {
       rc = save_state<T>(c, a.segm + 2 * n * (k - k0), nullptr, a.segk + kMsums * (k - k0));
       if (rc) return rc;
-      rc = hc_step(c, 1, nullptr);
+      rc = step_body(c, 1, nullptr);
       if (rc && rc != HC_ENOCONV) return rc;
       CU(cudaMemcpyAsync(a.segp + ns * (k - k0), c->p64, sizeof(cx<double>) * ns,
                          cudaMemcpyDeviceToDevice, s));

@@ -46,7 +46,7 @@ extern "C" {
 #define HC_ECUDA (-3)      /* a CUDA runtime call failed (the context should be destroyed) */
 #define HC_ENOCONV (-4)    /* CG hit its iteration cap; the state was still advanced */
 #define HC_ENONFINITE (-5) /* NaN/Inf in p or m, e.g. the activation exponential overflowed (Remark 2.1) */
-#define HC_ETIMEOUT (-6)   /* a bounded device-side wait gave up */
+#define HC_ETIMEOUT (-6)   /* a bounded device-side wait gave up (hc_set_loop_wait) */
 #define HC_ENOTSUP (-7)    /* valid request that this build does not implement */
 #define HC_EBOUNDS (-8)    /* bounds-checked build: a guard zone after a device buffer was written */
 
@@ -242,6 +242,17 @@ int hc_get_m(hc_ctx* ctx, double* out, size_t count);
  * link bandwidth.  Errors: HC_EINVAL (NULL, wrong counts), HC_ECUDA. */
 int hc_set_state(hc_ctx* ctx, const double* m, size_t m_count, const double* p, size_t p_count);
 int hc_get_state(hc_ctx* ctx, double* m_out, size_t m_count, double* p_out, size_t p_count);
+
+/* Limits of the waits inside the CG loop kernels (2D solves up to about 10^6
+ * points).  Their CTAs meet at grid barriers and may have to wait there for a
+ * CTA whose SM another kernel holds.  After `polls` looks at a barrier's count
+ * (default 2^20, most of a second; 0: no wait at all, so that no loop kernel
+ * ends) the launch leaves the solve as it found it and runs again; `seconds`
+ * (default 120) after the first such launch of a solve the call that made it
+ * returns HC_ETIMEOUT.  The context stays usable: its m and p are then those of
+ * an unfinished step, to be set anew.
+ * Errors: HC_EINVAL (NULL, seconds negative, above 1e9 or NaN), HC_ECUDA. */
+int hc_set_loop_wait(hc_ctx* ctx, unsigned polls, double seconds);
 
 /* --- Component entry points (each runs one part of the step on the GPU) --- */
 

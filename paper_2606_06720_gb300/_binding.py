@@ -96,6 +96,7 @@ def _load() -> C.CDLL:
         "hc_get_m": ([P, dp, C.c_size_t], C.c_int),
         "hc_set_state": ([P, dp, C.c_size_t, dp, C.c_size_t], C.c_int),
         "hc_get_state": ([P, dp, C.c_size_t, dp, C.c_size_t], C.c_int),
+        "hc_set_loop_wait": ([P, C.c_uint, C.c_double], C.c_int),
         "hc_gradient": ([P, dp, C.c_size_t], C.c_int),
         "hc_apply_operator": ([P, dp, dp, C.c_size_t], C.c_int),
         "hc_split_step": ([P], C.c_int),
@@ -142,6 +143,7 @@ hc_get_p = lib.hc_get_p
 hc_get_m = lib.hc_get_m
 hc_set_state = lib.hc_set_state
 hc_get_state = lib.hc_get_state
+hc_set_loop_wait = lib.hc_set_loop_wait
 hc_gradient = lib.hc_gradient
 hc_apply_operator = lib.hc_apply_operator
 hc_split_step = lib.hc_split_step
@@ -459,6 +461,10 @@ class Solver:
         nz, zone, owner = C.c_int(), C.c_int(), C.c_size_t()
         rc = hc_check_redzones(self.ctx, C.byref(nz), C.byref(zone), C.byref(owner))
         return {"rc": rc, "zones": nz.value, "zone": zone.value, "owner_bytes": owner.value}
+
+    def set_loop_wait(self, polls: int = 1 << 20, seconds: float = 120.0) -> None:
+        """Limits of the loop kernels' waits (see hc_set_loop_wait)."""
+        _check(hc_set_loop_wait(self.ctx, int(polls), float(seconds)), "hc_set_loop_wait")
 
     def launch_count(self) -> int:
         v = C.c_longlong()

@@ -215,6 +215,10 @@ struct hc_ctx {
   cudaEvent_t io_ev[2 + 4];             // entry, copies done, and one per row chunk of p
   bool tuned;   // launch shapes set by hc_set_tuning
   int loop_nt;  // CTA size of the CG loop kernel, 0: an iteration's kernels apart
+  // hc_set_loop_wait.  2^20 polls are most of a second: longer than any CTA of a loop takes to
+  // arrive, unless another kernel holds the SM that it needs.
+  unsigned loop_polls = 1u << 20;
+  double loop_patience = 120.0;
   int graph_nodes_fixed, graph_nodes_body, graph_nodes_outer;
 };
 
@@ -834,6 +838,8 @@ int push_config(hc_ctx* c) {
   cfg.max_sweeps = c->prm.max_sweeps;
   cfg.graph_mode = 0;  // set true only while a graph runs
   cfg.refined = c->refined;
+  cfg.loop_polls = c->loop_polls;
+  cfg.loop_patience = (unsigned long long)(c->loop_patience * 1e9);
   hc::set_config(c->st, cfg, c->stream);
   c->launches += 1;
   CU(cudaGetLastError());
@@ -1237,10 +1243,18 @@ void split_step(hc_ctx* c) {
     split_step_t<double>(c, c->gd, c->G64);
 }
 
+// HC_ETIMEOUT, once, if a loop kernel's solve was given up (st_host is up to date).
+int loop_reported(hc_ctx* c, cudaStream_t s) {
+  if (!c->st_host->loop_timeout) return HC_OK;
+  CU(cudaMemsetAsync(&c->st->loop_timeout, 0, sizeof(int), s));
+  CU(cudaStreamSynchronize(s));
+  return HC_ETIMEOUT;
+}
+
 int read_state(hc_ctx* c) {
   CU(cudaMemcpyAsync(c->st_host, c->st, sizeof(hc::SolveState), cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
-  return c->st_host->loop_timeout ? HC_ETIMEOUT : HC_OK;
+  return loop_reported(c, c->stream);
 }
 
 // One loop kernel at a time on a device: the CTAs of two might each hold SMs that the other's
@@ -1268,10 +1282,12 @@ void cg_loop(hc_ctx* c) {
 // Launch CG iterations in chunks until the device says done.
 int run_cg_host(hc_ctx* c, bool refined_inner) {
   if (c->loop_nt) {
-    cg_loop(c);
-    CU(cudaGetLastError());
-    int rc = read_state(c);
-    if (rc) return rc;
+    do {  // a launch that was given up ends nothing; the device counts the time
+      cg_loop(c);
+      CU(cudaGetLastError());
+      int rc = read_state(c);
+      if (rc) return rc;
+    } while (!c->st_host->done);
     c->launches += (long long)c->graph_nodes_body * c->st_host->it;
     return HC_OK;
   }
@@ -1844,8 +1860,8 @@ int step_lagged(hc_ctx* c, int nsteps) {
   c->launches += 3;
   CU(cudaGetLastError());
   rc = read_state(c);
-  if (!rc) rc = set_graph_mode(c, 0);
-  if (rc) return rc;
+  int rc2 = set_graph_mode(c, 0);
+  if (rc || rc2) return rc ? rc : rc2;
   const hc::SolveState& h = *c->st_host;  // counters were reset at the call's start
   c->launches += kPipeFixedKernels * (long long)h.acc_steps + (long long)(nsteps - h.acc_steps) +
                  (long long)c->graph_nodes_body * h.acc_iters +
@@ -1871,8 +1887,8 @@ int step_lagged(hc_ctx* c, int nsteps) {
   if (rc) return rc;
   for (int k = done; k < nsteps; ++k) CU(cudaGraphLaunch(c->gexec, c->stream));
   rc = read_state(c);
-  if (!rc) rc = set_graph_mode(c, 0);
-  if (rc) return rc;
+  rc2 = set_graph_mode(c, 0);
+  if (rc || rc2) return rc ? rc : rc2;
   const hc::SolveState& h2 = *c->st_host;
   c->launches += (long long)c->graph_nodes_fixed * (h2.acc_steps - b2.acc_steps) +
                  (long long)c->graph_nodes_body * (h2.acc_iters - b2.acc_iters) +
@@ -2063,6 +2079,16 @@ int hc_create(hc_ctx** out, const hc_grid* grid, const hc_params* params, void* 
     return rc;
   }
   *out = c;
+  return HC_OK;
+}
+
+int hc_set_loop_wait(hc_ctx* c, unsigned polls, double seconds) {
+  if (!c || !(seconds >= 0.0) || seconds > 1e9) return HC_EINVAL;
+  c->loop_polls = polls;
+  c->loop_patience = seconds;
+  const int rc = push_config(c);
+  if (rc) return rc;
+  CU(cudaStreamSynchronize(c->stream));
   return HC_OK;
 }
 
@@ -3453,7 +3479,8 @@ int hc_batch_step(hc_batch* b, int nsteps, hc_step_stats* stats) {
     if (b->cls_of[i] < 0) c->launches += graph_kernel_count(c, h);
     if (stats) fill_stats(c, &stats[i]);
     if (!first_bad && h.first_bad) first_bad = h.first_bad;
-    if (h.loop_timeout) first_bad = HC_ETIMEOUT;
+    const int lost = loop_reported(c, b->stream);
+    if (lost) first_bad = lost;
     int rc = set_graph_mode(c, 0);
     if (rc) return rc;
   }

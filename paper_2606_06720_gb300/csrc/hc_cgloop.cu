@@ -19,34 +19,61 @@
 
 namespace hc {
 
-// Polls of a grid barrier before it gives up, several seconds: another stream's kernel may
-// hold an SM that one of the CTAs waits for.
-constexpr unsigned kBarrierPolls = 1u << 23;
-
-// Grid barrier number `target / gridDim.x`.  The launch is cooperative, so every CTA is
-// resident and arrives.  False in every thread of a CTA whose wait ran out.  What any CTA
-// wrote before it is visible to every thread after it.
-// (One counter, polled with acquires: a word per CTA that a warp polls took 2.4 us more a
-// barrier at 128 CTAs, relaxed polls and one fence 0.3 us more.)
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target) {
-  __shared__ int s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-    int ok = 0;
-    for (unsigned i = 0; i < kBarrierPolls; ++i) {
-      unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-      if (v >= target) {
-        ok = 1;
-        break;
-      }
+// The grid barriers of one launch.  The launch is cooperative, so every CTA is resident and
+// arrives; a wait is bounded all the same (st->loop_polls polls), because another stream's
+// kernel may hold an SM that a CTA waits for.  A barrier completes for every CTA or for none: one
+// that gives up marks the word with a compare-and-swap that fails once the count is complete, and
+// whoever sees the mark gives up too.  A CTA still polling an earlier barrier leaves as well, and
+// no later one completes without it.  x is stored after the last barrier, so a launch that is
+// given up has changed nothing and can simply be repeated (loop_leave).
+// Arrivals count in twos (the count may wrap); the mark is bit 0, and 2^30 more, so that one
+// comparison ends a poll either way.
+struct LoopBar {
+  unsigned* word;
+  unsigned polls;
+  unsigned target = 0;
+  // What any CTA wrote before it is visible to every thread after it.  False in every thread
+  // once the launch is given up.
+  // (One counter, polled with acquires: a word per CTA that a warp polls took 2.4 us more a
+  // barrier at 128 CTAs, relaxed polls and one fence 0.3 us more; polls one at a time, ten steps
+  // of 64^2 FP64 13.84 ms, unrolled by four 13.79.)
+  __device__ __forceinline__ bool wait() {
+    __shared__ int s_ok;
+    target += 2 * gridDim.x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned v = target - 1u;
+      if (polls == 0)  // no wait at all: marked in place of arriving
+        asm volatile("red.release.gpu.global.or.b32 [%0], 1;" ::"l"(word) : "memory");
+      else
+        asm volatile("red.release.gpu.global.add.u32 [%0], 2;" ::"l"(word) : "memory");
+#pragma unroll 4
+      for (unsigned i = 0; i < polls && !past(v); ++i)
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
+      if (!past(v)) v = give_up();
+      s_ok = !(v & 1u);
     }
-    s_ok = ok;
+    __syncthreads();
+    return s_ok != 0;
   }
-  __syncthreads();
-  return s_ok != 0;
-}
+  __device__ __forceinline__ bool past(unsigned v) const { return (int)(v - target) >= 0; }
+  // The word after this CTA's mark, or as it is where it is marked or complete already.  Each
+  // failed swap is an arrival, or another CTA's mark: at most one round per CTA.
+  __device__ __noinline__ unsigned give_up() {
+    unsigned v, old;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
+    for (unsigned i = 0; i <= gridDim.x; ++i) {
+      if ((v & 1u) || past(v)) return v;
+      asm volatile("atom.acq_rel.gpu.global.cas.b32 %0, [%1], %2, %3;"
+                   : "=r"(old)
+                   : "l"(word), "r"(v), "r"((v + 0x40000000u) | 1u)
+                   : "memory");
+      if (old == v) break;
+      v = old;
+    }
+    return 1u;
+  }
+};
 
 // The scalars of a solve, kept by every thread alike.
 struct LoopCg {
@@ -87,7 +114,7 @@ __device__ __forceinline__ void loop_beta(LoopCg& k, double rr, double rz, doubl
 }
 // The end of the loop, one thread of the grid: the solve state as the kernels of an
 // iteration would have left it.
-__device__ __forceinline__ void loop_finish(SolveState* st, const LoopCg& k, int its, bool timeout) {
+__device__ __forceinline__ void loop_finish(SolveState* st, const LoopCg& k, int its) {
   st->rnorm2 = k.rnorm2;
   st->alpha = k.alpha;
   st->alpha_f = (float)k.alpha;
@@ -97,13 +124,12 @@ __device__ __forceinline__ void loop_finish(SolveState* st, const LoopCg& k, int
   st->it = k.it;
   st->total_it += its;
   if (k.status) st->status = k.status;
-  if (timeout) st->loop_timeout = 1;
   st->first = 0;
   st->done = 1;
   predict_residual(st);
   if (st->graph_mode) cudaGraphSetConditional(st->h_cur, 0u);
 }
-// After a wait that ran out nothing is tried again: the solve ends here.
+// A solve of a call in which an earlier one was given up for good ends here.
 __device__ __forceinline__ bool loop_gave_up(SolveState* st) {
   if (!st->loop_timeout) return false;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -112,15 +138,28 @@ __device__ __forceinline__ bool loop_gave_up(SolveState* st) {
   }
   return true;
 }
-// The last CTA to leave re-arms the barrier.
-__device__ __forceinline__ void loop_leave(SolveState* st) {
-  if (threadIdx.x == 0) {
-    unsigned t;
-    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(&st->loop_exit) : "memory");
-    if (t == gridDim.x - 1) {
-      st->loop_exit = 0u;
-      st->loop_bar = 0u;
-    }
+// The last CTA to leave re-arms the barriers.  A launch that was given up leaves the solve as it
+// found it, so it runs again (the WHILE node's next turn, or the host's next launch), until
+// st->loop_patience ns after the first one.
+__device__ __forceinline__ void loop_leave(SolveState* st, bool live) {
+  if (threadIdx.x != 0) return;
+  unsigned t;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(&st->loop_exit) : "memory");
+  if (t != gridDim.x - 1) return;
+  st->loop_exit = 0u;
+  st->loop_bar = 0u;
+  if (live) {
+    st->loop_since = 0ull;
+    return;
+  }
+  unsigned long long now;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+  if (!st->loop_since) st->loop_since = now;
+  if (now - st->loop_since >= st->loop_patience) {
+    st->loop_since = 0ull;
+    st->loop_timeout = 1;
+    st->done = 1;
+    if (st->graph_mode) cudaGraphSetConditional(st->h_cur, 0u);
   }
 }
 
@@ -190,8 +229,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
   const Pc<float> pc = pc_of<float>(st);
   LoopCg k{st->rho, st->rnorm2, 0.0, 0.0, st->it, 0, 0};
   const int it0 = k.it;
-  unsigned* const bar = &st->loop_bar;
-  unsigned target = 0;
+  LoopBar bar{&st->loop_bar, st->loop_polls};
   const float invn = exp2_neg<float>(g.lnx + g.lny), kx = g.kxd[c.kx];
   const float ax = kx * invn;
   const float wt = c.kx == 0 ? 1.0f : 2.0f;  // Parseval weight of a packed column
@@ -211,7 +249,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
     xs[(size_t)s * nt] = x[i];
   }
   cp_async_wait_all();
-  bool live = true;  // no wait has run out
+  bool live = true;  // the launch has not been given up
   while (true) {
     // gradient of d = M^-1 r + beta d
     const bool first = k.it == it0;
@@ -233,7 +271,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
       Gx[idx] = v[0][s];
       Gy[idx] = v[1][s];
     }
-    live = grid_barrier(bar, target += gridDim.x);
+    live = bar.wait();
     if (!live) break;
     // (m m + r I) grad d along the rows, in place
     load_rows_c2r<2>(v, (const C* const*)Ra, (const C* const*)Rb, rj, N8);
@@ -267,7 +305,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
       cta_pair_sums<1>(h, l, p);
       if (t == 0) g.dots[blockIdx.x] = p[0];
     }
-    live = grid_barrier(bar, target += gridDim.x);
+    live = bar.wait();
     if (!live) break;
     // A d = -div; x += alpha d, r -= alpha A d
     const double share = t < (int)gridDim.x ? __ldcg(&g.dots[t]) : 0.0;
@@ -307,7 +345,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
         g.partials[(size_t)blockIdx.x * kPartialStride + 1] = p[1];
       }
     }
-    live = grid_barrier(bar, target += gridDim.x);
+    live = bar.wait();
     if (!live) break;
     double tot[2];
     grid_total<2>(g.partials, kPartialStride, tot);
@@ -318,8 +356,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
 #pragma unroll
     for (int s = 0; s < 8; ++s) x[cmi(g, c.j + s * c.NY8, c.kx)] = xs[(size_t)s * nt];
   }
-  if (blockIdx.x == 0 && t == 0) loop_finish(st, k, k.it - it0, !live);
-  loop_leave(st);
+  if (live && blockIdx.x == 0 && t == 0) loop_finish(st, k, k.it - it0);
+  loop_leave(st, live);
 }
 
 // Plain FP64 solve (fx64 transforms, row-major x and r).  A warp's instructions are what
@@ -372,8 +410,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
   const int maxit = st->maxit;
   LoopCg k{st->rho, st->rnorm2, 0.0, 0.0, st->it, 0, 0};
   const int it0 = k.it;
-  unsigned* const bar = &st->loop_bar;
-  unsigned target = 0;
+  LoopBar bar{&st->loop_bar, st->loop_polls};
   const double kx = g.kxd[col].v;
   const double w = col == 0 ? 1.0 : 2.0;  // Parseval weight of a packed column
   cx<double> xv[4], rv[4], dv[4];
@@ -387,7 +424,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
     pv[i] = g.pinv[e];
   }
   cp_async_wait_all();
-  bool live = true;  // no wait has run out
+  bool live = true;  // the launch has not been given up
   C v[1][8];
   int phase = 0;  // columns inverse, rows inverse, rows forward, columns forward
 #pragma unroll 1
@@ -442,7 +479,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
 #pragma unroll
       for (int s = 0; s < 8; ++s)
         G[(size_t)(j + s * NY8) * H + col] = cmk<fx64>(v[0][s].y, v[0][s].x);
-      live = grid_barrier(bar, target += gridDim.x);
+      live = bar.wait();
       if (!live) break;
       phase = 1;
     } else if (phase == 1) {
@@ -467,7 +504,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
     } else if (phase == 2) {
       if (lN >= kFxMinLog) fx_store_r2c<1>(fi, sc, sl, rj, lN, Ra, Rb);
       else store_rows_r2c<1>(v, sl, rj, N, H, Ra, Rb);
-      live = grid_barrier(bar, target += gridDim.x);
+      live = bar.wait();
       if (!live) break;
       phase = 3;
     } else {
@@ -499,7 +536,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
         g.partials[(size_t)blockIdx.x * kPartialStride] = acc[0];
         g.partials[(size_t)blockIdx.x * kPartialStride + 1] = acc[1];
       }
-      live = grid_barrier(bar, target += gridDim.x);
+      live = bar.wait();
       if (!live) break;
       double tot[2];
       grid_total<2>(g.partials, kPartialStride, tot);
@@ -512,8 +549,8 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
 #pragma unroll
     for (int i = 0; i < 4; ++i) x[(size_t)(j + (4 * f + i) * NY8) * H + col] = xv[i];
   }
-  if (blockIdx.x == 0 && t == 0) loop_finish(st, k, k.it - it0, !live);
-  loop_leave(st);
+  if (live && blockIdx.x == 0 && t == 0) loop_finish(st, k, k.it - it0);
+  loop_leave(st, live);
 }
 
 static inline size_t loop_smem(int nt, int rpc, int nx) {

@@ -201,9 +201,12 @@ struct SolveState {
   int delta_added;           // the fx64 residual has added the pending correction to p64
   int acc_again;             // fx64 residuals that missed, summed over the steps since the last reset
   unsigned int ticket[8];    // last-CTA tickets, one per reduction site
-  unsigned int loop_bar;     // CG loop kernel: arrivals at its grid barriers (0 between launches)
+  unsigned int loop_bar;     // CG loop kernel: its grid barriers' word (0 between launches)
   unsigned int loop_exit;    // CTAs that have left it
-  int loop_timeout;          // a barrier's bounded wait ran out (sticky)
+  unsigned int loop_polls;   // polls of one barrier before the launch is given up
+  int loop_timeout;          // a solve was given up for good (until the host has read it)
+  unsigned long long loop_patience;  // ns for which launches that were given up are repeated
+  unsigned long long loop_since;     // global timer at the first of them, 0: none
   // Diagnostics of Section 2.5, accumulated by the split step when diag != 0.
   // A step solves p[m^k] and so evaluates E_h(m^k) with its own pressure.
   double dsum[3];            // running step: sum r|g|^2, sum (m.g)^2, sum |m|^(2 gamma) (gamma = 0: sum ln|m|); m = m^k, g = grad p[m^k]
@@ -254,6 +257,8 @@ struct SolveConfig {
   int refined;
   int dim;
   int diag;
+  unsigned int loop_polls;   // see SolveState
+  unsigned long long loop_patience;
 };
 
 // Doubles of per-CTA partial sums a reducing kernel may hand to its last CTA.

@@ -72,6 +72,8 @@ __global__ void k_set_config(SolveState* st, SolveConfig c) {
   st->max_sweeps = c.max_sweeps;
   st->graph_mode = c.graph_mode;
   st->refined = c.refined;
+  st->loop_polls = c.loop_polls;
+  st->loop_patience = c.loop_patience;
 }
 
 __global__ void k_step_begin(SolveState* st, int npts) { step_begin_body(st, npts); }

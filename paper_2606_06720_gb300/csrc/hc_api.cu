@@ -12,6 +12,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -556,6 +557,21 @@ int cuda_fail(cudaError_t e, const char* call, int line) {
     cudaError_t e_ = (x);                                       \
     if (e_ != cudaSuccess) return cuda_fail(e_, #x, __LINE__);  \
   } while (0)
+#define HC_TRY(x)         \
+  do {                    \
+    const int rc_ = (x);  \
+    if (rc_) return rc_;  \
+  } while (0)
+
+// Host values that the context's kernels read, on its own stream: a cudaMemcpy from pageable
+// memory may return before its last piece has arrived, and orders nothing with a non-blocking
+// stream.  (The handles of a step's graph so came late where several solvers stepped on threads of
+// their own: steps whose loops were skipped, or ran for ever.)
+int upload(hc_ctx* c, void* dst, const void* src, size_t bytes) {
+  CU(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream));
+  CU(cudaStreamSynchronize(c->stream));
+  return HC_OK;
+}
 
 // ------------------------------------------------------------------ guard zones
 #if HC_CHECK
@@ -627,13 +643,13 @@ int scan_zones(cudaStream_t s, const char* base, const Zones& z, int* bad) {
 // the ny rows.
 int upload_tables_generic(hc_ctx* c) {
   const std::vector<hc::FxTw> qx = twiddles_q62(c->nx), qy = twiddles_q62(c->ny);
-  CU(cudaMemcpy(c->twx_x, qx.data(), sizeof(hc::FxTw) * c->nx, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->twy_x, qy.data(), sizeof(hc::FxTw) * c->ny, cudaMemcpyHostToDevice));
+  HC_TRY(upload(c, c->twx_x, qx.data(), sizeof(hc::FxTw) * c->nx));
+  HC_TRY(upload(c, c->twy_x, qy.data(), sizeof(hc::FxTw) * c->ny));
   std::vector<double> kx(c->H), ky(c->ny);
   for (int k = 0; k < c->H; ++k) kx[k] = xid(k, c->nx, c->grid.L[0]);
   for (int k = 0; k < c->ny; ++k) ky[k] = xid(k, c->ny, c->grid.L[1]);
-  CU(cudaMemcpy(c->kxd_d, kx.data(), sizeof(double) * c->H, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->kyd_d, ky.data(), sizeof(double) * c->ny, cudaMemcpyHostToDevice));
+  HC_TRY(upload(c, c->kxd_d, kx.data(), sizeof(double) * c->H));
+  HC_TRY(upload(c, c->kyd_d, ky.data(), sizeof(double) * c->ny));
   return HC_OK;
 }
 
@@ -678,11 +694,11 @@ int upload_tables(hc_ctx* c) {
       hq[m].x = df64(re[m]);
       hq[m].y = df64(im[m]);
     }
-    CU(cudaMemcpy(df, hf.data(), sizeof(cx<float>) * N, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(dd, hd.data(), sizeof(cx<double>) * N, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(dq, hq.data(), sizeof(cx<df64>) * N, cudaMemcpyHostToDevice));
+    HC_TRY(upload(c, df, hf.data(), sizeof(cx<float>) * N));
+    HC_TRY(upload(c, dd, hd.data(), sizeof(cx<double>) * N));
+    HC_TRY(upload(c, dq, hq.data(), sizeof(cx<df64>) * N));
     const std::vector<hc::FxTw> hx = twiddles_fx(N);
-    CU(cudaMemcpy(dx, hx.data(), sizeof(hc::FxTw) * N, cudaMemcpyHostToDevice));
+    HC_TRY(upload(c, dx, hx.data(), sizeof(hc::FxTw) * N));
     return HC_OK;
   };
   int rc = put_tw(c->nx, c->twx_f, c->twx_d, c->twx_q, c->twx_x);
@@ -693,21 +709,21 @@ int upload_tables(hc_ctx* c) {
   for (int k = 0; k < c->H; ++k) kx[k] = (k == 0) ? 0.0 : xid(k, c->nx, c->grid.L[0]);
   for (int k = 0; k < c->ny; ++k) ky[k] = xid(k, c->ny, c->grid.L[1]);
   std::vector<float> kxf(kx.begin(), kx.end()), kyf(ky.begin(), ky.end());
-  CU(cudaMemcpy(c->kxd_d, kx.data(), sizeof(double) * c->H, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->kyd_d, ky.data(), sizeof(double) * c->ny, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->kxd_f, kxf.data(), sizeof(float) * c->H, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->kyd_f, kyf.data(), sizeof(float) * c->ny, cudaMemcpyHostToDevice));
+  HC_TRY(upload(c, c->kxd_d, kx.data(), sizeof(double) * c->H));
+  HC_TRY(upload(c, c->kyd_d, ky.data(), sizeof(double) * c->ny));
+  HC_TRY(upload(c, c->kxd_f, kxf.data(), sizeof(float) * c->H));
+  HC_TRY(upload(c, c->kyd_f, kyf.data(), sizeof(float) * c->ny));
   std::vector<double> x2x(c->H + 1), x2y(c->ny);
   for (int k = 0; k <= c->H; ++k) x2x[k] = xi(k, c->nx, c->grid.L[0]) * xi(k, c->nx, c->grid.L[0]);
   for (int k = 0; k < c->ny; ++k) x2y[k] = xi(k, c->ny, c->grid.L[1]) * xi(k, c->ny, c->grid.L[1]);
   std::vector<float> x2xf(x2x.begin(), x2x.end()), x2yf(x2y.begin(), x2y.end());
-  CU(cudaMemcpy(c->x2x_d, x2x.data(), sizeof(double) * (c->H + 1), cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->x2y_d, x2y.data(), sizeof(double) * c->ny, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->x2x_f, x2xf.data(), sizeof(float) * (c->H + 1), cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->x2y_f, x2yf.data(), sizeof(float) * c->ny, cudaMemcpyHostToDevice));
+  HC_TRY(upload(c, c->x2x_d, x2x.data(), sizeof(double) * (c->H + 1)));
+  HC_TRY(upload(c, c->x2y_d, x2y.data(), sizeof(double) * c->ny));
+  HC_TRY(upload(c, c->x2x_f, x2xf.data(), sizeof(float) * (c->H + 1)));
+  HC_TRY(upload(c, c->x2y_f, x2yf.data(), sizeof(float) * c->ny));
   std::vector<df64> kxq(kx.begin(), kx.end()), kyq(ky.begin(), ky.end());
-  CU(cudaMemcpy(c->kxd_q, kxq.data(), sizeof(df64) * c->H, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(c->kyd_q, kyq.data(), sizeof(df64) * c->ny, cudaMemcpyHostToDevice));
+  HC_TRY(upload(c, c->kxd_q, kxq.data(), sizeof(df64) * c->H));
+  HC_TRY(upload(c, c->kyd_q, kyq.data(), sizeof(df64) * c->ny));
   if (c->dim == 3) {
     rc = put_tw(c->nz, c->twz_f, c->twz_d, c->twz_q, c->twz_x);
     if (rc) return rc;
@@ -715,9 +731,9 @@ int upload_tables(hc_ctx* c) {
     for (int k = 0; k < c->nz; ++k) kz[k] = xid(k, c->nz, c->grid.L[2]);
     std::vector<float> kzf(kz.begin(), kz.end());
     std::vector<df64> kzq(kz.begin(), kz.end());
-    CU(cudaMemcpy(c->kzd_d, kz.data(), sizeof(double) * c->nz, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(c->kzd_f, kzf.data(), sizeof(float) * c->nz, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(c->kzd_q, kzq.data(), sizeof(df64) * c->nz, cudaMemcpyHostToDevice));
+    HC_TRY(upload(c, c->kzd_d, kz.data(), sizeof(double) * c->nz));
+    HC_TRY(upload(c, c->kzd_f, kzf.data(), sizeof(float) * c->nz));
+    HC_TRY(upload(c, c->kzd_q, kzq.data(), sizeof(df64) * c->nz));
   }
   return HC_OK;
 }
@@ -1523,10 +1539,12 @@ long long graph_kernel_count(const hc_ctx* c, const hc::SolveState& h) {
 
 // Device handles the kernels drive: the context's own graph or a batch graph.
 int use_handles(hc_ctx* c, const Handles& h, cudaGraphConditionalHandle hgate = 0) {
-  unsigned long long v[4] = {h.inner, h.outer, hgate, h.first};
-  CU(cudaMemcpy(&c->st->h_inner, v, sizeof(v), cudaMemcpyHostToDevice));
-  unsigned long long w[4] = {h.mid, h.mid_inner, h.dec, h.again};
-  CU(cudaMemcpy(&c->st->h_mid, w, sizeof(w), cudaMemcpyHostToDevice));
+  // h_inner .. h_again of SolveState (h_cur is set by the kernels that open a loop)
+  const unsigned long long v[9] = {h.inner, h.outer, hgate, h.first, 0ull, h.mid, h.mid_inner,
+                                   h.dec, h.again};
+  static_assert(offsetof(hc::SolveState, h_again) - offsetof(hc::SolveState, h_inner) ==
+                    sizeof(v) - sizeof(v[0]), "one block of handles");
+  HC_TRY(upload(c, &c->st->h_inner, v, sizeof(v)));
   return HC_OK;
 }
 
@@ -3359,7 +3377,7 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
       cudaGetLastError();
       return fail(HC_ENOMEM);
     }
-    if (cudaMemset(b->dmem, 0, bytes) != cudaSuccess) return fail(HC_ECUDA);
+    if (cudaMemsetAsync(b->dmem, 0, bytes, b->stream) != cudaSuccess) return fail(HC_ECUDA);
     char* p = static_cast<char*>(b->dmem);
     hc::set_smem_limits_batch();
     for (auto& bc : b->cls) {
@@ -3378,8 +3396,9 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
         class_widen(gq, nb, 256);
       }
       for (int k : bc.members) recs.push_back(member_record(b->ctx[k], gf, gd, gq));
-      if (cudaMemcpy(bc.d_inst, recs.data(), recs.size() * sizeof(hc::BInst),
-                     cudaMemcpyHostToDevice) != cudaSuccess)
+      if (cudaMemcpyAsync(bc.d_inst, recs.data(), recs.size() * sizeof(hc::BInst),
+                          cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+          cudaStreamSynchronize(b->stream) != cudaSuccess)
         return fail(HC_ECUDA);
       bc.sh.gf = recs[0].gf;
       bc.sh.gfn = recs[0].gfn;

@@ -206,7 +206,11 @@ int hc_set_p(hc_ctx* ctx, const double* p, size_t count);
 
 /* Run nsteps passes of the loop body of Algorithm 1.  `last` (may be NULL)
  * receives the stats of the final step.  Returns HC_OK, or the first non-OK
- * step status (HC_ENOCONV: the steps still ran; HC_ENONFINITE: stopped). */
+ * step status (HC_ENOCONV: the steps still ran; HC_ENONFINITE: stopped).
+ * Contexts step side by side from threads and streams of their own.  The loop
+ * kernels of 2D solves up to about 10^6 points run together as far as their
+ * CTAs fit the device; a solve that finds no room waits for it on the device
+ * (hc_set_loop_wait, hc_loop_count). */
 int hc_step(hc_ctx* ctx, int nsteps, hc_step_stats* last);
 
 /* Algorithm 1 with its stopping rules (Section 2.5): run loop bodies until
@@ -253,6 +257,12 @@ int hc_get_state(hc_ctx* ctx, double* m_out, size_t m_count, double* p_out, size
  * an unfinished step, to be set anew.
  * Errors: HC_EINVAL (NULL, seconds negative, above 1e9 or NaN), HC_ECUDA. */
 int hc_set_loop_wait(hc_ctx* ctx, unsigned polls, double seconds);
+
+/* The context's loop kernels since its creation: launches that ran their solve
+ * to its end, the CG iterations in them, launches that found no room on the
+ * device beside other loops and launches given up at a barrier (both of which
+ * ran again).  Errors: HC_EINVAL (NULL), HC_ECUDA. */
+int hc_loop_count(hc_ctx* ctx, long long count[4]);
 
 /* --- Component entry points (each runs one part of the step on the GPU) --- */
 

@@ -97,6 +97,7 @@ def _load() -> C.CDLL:
         "hc_set_state": ([P, dp, C.c_size_t, dp, C.c_size_t], C.c_int),
         "hc_get_state": ([P, dp, C.c_size_t, dp, C.c_size_t], C.c_int),
         "hc_set_loop_wait": ([P, C.c_uint, C.c_double], C.c_int),
+        "hc_loop_count": ([P, C.POINTER(C.c_longlong)], C.c_int),
         "hc_gradient": ([P, dp, C.c_size_t], C.c_int),
         "hc_apply_operator": ([P, dp, dp, C.c_size_t], C.c_int),
         "hc_split_step": ([P], C.c_int),
@@ -144,6 +145,7 @@ hc_get_m = lib.hc_get_m
 hc_set_state = lib.hc_set_state
 hc_get_state = lib.hc_get_state
 hc_set_loop_wait = lib.hc_set_loop_wait
+hc_loop_count = lib.hc_loop_count
 hc_gradient = lib.hc_gradient
 hc_apply_operator = lib.hc_apply_operator
 hc_split_step = lib.hc_split_step
@@ -465,6 +467,12 @@ class Solver:
     def set_loop_wait(self, polls: int = 1 << 20, seconds: float = 120.0) -> None:
         """Limits of the loop kernels' waits (see hc_set_loop_wait)."""
         _check(hc_set_loop_wait(self.ctx, int(polls), float(seconds)), "hc_set_loop_wait")
+
+    def loop_count(self) -> dict:
+        """Launches of the loop kernels since creation (see hc_loop_count)."""
+        v = (C.c_longlong * 4)()
+        _check(hc_loop_count(self.ctx, v), "hc_loop_count")
+        return dict(zip(("ran", "iterations", "refused", "given_up"), v))
 
     def launch_count(self) -> int:
         v = C.c_longlong()

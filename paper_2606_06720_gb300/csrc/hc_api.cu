@@ -215,7 +215,7 @@ struct hc_ctx {
   cudaStream_t io_stream;               // hc_set_state / hc_get_state: copies beside p's transform
   cudaEvent_t io_ev[2 + 4];             // entry, copies done, and one per row chunk of p
   bool tuned;   // launch shapes set by hc_set_tuning
-  int loop_nt;  // CTA size of the CG loop kernel, 0: an iteration's kernels apart
+  hc::LoopShape loop;  // the CG loop kernel, nt = 0: an iteration's kernels apart
   // hc_set_loop_wait.  2^20 polls are most of a second: longer than any CTA of a loop takes to
   // arrive, unless another kernel holds the SM that it needs.
   unsigned loop_polls = 1u << 20;
@@ -1273,32 +1273,20 @@ int read_state(hc_ctx* c) {
   return loop_reported(c, c->stream);
 }
 
-// One loop kernel at a time on a device: the CTAs of two might each hold SMs that the other's
-// missing ones wait for.  Held by the calls that launch them until they have synchronised.
-std::mutex g_loop_mu[64];  // by device
-struct LoopGuard {
-  std::unique_lock<std::mutex> lk;
-  template <typename C>
-  explicit LoopGuard(const C* c) {
-    int dev = 0;
-    if (c->loop_nt && cudaGetDevice(&dev) == cudaSuccess) lk = std::unique_lock<std::mutex>(g_loop_mu[dev & 63]);
-  }
-};
-
-// The whole CG loop of a solve in one launch (loop_nt > 0).
+// The whole CG loop of a solve in one launch (loop.nt > 0).
 void cg_loop(hc_ctx* c) {
   if (c->refined)
-    hc::cg_loop_f32(c->gf, c->loop_nt, c->x32, c->r32, c->G32, c->G32 + c->ns, (const float*)c->m[0],
+    hc::cg_loop_f32(c->gf, c->loop, c->x32, c->r32, c->G32, c->G32 + c->ns, (const float*)c->m[0],
                     (const float*)c->m[1], (const float*)c->rf, c->st, c->stream);
   else
-    hc::cg_loop_fx(c->gd, c->loop_nt, c->p64, c->r64, c->G64, c->G64 + c->ns, (const double*)c->m[0],
+    hc::cg_loop_fx(c->gd, c->loop, c->p64, c->r64, c->G64, c->G64 + c->ns, (const double*)c->m[0],
                    (const double*)c->m[1], (const double*)c->rf, c->st, c->stream);
 }
 
 // Launch CG iterations in chunks until the device says done.
 int run_cg_host(hc_ctx* c, bool refined_inner) {
-  if (c->loop_nt) {
-    do {  // a launch that was given up ends nothing; the device counts the time
+  if (c->loop.nt) {
+    do {  // a launch refused or given up ends nothing; the device counts the time
       cg_loop(c);
       CU(cudaGetLastError());
       int rc = read_state(c);
@@ -1386,10 +1374,7 @@ int step_host(hc_ctx* c) {
 //            [HC_FP32_REFINED: IF(mid){double-float residual, WHILE(mid_inner){CG}}],
 //            WHILE(outer){IF(dec){fx64 residual}, IF(again){FP64 residual, WHILE(inner){CG}}} with the default
 //            residual switches, else WHILE(outer){FP64 residual, WHILE(inner){CG}}, split, step_end
-// link: nodes that the chain follows, and then its own last ones (chains with loop kernels, of
-// which one at a time may run).
-int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h,
-                std::vector<cudaGraphNode_t>* link = nullptr) {
+int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h) {
   cudaStream_t s = c->stream;
   Handles hh;
   cudaStreamCaptureStatus cs;
@@ -1420,7 +1405,7 @@ int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h,
   auto capture_iter = [&](cudaGraph_t body) -> int {
     CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0,
                                      cudaStreamCaptureModeThreadLocal));
-    if (c->loop_nt)
+    if (c->loop.nt)
       cg_loop(c);
     else if (c->refined)
       refined_iter(c);
@@ -1431,8 +1416,7 @@ int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h,
     return HC_OK;
   };
   std::vector<cudaGraphNode_t> tail;
-  CU(cudaStreamBeginCaptureToGraph(s, target, link ? link->data() : nullptr, nullptr,
-                                   link ? link->size() : 0, cudaStreamCaptureModeThreadLocal));
+  CU(cudaStreamBeginCaptureToGraph(s, target, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   hc::step_begin(c->st, (int)c->n, s);
   if (c->refined)
     first_resid32(c);
@@ -1500,9 +1484,8 @@ int build_chain(hc_ctx* c, cudaGraph_t target, Handles* h,
                                    cudaStreamCaptureModeThreadLocal));
   split_step(c);
   hc::step_end(c->st, c->refined, s);
-  rc = end_capture(target, tail);
-  if (rc) return rc;
-  if (link) *link = tail;
+  cudaGraph_t same = target;
+  CU(cudaStreamEndCapture(s, &same));
   *h = hh;
   return HC_OK;
 }
@@ -1736,7 +1719,7 @@ int build_pipe_graph(hc_ctx* c) {
     };
     auto capture_iter = [&](cudaGraph_t body) -> int {
       CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-      if (c->loop_nt)
+      if (c->loop.nt)
         cg_loop(c);
       else
         refined_iter(c);
@@ -2065,7 +2048,7 @@ int hc_create(hc_ctx** out, const hc_grid* grid, const hc_params* params, void* 
       fill_geo3<df64>(c, c->gq, c->rowq, c->twz_q, c->kzd_q, nullptr);
     }
     if (c->dim == 2)
-      c->loop_nt = c->refined ? hc::cg_loop_threads_f32(c->nx, c->ny) : hc::cg_loop_threads_fx(c->nx, c->ny);
+      c->loop = c->refined ? hc::cg_loop_shape_f32(c->nx, c->ny) : hc::cg_loop_shape_fx(c->nx, c->ny);
     hc::set_smem_limits_fx(c->refined);
     if (c->dim == 3) hc::set_smem_limits_3d_fx(c->refined);
     if (c->refined) {  // a plain FP64 context runs the fx64 kernels alone
@@ -2106,6 +2089,13 @@ int hc_set_loop_wait(hc_ctx* c, unsigned polls, double seconds) {
   c->loop_patience = seconds;
   const int rc = push_config(c);
   if (rc) return rc;
+  CU(cudaStreamSynchronize(c->stream));
+  return HC_OK;
+}
+
+int hc_loop_count(hc_ctx* c, long long count[4]) {
+  if (!c || !count) return HC_EINVAL;
+  CU(cudaMemcpyAsync(count, c->st->loop_count, 4 * sizeof(long long), cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
   return HC_OK;
 }
@@ -2508,8 +2498,9 @@ int hc_get_state(hc_ctx* c, double* m_out, size_t m_count, double* p_out, size_t
   return HC_OK;
 }
 
-// nsteps > 0 steps; the caller holds the LoopGuard (exported calls take it, bodies do not).
-static int step_body(hc_ctx* c, int nsteps, hc_step_stats* last) {
+int hc_step(hc_ctx* c, int nsteps, hc_step_stats* last) {
+  if (!c || nsteps < 0) return HC_EINVAL;
+  if (nsteps == 0) return HC_OK;
   hc::reset_accum(c->st, c->stream);
   c->launches += 1;
   if (pipe_on(c, nsteps)) {
@@ -2546,13 +2537,6 @@ static int step_body(hc_ctx* c, int nsteps, hc_step_stats* last) {
   return c->st_host->first_bad;
 }
 
-int hc_step(hc_ctx* c, int nsteps, hc_step_stats* last) {
-  if (!c || nsteps < 0) return HC_EINVAL;
-  if (nsteps == 0) return HC_OK;
-  LoopGuard guard(c);
-  return step_body(c, nsteps, last);
-}
-
 static void gradient3(hc_ctx* c) {
   const size_t n = c->n;
   if (c->refined) {
@@ -2584,7 +2568,6 @@ static void gradient3(hc_ctx* c) {
 int hc_run(hc_ctx* c, int max_steps, double eps, int stop_on_energy, int* steps_done,
            hc_step_stats* last) {
   if (!c || max_steps < 0) return HC_EINVAL;
-  LoopGuard guard(c);
   if (steps_done) *steps_done = 0;
   const int forced = c->prm.diagnostics ? 0 : 1;
   if (forced) {
@@ -2999,7 +2982,7 @@ int adjoint_t(hc_ctx* c, hc::Geo<T>& g, int nsteps, int every, const double* lam
                          a.cpk + kMsums * (k / every));
       if (rc) return rc;
     }
-    rc = step_body(c, 1, nullptr);
+    rc = hc_step(c, 1, nullptr);
     if (rc == HC_ENOCONV) status = status ? status : rc;
     else if (rc) return rc;
   }
@@ -3023,7 +3006,7 @@ int adjoint_t(hc_ctx* c, hc::Geo<T>& g, int nsteps, int every, const double* lam
     for (int k = k0; k < k1; ++k) {
       rc = save_state<T>(c, a.segm + 2 * n * (k - k0), nullptr, a.segk + kMsums * (k - k0));
       if (rc) return rc;
-      rc = step_body(c, 1, nullptr);
+      rc = hc_step(c, 1, nullptr);
       if (rc && rc != HC_ENOCONV) return rc;
       CU(cudaMemcpyAsync(a.segp + ns * (k - k0), c->p64, sizeof(cx<double>) * ns,
                          cudaMemcpyDeviceToDevice, s));
@@ -3090,7 +3073,6 @@ int hc_adjoint(hc_ctx* c, int nsteps, int every, const double* lamT, double* dc2
   if (!c || !lamT || nsteps < 0 || every < 1) return HC_EINVAL;
   if (c->df || c->dim != 2 || c->gen) return HC_ENOTSUP;
   if (workspace && (reinterpret_cast<uintptr_t>(workspace) % kAlign)) return HC_EINVAL;
-  LoopGuard guard(c);
   size_t need = 0;
   int rc = hc_adjoint_workspace_size(c, nsteps, every, &need);
   if (rc) return rc;
@@ -3152,7 +3134,6 @@ struct hc_batch {
   std::vector<Handles> h;     // per-context chains
   std::vector<int> cls_of;    // class of each context, -1: its own chain
   std::vector<BatchClass> cls;
-  int loop_nt = 0;            // some chain has loop kernels
   void* dmem;                 // device memory of the classes
   cudaStream_t stream;
   cudaStream_t cap;
@@ -3423,7 +3404,13 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
       return fail(rc);
     }
   }
-  std::vector<cudaGraphNode_t> link;
+  // Refined chains whose loops would take the device in turns run the separate kernels, which
+  // run side by side and give the same results (double-float, four steps, ms, loops / separate:
+  // two of 1024^2 9.9 / 9.0, four 19.4 / 15.8; four of 1024x512 12.0 / 8.3).  FP64 chains keep
+  // their loops: the separate kernels sum in another order.
+  int alone = 0;
+  for (int i = 0; i < count; ++i)
+    if (b->cls_of[i] < 0 && b->ctx[i]->loop.nt && !hc::cg_loop_shares(b->ctx[i]->loop)) alone += 1;
   for (int i = 0; i < count; ++i) {
     if (b->cls_of[i] >= 0) continue;
     hc_ctx* c = b->ctx[i];
@@ -3434,8 +3421,10 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
     cudaStream_t keep = c->stream;
     long long before = c->launches;
     c->stream = b->cap;
-    int rc = build_chain(c, graph, &b->h[i], c->loop_nt ? &link : nullptr);
-    b->loop_nt = b->loop_nt ? b->loop_nt : c->loop_nt;
+    const hc::LoopShape loop = c->loop;
+    if (c->refined && alone > 1 && !hc::cg_loop_shares(loop)) c->loop = hc::LoopShape{};
+    int rc = build_chain(c, graph, &b->h[i]);
+    c->loop = loop;
     c->stream = keep;
     c->launches = before;
     if (rc) {
@@ -3456,7 +3445,6 @@ int hc_batch_create(hc_batch** out, hc_ctx* const* ctxs, int count, void* stream
 
 int hc_batch_step(hc_batch* b, int nsteps, hc_step_stats* stats) {
   if (!b || nsteps < 0) return HC_EINVAL;
-  LoopGuard guard(b);
   if (nsteps == 0) return HC_OK;
   const int n = (int)b->ctx.size();
   for (int i = 0; i < n; ++i) {

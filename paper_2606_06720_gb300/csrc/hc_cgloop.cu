@@ -19,6 +19,44 @@
 
 namespace hc {
 
+// Loops of several callers on one device (threads, streams, the chains of a batch).  Two loops
+// whose CTAs each hold SMs that the other's missing ones wait for would both stand still, so the
+// CTAs that wait at a time must all fit.  They are counted on the device, solve by solve: a
+// one-thread kernel before the loop claims its room or, where there is none, refuses the launch,
+// which then returns at once and is tried again.  (A lock held by the host call, the rule before,
+// kept callers apart for all steps of a call: eight solvers of 64^2 FP64 on eight threads 28 ms for
+// four steps, sixteen in a batch 55, now 10 and 8; with separate kernels, FP64 passes 24 and 23.
+// The claim inside the loop kernel saved its launch but changed the code of the FP64 loop: 64^2
+// 30.1 -> 31.5 us an iteration.)
+//
+// What fits: a CTA of a kernel of which `per` fit an SM takes 1/per of every resource at most,
+// counted in sixteenths, u = 16 / per (per rounded down to a power of two, 16 at most).  An SM has
+// room for it unless more than 16 - u sixteenths are taken, and with u_min the smallest u about
+// that means 16 - u + u_min at least.  So each of the CTAs has an SM to go to if all of them
+// together are no more than the SMs, or take no more than SMs * (16 - u_max + u_min) sixteenths.
+// (An SM's free registers may lie in pieces; a barrier whose CTA finds no place is then given up
+// and the launch repeated.  In the crowds of the tests none was.)
+// g_loop_room holds the CTAs per u = 1, 2, 4, 8, 16 in fields of 12 bits (2432 CTAs at most), and
+// in bit 60 that a solve has waited for long (kLoopTurnNs): then only such solves enter, so that
+// one that needs the whole device gets it.
+constexpr int kRoomBits = 12;
+constexpr unsigned long long kRoomTurn = 1ull << 60, kLoopTurnNs = 2000000ull;
+constexpr unsigned kLoopPauseNs = 4000;  // after a refusal, before the next try
+__device__ unsigned long long g_loop_room;
+
+__host__ __device__ inline bool room_ok(unsigned long long room, int sms) {
+  int ctas = 0, units = 0, lo = 0, hi = 0;
+  for (int k = 0; k < 5; ++k) {
+    const int n = (int)(room >> (k * kRoomBits)) & ((1 << kRoomBits) - 1);
+    if (!n) continue;
+    if (!ctas) lo = 1 << k;
+    hi = 1 << k;
+    ctas += n;
+    units += n << k;
+  }
+  return ctas <= sms || units <= sms * (16 - hi + lo);
+}
+
 // The grid barriers of one launch.  The launch is cooperative, so every CTA is resident and
 // arrives; a wait is bounded all the same (st->loop_polls polls), because another stream's
 // kernel may hold an SM that a CTA waits for.  A barrier completes for every CTA or for none: one
@@ -123,6 +161,7 @@ __device__ __forceinline__ void loop_finish(SolveState* st, const LoopCg& k, int
   st->rho = k.rho;
   st->it = k.it;
   st->total_it += its;
+  st->loop_count[1] += its;
   if (k.status) st->status = k.status;
   st->first = 0;
   st->done = 1;
@@ -138,29 +177,63 @@ __device__ __forceinline__ bool loop_gave_up(SolveState* st) {
   }
   return true;
 }
-// The last CTA to leave re-arms the barriers.  A launch that was given up leaves the solve as it
-// found it, so it runs again (the WHILE node's next turn, or the host's next launch), until
-// st->loop_patience ns after the first one.
-__device__ __forceinline__ void loop_leave(SolveState* st, bool live) {
+// A launch that was refused (2) or given up (3): one thread.  The solve is as it was, so it runs
+// again (the WHILE node's next turn, or the host's next launch), until st->loop_patience ns after
+// the first such launch.
+__device__ __forceinline__ void loop_lost(SolveState* st, int how) {
+  st->loop_count[how] += 1;
+  unsigned long long now;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+  if (!st->loop_since) st->loop_since = now;
+  if (now - st->loop_since >= st->loop_patience) {
+    st->loop_since = 0ull;
+    st->loop_turn = 0;
+    st->loop_timeout = 1;
+    st->done = 1;
+    if (st->graph_mode) cudaGraphSetConditional(st->h_cur, 0u);
+  } else if (now - st->loop_since >= kLoopTurnNs) {
+    st->loop_turn = 1;
+  }
+}
+// The last CTA to leave re-arms the barriers and gives the launch's room back.
+__device__ __forceinline__ void loop_leave(SolveState* st, const LoopRoom& room, bool live) {
   if (threadIdx.x != 0) return;
   unsigned t;
   asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(&st->loop_exit) : "memory");
   if (t != gridDim.x - 1) return;
   st->loop_exit = 0u;
   st->loop_bar = 0u;
+  if (room.need) atomicAdd(&g_loop_room, 0ull - room.need);
   if (live) {
     st->loop_since = 0ull;
-    return;
+    st->loop_turn = 0;
+    st->loop_count[0] += 1;
+  } else {
+    loop_lost(st, 3);
   }
-  unsigned long long now;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-  if (!st->loop_since) st->loop_since = now;
-  if (now - st->loop_since >= st->loop_patience) {
-    st->loop_since = 0ull;
-    st->loop_timeout = 1;
-    st->done = 1;
-    if (st->graph_mode) cudaGraphSetConditional(st->h_cur, 0u);
+}
+
+// One thread, before a loop kernel: room for it, or a refusal.  The swap assumes an idle device at
+// first; each failed one is another solve's.
+__global__ void k_loop_claim(SolveState* st, LoopRoom room) {
+  if (st->done || st->loop_timeout) return;
+  const bool turn = st->loop_turn != 0;
+  unsigned long long cur = 0ull;
+  for (int i = 0; i < 256; ++i) {
+    const unsigned long long next = (turn ? cur & ~kRoomTurn : cur) + room.need;
+    const bool fits = room_ok(next & ~kRoomTurn, room.sms) && (turn || !(cur & kRoomTurn));
+    if (!fits && i > 0) break;
+    const unsigned long long old = atomicCAS(&g_loop_room, cur, fits ? next : cur);
+    if (old == cur && fits) {
+      st->loop_refused = 0;
+      return;
+    }
+    cur = old;
   }
+  st->loop_refused = 1;
+  loop_lost(st, 2);
+  if (st->loop_turn) atomicOr(&g_loop_room, kRoomTurn);
+  __nanosleep(kLoopPauseNs);
 }
 
 // Sum over the CTAs of K values (K doubles each at p[cta * stride]), in every thread.
@@ -193,10 +266,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
                                                         const cx<float>* r, cx<float>* Gx,
                                                         cx<float>* Gy, const float* mx,
                                                         const float* my, const float* rf,
-                                                        SolveState* st, int row_sums) {
+                                                        SolveState* st, LoopRoom room, int row_sums) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (st->done) return;  // nothing writes it before every CTA has passed a barrier
-  if (loop_gave_up(st)) return;
+  if (loop_gave_up(st) || st->loop_refused) return;
   using C = cx<float>;
   C* sm = reinterpret_cast<C*>(smem_raw);
   const int nt = blockDim.x, t = threadIdx.x, H = g.H;
@@ -357,7 +430,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_loop_f32(Geo<float> g, cx<float>
     for (int s = 0; s < 8; ++s) x[cmi(g, c.j + s * c.NY8, c.kx)] = xs[(size_t)s * nt];
   }
   if (live && blockIdx.x == 0 && t == 0) loop_finish(st, k, k.it - it0);
-  loop_leave(st, live);
+  loop_leave(st, room, live);
 }
 
 // Plain FP64 solve (fx64 transforms, row-major x and r).  A warp's instructions are what
@@ -372,10 +445,10 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
                                                         const cx<double>* r, cx<fx64>* Gx,
                                                         cx<fx64>* Gy, const fx64* mx,
                                                         const fx64* my, const fx64* rf,
-                                                        SolveState* st) {
+                                                        SolveState* st, LoopRoom room) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (st->done) return;  // nothing writes it before every CTA has passed a barrier
-  if (loop_gave_up(st)) return;
+  if (loop_gave_up(st) || st->loop_refused) return;
   using C = cx<fx64>;
   C* sm = reinterpret_cast<C*>(smem_raw);
   const int nt = blockDim.x, hn = nt >> 1, t = threadIdx.x, H = g.H;
@@ -550,7 +623,7 @@ __global__ void __launch_bounds__(256, 1) k_cg_loop_fx(Geo<fx64> g, cx<double>* 
     for (int i = 0; i < 4; ++i) x[(size_t)(j + (4 * f + i) * NY8) * H + col] = xv[i];
   }
   if (live && blockIdx.x == 0 && t == 0) loop_finish(st, k, k.it - it0);
-  loop_leave(st, live);
+  loop_leave(st, room, live);
 }
 
 static inline size_t loop_smem(int nt, int rpc, int nx) {
@@ -574,9 +647,9 @@ static int loop_threads(int nx, int ny, int per) {
   return tc > 32 || tc > nx / 2 ? 0 : nt;
 }
 
-// All CTAs of the loop kernel resident at once on this device.
+// The shape of a loop of `grid` CTAs, or none where this device cannot hold them all.
 template <typename K>
-static bool loop_fits(K kernel, int nt, size_t smem, long long grid) {
+static LoopShape loop_shape(K kernel, int nt, size_t smem, long long grid) {
   allow_smem(kernel);
   int dev = 0, sms = 0, coop = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -584,9 +657,14 @@ static bool loop_fits(K kernel, int nt, size_t smem, long long grid) {
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, nt, smem) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return LoopShape{};
   }
-  return coop && (long long)per * sms >= grid;
+  if (!coop || per < 1) return LoopShape{};
+  int k = 4;  // a CTA takes 2^k sixteenths of an SM
+  while (k > 0 && per >= 2 << (4 - k)) --k;
+  // a single CTA waits for nobody
+  const LoopRoom room{grid > 1 ? (unsigned long long)grid << (k * kRoomBits) : 0ull, sms};
+  return room_ok(room.need, sms) ? LoopShape{nt, room} : LoopShape{};
 }
 
 // Geometry of the loop's passes: per values a thread.
@@ -600,38 +678,44 @@ static Geo<T> loop_geo(const Geo<T>& g0, int nt, int per) {
   return g;
 }
 
-int cg_loop_threads_f32(int nx, int ny) {
+bool cg_loop_shares(const LoopShape& sh) { return room_ok(2 * sh.room.need, sh.room.sms); }
+
+LoopShape cg_loop_shape_f32(int nx, int ny) {
   const int nt = loop_threads(nx, ny, 16);
-  if (!nt) return 0;
+  if (!nt) return LoopShape{};
   const long long grid = (long long)nx * ny / (16 * nt);
-  const size_t smem = loop_smem(nt, 16 * nt / nx, nx);
-  return loop_fits(nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>, nt, smem, grid) ? nt : 0;
+  return loop_shape(nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>, nt,
+                    loop_smem(nt, 16 * nt / nx, nx), grid);
 }
-int cg_loop_threads_fx(int nx, int ny) {
+LoopShape cg_loop_shape_fx(int nx, int ny) {
   const int nt = loop_threads(nx, ny, 8);
   // 512 threads would have to fit 128 registers: 1024x512 108 us an iteration either way,
   // 32x2048 (16 CTAs) 110 -> 129
-  if (!nt || nt > 256) return 0;
-  const long long grid = (long long)nx * ny / (8 * nt);
-  return loop_fits(k_cg_loop_fx, nt, loop_smem_fx(nt), grid) ? nt : 0;
+  if (!nt || nt > 256) return LoopShape{};
+  return loop_shape(k_cg_loop_fx, nt, loop_smem_fx(nt), (long long)nx * ny / (8 * nt));
 }
 
-void cg_loop_f32(const Geo<float>& g0, int nt, cx<float>* x, const cx<float>* r, cx<float>* Gx,
-                 cx<float>* Gy, const float* mx, const float* my, const float* rf, SolveState* st,
-                 cudaStream_t s) {
+void cg_loop_f32(const Geo<float>& g0, const LoopShape& sh, cx<float>* x, const cx<float>* r,
+                 cx<float>* Gx, cx<float>* Gy, const float* mx, const float* my, const float* rf,
+                 SolveState* st, cudaStream_t s) {
+  const int nt = sh.nt;
   Geo<float> g = loop_geo(g0, nt, 16);
+  LoopRoom room = sh.room;
   int row_sums = g0.rpc < 2;
-  void* args[] = {&g, &x, &r, &Gx, &Gy, &mx, &my, &rf, &st, &row_sums};
+  void* args[] = {&g, &x, &r, &Gx, &Gy, &mx, &my, &rf, &st, &room, &row_sums};
+  if (room.need) k_loop_claim<<<1, 1, 0, s>>>(st, room);
   cudaLaunchCooperativeKernel((const void*)(nt <= 256 ? k_cg_loop_f32<256> : k_cg_loop_f32<512>),
                               dim3(g.H >> g.ltc), dim3(nt), args, loop_smem(nt, g.rpc, g.nx), s);
 }
-void cg_loop_fx(const Geo<double>& g0, int nt, cx<double>* x, const cx<double>* r, cx<double>* Gx,
-                cx<double>* Gy, const double* mx, const double* my, const double* rf,
-                SolveState* st, cudaStream_t s) {
-  Geo<fx64> g = loop_geo(as_fx(g0), nt, 8);
-  void* args[] = {&g, &x, &r, &Gx, &Gy, &mx, &my, &rf, &st};
-  cudaLaunchCooperativeKernel((const void*)k_cg_loop_fx,
-                              dim3(g.H >> g.ltc), dim3(nt), args, loop_smem_fx(nt), s);
+void cg_loop_fx(const Geo<double>& g0, const LoopShape& sh, cx<double>* x, const cx<double>* r,
+                cx<double>* Gx, cx<double>* Gy, const double* mx, const double* my,
+                const double* rf, SolveState* st, cudaStream_t s) {
+  Geo<fx64> g = loop_geo(as_fx(g0), sh.nt, 8);
+  LoopRoom room = sh.room;
+  void* args[] = {&g, &x, &r, &Gx, &Gy, &mx, &my, &rf, &st, &room};
+  if (room.need) k_loop_claim<<<1, 1, 0, s>>>(st, room);
+  cudaLaunchCooperativeKernel((const void*)k_cg_loop_fx, dim3(g.H >> g.ltc), dim3(sh.nt), args,
+                              loop_smem_fx(sh.nt), s);
 }
 
 }  // namespace hc

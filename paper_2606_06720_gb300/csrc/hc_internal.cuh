@@ -203,10 +203,13 @@ struct SolveState {
   unsigned int ticket[8];    // last-CTA tickets, one per reduction site
   unsigned int loop_bar;     // CG loop kernel: its grid barriers' word (0 between launches)
   unsigned int loop_exit;    // CTAs that have left it
+  int loop_refused;          // its launch found no room on the device
+  int loop_turn;             // its solve has waited for long
   unsigned int loop_polls;   // polls of one barrier before the launch is given up
   int loop_timeout;          // a solve was given up for good (until the host has read it)
-  unsigned long long loop_patience;  // ns for which launches that were given up are repeated
+  unsigned long long loop_patience;  // ns for which launches refused or given up are repeated
   unsigned long long loop_since;     // global timer at the first of them, 0: none
+  long long loop_count[4];   // since creation: its launches that ran, their iterations, refused, given up
   // Diagnostics of Section 2.5, accumulated by the split step when diag != 0.
   // A step solves p[m^k] and so evaluates E_h(m^k) with its own pressure.
   double dsum[3];            // running step: sum r|g|^2, sum (m.g)^2, sum |m|^(2 gamma) (gamma = 0: sum ln|m|); m = m^k, g = grad p[m^k]
@@ -241,6 +244,19 @@ struct SolveState {
 };
 
 // Values the host changes between steps (tolerances, caps, r statistics).
+// What a CG loop kernel takes of its device (hc_cgloop.cu): its CTAs, in the field of their size,
+// of the count that all such kernels share (0: a single CTA, not counted), and the device's SMs.
+struct LoopRoom {
+  unsigned long long need = 0;
+  int sms = 0;
+};
+// CTA size of the loop kernel for a grid, 0 where the separate kernels are the better ones or
+// this device does not hold all its CTAs, and its room.
+struct LoopShape {
+  int nt = 0;
+  LoopRoom room;
+};
+
 struct SolveConfig {
   double outer_thresh2_rel;  // cg_rtol^2 (multiplied by ||S||^2 on the device)
   double inner_rtol2;
@@ -607,16 +623,16 @@ void col_div_upd(const Geo<double>& g, const cx<double>* Qx, const cx<double>* Q
                  cx<double>* x, cx<double>* r, SolveState* st, cudaStream_t s);
 void set_smem_limits_fx(int refined);
 // The CG loop of a 2D solve as one cooperative kernel (hc_cgloop.cu): FP32 inner solves and
-// plain FP64 ones (fx64).  cg_loop_threads_*: its CTA size for a grid, 0 where the separate
-// kernels are the better ones or this device does not keep all its CTAs resident.
-int cg_loop_threads_f32(int nx, int ny);
-int cg_loop_threads_fx(int nx, int ny);
-void cg_loop_fx(const Geo<double>& g, int nt, cx<double>* x, const cx<double>* r, cx<double>* Gx,
-                cx<double>* Gy, const double* mx, const double* my, const double* rf,
-                SolveState* st, cudaStream_t s);
-void cg_loop_f32(const Geo<float>& g, int nt, cx<float>* x, const cx<float>* r, cx<float>* Gx,
-                 cx<float>* Gy, const float* mx, const float* my, const float* rf, SolveState* st,
-                 cudaStream_t s);
+// plain FP64 ones (fx64).
+LoopShape cg_loop_shape_f32(int nx, int ny);
+LoopShape cg_loop_shape_fx(int nx, int ny);
+bool cg_loop_shares(const LoopShape& sh);  // two such loops have room side by side
+void cg_loop_fx(const Geo<double>& g, const LoopShape& sh, cx<double>* x, const cx<double>* r,
+                cx<double>* Gx, cx<double>* Gy, const double* mx, const double* my,
+                const double* rf, SolveState* st, cudaStream_t s);
+void cg_loop_f32(const Geo<float>& g, const LoopShape& sh, cx<float>* x, const cx<float>* r,
+                 cx<float>* Gx, cx<float>* Gy, const float* mx, const float* my, const float* rf,
+                 SolveState* st, cudaStream_t s);
 // Lagged certification (2D refined steps): the FP64 certifying residual of
 // pressure p with the FP32 m, r it was solved with (sc: the certifying state,
 // skipped when nothing is pending); the commit after a lagged step (copies

@@ -78,3 +78,80 @@ def test_adjoint_returns_and_leaves_the_device_free(hc, precision):
         assert same(both[0], alone) and same(both[1], step_alone)
     a.close()
     b.close()
+
+
+# (size, precision, how many): loops that fit an SM together in twos, fours and eights, loops that
+# take the device for themselves, and more of each than fit at a time.
+CROWDS = [
+    [((64, 64), "fp64")] * 16,
+    [((256, 256), "fp64")] * 6,
+    [((256, 256), "fp32_refined")] * 8,
+    [((512, 512), "fp32_refined"), ((512, 512), "fp64"), ((64, 64), "fp64"), ((128, 64), "fp64"),
+     ((32, 8), "fp64"), ((256, 128), "fp32_refined"), ((512, 512), "fp32_refined_df"),
+     ((1024, 512), "fp32_refined")],
+]
+
+
+@pytest.mark.parametrize("crowd", range(len(CROWDS)))
+def test_crowd_on_threads(hc, crowd):
+    """Solvers stepped at once, each from its thread on its stream: as each is alone, bit for bit,
+    whether its loops find room at once or have to wait for it."""
+    members = [make(hc, n, precision, k) for k, (n, precision) in enumerate(CROWDS[crowd])]
+    alone = [stepped(*x) for x in members]
+    for _ in range(3):
+        out = in_threads([lambda x=x: stepped(*x) for x in members])
+        assert all(same(a, b) for a, b in zip(out, alone))
+    for s, _, _ in members:
+        s.close()
+
+
+# Loops that share the device, and refined ones that would take it in turns: those run the separate
+# kernels in a batch, with the same results.
+@pytest.mark.parametrize("n, precision, count", [((64, 64), "fp64", 16), ((256, 256), "fp64", 6),
+                                                 ((512, 512), "fp32_refined_df", 3),
+                                                 ((1024, 512), "fp32_refined_df", 3)])
+def test_crowd_in_a_batch(hc, n, precision, count):
+    """Contexts outside a size class, each on a chain of its own."""
+    members = [make(hc, n, precision, k) for k in range(count)]
+    alone = [stepped(*x) for x in members]
+    with hc.Batch([s for s, _, _ in members]) as b:
+        assert b.classes() == (0, 0)
+        for _ in range(3):
+            for s, m0, p0 in members:
+                s.set_state(m0, p0)
+            assert all(st.status == 0 for st in b.step(4))
+            assert all(same(s.get_state(), w) for (s, _, _), w in zip(members, alone))
+    for s, _, _ in members:
+        s.close()
+
+
+def test_large_loop_is_not_starved(hc):
+    """A solver whose loops need every SM, beside eight small ones that never rest: it returns
+    while they still step."""
+    big, mb, pb = make(hc, (512, 512), "fp64", 0)
+    small = [make(hc, (64, 64), "fp64", k) for k in range(1, 9)]
+    want = stepped(big, mb, pb)
+    for x in small:
+        stepped(*x)
+    stop = threading.Event()
+    ran = [0] * len(small)
+
+    def keep(k):
+        while not stop.is_set():
+            small[k][0].step(1)
+            ran[k] += 1
+
+    threads = [threading.Thread(target=keep, args=(k,), daemon=True) for k in range(len(small))]
+    for t in threads:
+        t.start()
+    try:
+        got = in_threads([lambda: stepped(big, mb, pb)])[0]
+    finally:
+        stop.set()
+        for t in threads:
+            t.join(LIMIT)
+    assert not any(t.is_alive() for t in threads)
+    assert same(got, want) and min(ran) > 0
+    big.close()
+    for s, _, _ in small:
+        s.close()

@@ -71,8 +71,9 @@ BYTES_PER_POINT = {
         "split_c2r": 32,
     },
 }
-FP64_KERNELS = {"fp32_refined": {"res_grad", "res_apply", "res_div", "res_ypass"},
-                "fp64": set(BYTES_PER_POINT["fp64"])}
+# The refinement residual as it usually runs: fixed-point transforms, bound by the integer
+# pipes' issue rate; neither HBM nor the FP64 FMA peak is its roof.
+INT_KERNELS = {"res_grad", "res_apply", "res_div", "res_ypass"}
 # Double-float kernels (the mid-step residual of the FP64-refined path): bound
 # by the FP32 pipes running the emulated arithmetic; no roofline fraction.
 DF_KERNELS = {"mid_grad", "mid_apply", "mid_div", "mid_ypass"}
@@ -162,24 +163,22 @@ def fft_flops_per_point_3d(kernel: str, nx: int, ny: int, nz: int) -> float:
     }[kernel]
 
 
-def kernel_table(s, counts: dict, bytes_pp: dict, flops_pp, fp64_names: set, npts: int,
-                 reps: int, hbm_peak: float, fp64_peak: float) -> dict:
+def kernel_table(s, counts: dict, bytes_pp: dict, flops_pp, npts: int, reps: int,
+                 hbm_peak: float) -> dict:
     """Per-kernel CUDA-event durations (hc_time_kernel: back-to-back launches
-    on the same data) with algorithmic GB/s and TFLOP/s and the fraction of
-    the kernel's roof: HBM for the FP32 kernels, the measured FP64 FMA peak
-    for the FP64 ones."""
+    on the same data) with algorithmic GB/s and TFLOP/s and, for the FP32
+    kernels, the fraction of HBM's measured rate."""
     kernels = {}
     for name, cnt in counts.items():
         kms = s.time_kernel(name, reps=reps)
         gbs = bytes_pp[name] * npts / (kms / 1e3) / 1e9
         tfl = flops_pp(name) * npts / (kms / 1e3) / 1e12
-        is64 = name in fp64_names
+        isint = name in INT_KERNELS
         isdf = name in DF_KERNELS
         kernels[name] = {"ms": kms, "launches_per_step": cnt, "ms_per_step": kms * cnt,
                          "alg_GBs": gbs, "alg_TFLOPs": tfl,
-                         "bound": "alu-df" if isdf else ("alu" if is64 else "hbm"),
-                         "frac": None if isdf else ((tfl / fp64_peak) if is64
-                                                    else (gbs / hbm_peak))}
+                         "bound": "alu-df" if isdf else ("alu-int" if isint else "hbm"),
+                         "frac": None if isdf or isint else gbs / hbm_peak}
     return kernels
 
 
@@ -456,7 +455,7 @@ def run_convergence(P, W, args, dev, job_rate) -> dict:
 
 
 # ----------------------------------------------------------------- 3D leg
-def run_3d(P, W, args, dev, barrier, job_rate, hbm_peak, hbm_src, fp64_peak) -> dict:
+def run_3d(P, W, args, dev, barrier, job_rate, hbm_peak, hbm_src) -> dict:
     """The 256^3 source/sink workload (r = 0.1, sigma 0.05 pair at
     (0.3,0.5,0.5)/(0.7,0.5,0.5), m0 ~ U[0,0.5], c = 25, D = 0.03,
     gamma = 0.75, dt = 5e-4), FP32 + FP64 refinement to 1e-8, graph mode."""
@@ -496,8 +495,7 @@ def run_3d(P, W, args, dev, barrier, job_rate, hbm_peak, hbm_src, fp64_peak) -> 
         counts.update({"mid_grad": mid, "mid_ypass": 2 * mid, "mid_apply": mid, "mid_div": mid})
     kernels = kernel_table(s, counts, BYTES_PER_POINT_3D,
                            lambda k: fft_flops_per_point_3d(k, *w.n),
-                           FP64_KERNELS["fp32_refined"], npts, max(3, args.kernel_reps // 3),
-                           hbm_peak, fp64_peak)
+                           npts, max(3, args.kernel_reps // 3), hbm_peak)
     s.close()
     # dominant FP32 kernel of the CG iteration against HBM
     fp32 = [k for k in kernels if kernels[k]["bound"] == "hbm"]
@@ -731,25 +729,17 @@ def run_gb300(args) -> None:
     if mid_per_step > 0:
         counts.update({"mid_grad": mid_per_step, "mid_apply": mid_per_step, "mid_div": mid_per_step})
     kernels = kernel_table(s, counts, BYTES_PER_POINT["fp32_refined"],
-                           lambda k: fft_flops_per_point(k, *w.n), FP64_KERNELS["fp32_refined"],
-                           npts, args.kernel_reps, hbm_peak, fp64_peak)
+                           lambda k: fft_flops_per_point(k, *w.n), npts, args.kernel_reps,
+                           hbm_peak)
     bytes_step = sum(BYTES_PER_POINT["fp32_refined"][k] * npts * c for k, c in counts.items())
-    dom = max(kernels, key=lambda k: kernels[k]["ms_per_step"])
+    dom = max((k for k in kernels if kernels[k]["bound"] == "hbm"),
+              key=lambda k: kernels[k]["ms_per_step"])
     dk = kernels[dom]
     traffic = NCU_TRAFFIC_2048.get(dom) if w.n == (2048, 2048) else None
-    if dk["bound"] == "alu":
-        roofline = {"bound": "alu", "kernel": dom, "achieved": dk["alg_TFLOPs"],
-                    "peak": fp64_peak, "unit": "TFLOP/s", "frac": dk["frac"],
-                    "traffic": traffic,
-                    "peak_source": "measured: FP64 FMA throughput of this GPU in this run "
-                                   "(hc_fp64_fma_peak: fastest of 10 launches; FMA = 2 flops); "
-                                   "nominal 1.25",
-                    "alg_bytes": BYTES_PER_POINT["fp32_refined"][dom] * npts}
-    else:
-        roofline = {"bound": "hbm", "kernel": dom, "achieved": dk["alg_GBs"], "peak": hbm_peak,
-                    "unit": "GB/s", "frac": dk["frac"], "traffic": traffic,
-                    "peak_source": hbm_src,
-                    "alg_bytes": BYTES_PER_POINT["fp32_refined"][dom] * npts}
+    roofline = {"bound": "hbm", "kernel": dom, "achieved": dk["alg_GBs"], "peak": hbm_peak,
+                "unit": "GB/s", "frac": dk["frac"], "traffic": traffic,
+                "peak_source": hbm_src,
+                "alg_bytes": BYTES_PER_POINT["fp32_refined"][dom] * npts}
     share = dk["ms_per_step"] / (ms / K)
     roofline["share_of_step"] = share
 
@@ -954,7 +944,7 @@ def run_gb300(args) -> None:
     # ---- 3D: the 256^3 source/sink problem (d = 3), FP32 + FP64 refinement
     three_d = None
     if not args.no_3d:
-        three_d = run_3d(P, W, args, dev, barrier, job_rate, hbm_peak, hbm_src, fp64_peak)
+        three_d = run_3d(P, W, args, dev, barrier, job_rate, hbm_peak, hbm_src)
 
     # ---- equal accuracy (every rank runs its own replica): the refined path
     # and the plain FP64 path at each candidate tolerance, 100 steps from m0,
@@ -997,7 +987,7 @@ def run_gb300(args) -> None:
         for name in ("cg_apply", "cg_div", "cg_grad"):
             kms = s64.time_kernel(name, reps=max(3, args.kernel_reps // 5))
             tfl = fft_flops_per_point(name, *w.n) * npts / (kms / 1e3) / 1e12
-            k64[name] = {"ms": kms, "alg_TFLOPs": tfl, "frac_of_fp64_peak": tfl / fp64_peak}
+            k64[name] = {"ms": kms, "alg_TFLOPs": tfl}  # fixed-point transforms: no FP64 roof
         s64.close()
         fp64 = {"value": v64, "unit": UNIT, "ms_per_step": ms64 / K64, "steps": K64,
                 "cg_rtol": fp64_rtol, "cg_iters_per_step": st64.total_cg_iters / K64,

@@ -316,19 +316,22 @@ int hc_get_tuning(const hc_ctx* ctx, hc_tuning* out);
 int hc_set_tuning(hc_ctx* ctx, const hc_tuning* in);
 
 /* Kernels of one step, as timed by hc_time_kernel.  The CG_* kernels are the
- * CG iteration (FP32 inner CG in refined mode, FP64 CG in plain mode); RES_*
- * the FP64 residual evaluation (refined: p64 += delta then S - A p64; plain:
- * the initial residual); SPLIT_* Step 2 of Algorithm 1.  On a 3D grid the
- * same ids time the 3D kernels: *_GRAD the z pass with the gradient
- * multipliers, *_APPLY the row-pair pass, *_DIV the z pass with the
+ * CG iteration (FP32 inner CG in refined mode, FP64 CG in plain mode) where it
+ * runs as kernels of its own: 3D, 2D grids without a loop kernel, and a batch's
+ * classes; RES_* the residual evaluation (refined: p64 += delta then S - A p64,
+ * with the default residual switches in the fixed-point transforms that usually
+ * end the loop; plain: the initial residual); SPLIT_* Step 2 of Algorithm 1.
+ * On a 3D grid the same ids time the 3D kernels: *_GRAD the z pass with the
+ * gradient multipliers, *_APPLY the row-pair pass, *_DIV the z pass with the
  * divergence, *_YPASS the y pass between them, SPLIT_ROW the row pass with
  * activation, relaxation and diffusion along x, SPLIT_HEAT / SPLIT_C2R the
  * diffusion along y / along z. */
 enum {
   HC_K_CG_GRAD = 0,    /* column pass: d-update, i xi d / n, inverse FFT_y */
   HC_K_CG_APPLY = 1,   /* row pass: C2R, (m m^T + r I) g, R2C */
-  HC_K_CG_DIV = 2,     /* column pass: FFT_y, -i xi . q (alpha comes from the row pass) */
-  HC_K_CG_UPDATE = 3,  /* x += alpha d, r -= alpha A d, <r, M^-1 r> */
+  HC_K_CG_DIV = 2,     /* column pass: FFT_y, -i xi . q (alpha comes from the row pass); 2D plain
+                          FP64: with the update */
+  HC_K_CG_UPDATE = 3,  /* x += alpha d, r -= alpha A d, <r, M^-1 r>; 2D plain FP64: 0 */
   HC_K_RES_GRAD = 4,
   HC_K_RES_APPLY = 5,
   HC_K_RES_DIV = 6,
@@ -345,7 +348,10 @@ enum {
   HC_K_MID_APPLY = 17,   /* its row pass (2D) / row-pair pass (3D) */
   HC_K_MID_DIV = 18,     /* its divergence pass */
   HC_K_MID_YPASS = 19,   /* 3D only: its y pass */
-  HC_K_COUNT = 20
+  HC_K_CG_LOOP = 20,     /* 2D: one iteration of the loop kernel that replaces the CG_* kernels on
+                            grids up to about 10^6 points, of `reps` in one launch
+                            (HC_ENOTSUP where the grid has none) */
+  HC_K_COUNT = 21
 };
 
 /* Launch one step kernel `reps` times back to back on the context's current
@@ -358,7 +364,8 @@ int hc_time_kernel(hc_ctx* ctx, int kernel, int reps, double* ms_per_launch);
 /* Number of this library's kernel launches issued by the context so far
  * (graph launches count every kernel node).  Where the CG loop runs as one
  * kernel (2D, up to about 10^6 points) its iterations still count as the
- * kernels that each stands for, so that counts compare between grids. */
+ * kernels that each stands for, so that counts compare between grids;
+ * hc_loop_count tells the loop launches themselves. */
 int hc_launch_count(const hc_ctx* ctx, long long* count);
 
 /* Measured FP64 FMA throughput of the current device in TFLOP/s (an FMA counts

@@ -169,7 +169,8 @@ hc_check_poke = lib.hc_check_poke
 # kernel ids of hc_time_kernel (include/hc.h)
 KERNELS = ["cg_grad", "cg_apply", "cg_div", "cg_update", "res_grad", "res_apply", "res_div",
            "split_grad", "split_row", "split_heat", "split_c2r", "cg_ypass", "res_ypass",
-           "first_grad", "first_apply", "first_div", "mid_grad", "mid_apply", "mid_div", "mid_ypass"]
+           "first_grad", "first_apply", "first_div", "mid_grad", "mid_apply", "mid_div", "mid_ypass",
+           "cg_loop"]
 
 
 def strerror(code: int) -> str:

@@ -5,6 +5,9 @@ every admissible column-tile width and rows-per-CTA count of the FP32 and
 FP64 kernel families and keeps the fastest.  Results are cached on disk per
 (GPU name, grid, precision) so later processes reuse them; the cache lives in
 ``$HC_TUNING_CACHE`` or ``~/.cache/hucai_gb300/tuning.json``.
+
+The CG kernels' shapes are those of the separate kernels: grids without a loop
+kernel, and the size classes of a batch, which run their first member's.
 """
 from __future__ import annotations
 
@@ -38,7 +41,7 @@ _WEIGHT = {"cg_grad": 20, "cg_apply": 20, "cg_div": 20}
 
 # Bumped whenever the kernels' launch-shape trade-offs change, so cached
 # choices made for older kernels are not reused.
-_KERNELS_VERSION = 7
+_KERNELS_VERSION = 8
 
 
 def _key(solver) -> str:
@@ -104,7 +107,8 @@ def autotune(solver, reps: int = 20, use_cache: bool = True, verbose: bool = Fal
             # the knob's pipelined variants: col_pipe 0/1 for the column
             # passes, row_pipe 0/1 for the FP32 apply row pass
             if knob == "col_tile":
-                pipes, pkey = (0, 1), "col_pipe"
+                # plain FP64's fixed-point passes have no pipelined form
+                pipes, pkey = ((0,) if prec == "fp64" else (0, 1)), "col_pipe"
             else:
                 pipes, pkey = ((0, 1) if idx == 0 else (None,)), "row_pipe"
             for pipe in pipes:

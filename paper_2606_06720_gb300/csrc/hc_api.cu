@@ -1273,15 +1273,16 @@ int read_state(hc_ctx* c) {
   return loop_reported(c, c->stream);
 }
 
-// The whole CG loop of a solve in one launch (loop.nt > 0).
-void cg_loop(hc_ctx* c) {
+// The whole CG loop of a solve in one launch (loop.nt > 0); x64: the plain mode's solution.
+void cg_loop_on(hc_ctx* c, hc::SolveState* st, cx<double>* x64) {
   if (c->refined)
     hc::cg_loop_f32(c->gf, c->loop, c->x32, c->r32, c->G32, c->G32 + c->ns, (const float*)c->m[0],
-                    (const float*)c->m[1], (const float*)c->rf, c->st, c->stream);
+                    (const float*)c->m[1], (const float*)c->rf, st, c->stream);
   else
-    hc::cg_loop_fx(c->gd, c->loop, c->p64, c->r64, c->G64, c->G64 + c->ns, (const double*)c->m[0],
-                   (const double*)c->m[1], (const double*)c->rf, c->st, c->stream);
+    hc::cg_loop_fx(c->gd, c->loop, x64, c->r64, c->G64, c->G64 + c->ns, (const double*)c->m[0],
+                   (const double*)c->m[1], (const double*)c->rf, st, c->stream);
 }
+void cg_loop(hc_ctx* c) { cg_loop_on(c, c->st, c->p64); }
 
 // Launch CG iterations in chunks until the device says done.
 int run_cg_host(hc_ctx* c, bool refined_inner) {
@@ -3591,6 +3592,40 @@ int hc_set_tuning(hc_ctx* c, const hc_tuning* t) {
   return HC_OK;
 }
 
+// One iteration of the loop kernel: `reps` of them in one launch from the current residual, on
+// scratch (x32, the stage) and the scratch state.
+static int time_loop(hc_ctx* c, hc::SolveState init, int reps, double* ms) {
+  if (!c->loop.nt) return HC_ENOTSUP;
+  init.it = 0;
+  init.maxit = reps;
+  hc::SolveState out;
+  cudaEvent_t e0, e1;
+  CU(cudaEventCreate(&e0));
+  CU(cudaEventCreate(&e1));
+  for (int warm = 1; warm >= 0; --warm) {
+    do {  // again where the device had no room
+      CU(cudaMemcpyAsync(c->st_time, &init, sizeof(init), cudaMemcpyHostToDevice, c->stream));
+      CU(cudaStreamSynchronize(c->stream));
+      CU(cudaEventRecord(e0, c->stream));
+      cg_loop_on(c, c->st_time, reinterpret_cast<cx<double>*>(c->stage));
+      CU(cudaEventRecord(e1, c->stream));
+      CU(cudaMemcpyAsync(&out, c->st_time, sizeof(out), cudaMemcpyDeviceToHost, c->stream));
+      CU(cudaStreamSynchronize(c->stream));
+      CU(cudaGetLastError());
+      init.loop_since = out.loop_since;
+      init.loop_turn = out.loop_turn;
+    } while (!out.done);
+    if (out.loop_timeout) break;
+  }
+  float t = 0;
+  CU(cudaEventElapsedTime(&t, e0, e1));
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  c->launches += 2;
+  *ms = (double)t / std::max(1, out.it);
+  return out.loop_timeout ? HC_ETIMEOUT : HC_OK;
+}
+
 int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
   if (!c || !ms_per_launch || reps < 1 || kernel < 0 || kernel >= HC_K_COUNT) return HC_EINVAL;
   if (c->gen) return HC_ENOTSUP;
@@ -3604,6 +3639,7 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
   init.alpha = 0;
   init.beta = 0;
   init.rho = 0;  // alpha = rho / <d, A d> stays 0 whichever kernel computes it
+  init.timing = 1;
   init.maxit = 0x7fffffff;
   init.thresh2 = -1.0;
   init.outer_thresh2 = -1.0;
@@ -3614,9 +3650,15 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
   hc::SolveState* ts = c->st_time;
   const size_t ns = c->ns;
   if (c->dim == 2 && (kernel == HC_K_CG_YPASS || kernel == HC_K_RES_YPASS)) return HC_EINVAL;
-  if (!c->refined && kernel >= HC_K_FIRST_GRAD) return HC_EINVAL;
-  if (kernel >= HC_K_MID_GRAD && (c->df || !c->refined)) return HC_EINVAL;  // HC_FP32_REFINED only
+  if (!c->refined && kernel >= HC_K_FIRST_GRAD && kernel <= HC_K_MID_YPASS) return HC_EINVAL;
+  if (kernel >= HC_K_MID_GRAD && kernel <= HC_K_MID_YPASS && (c->df || !c->refined))
+    return HC_EINVAL;  // HC_FP32_REFINED only
   if (c->dim == 2 && kernel == HC_K_MID_YPASS) return HC_EINVAL;
+  if (kernel == HC_K_CG_LOOP) return time_loop(c, init, reps, ms_per_launch);
+  if (kernel == HC_K_CG_UPDATE && c->dim == 2 && !c->refined) {  // in the divergence pass
+    *ms_per_launch = 0.0;
+    return HC_OK;
+  }
   // 3D: the same roles with the 3D kernels; the SPLIT_HEAT / SPLIT_C2R slots
   // time the y and z diffusion passes.  Scratch outputs never alias inputs
   // that a later repetition reads.
@@ -3624,6 +3666,7 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
     const hc::SplitCoef cf = split_coef(c->prm);
     if (c->refined) {
       auto& g = c->gf;
+      const hc::Geo<double> gd = decide_on(c) ? fx_geo(c->gd) : c->gd;  // the usual evaluation
       auto G = tri(c->G32, ns);
       auto* G64 = c->G64;
       auto mw = hc::Tri<float*>{{(float*)c->q32, (float*)c->x32, (float*)c->d32}};
@@ -3650,7 +3693,7 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
                                    nullptr, nullptr, nullptr, tri((cx<df64>*)G64, ns), ts, 0,
                                    c->stream);
           else
-            hc::z_grad<double, double>(c->gd, hc::CG_PLAIN, c->p64, nullptr, nullptr, nullptr,
+            hc::z_grad<double, double>(gd, hc::CG_PLAIN, c->p64, nullptr, nullptr, nullptr,
                                        tri(G64, ns), ts, 0, c->stream);
           break;
         case HC_K_RES_YPASS:
@@ -3658,7 +3701,7 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
             hc::axis_fft<df64>(c->gq, 1, +1, 3, tri((cx<df64>*)G64, ns), tri((cx<df64>*)G64, ns),
                                df64(1.0), c->stream);
           else
-            hc::axis_fft<double>(c->gd, 1, +1, 3, tri(G64, ns), tri(G64, ns), 1.0, c->stream);
+            hc::axis_fft<double>(gd, 1, +1, 3, tri(G64, ns), tri(G64, ns), 1.0, c->stream);
           break;
         case HC_K_RES_APPLY:
           if (c->df)
@@ -3666,7 +3709,7 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
                                         (const float*)c->rf, tri((cx<df64>*)G64, ns), nullptr,
                                         c->stream);
           else
-            hc::row_apply3<double, float>(c->gd, tri(G64, ns), mtri<float>(c), (const float*)c->rf,
+            hc::row_apply3<double, float>(gd, tri(G64, ns), mtri<float>(c), (const float*)c->rf,
                                           tri(G64, ns), nullptr, c->stream);
           break;
         case HC_K_RES_DIV:
@@ -3675,8 +3718,8 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
                             (const cx<df64>*)c->b64, (cx<df64>*)c->r64, c->d32, c->q32, ts,
                             c->stream);
           else
-            hc::z_div<double>(c->gd, hc::CD_RESID_REFINE, tri(G64, ns), nullptr, c->b64, c->r64,
-                              c->d32, c->q32, ts, c->stream);
+            hc::z_div<double>(gd, decide_on(c) ? hc::CD_DECIDE : hc::CD_RESID_REFINE,
+                              tri(G64, ns), nullptr, c->b64, c->r64, c->d32, c->q32, ts, c->stream);
           break;
         case HC_K_SPLIT_GRAD:
           hc::z_grad<float, double>(g, hc::CG_PLAIN, c->p64, nullptr, nullptr, nullptr, G, ts, 0,
@@ -3896,12 +3939,7 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
                                         c->stream);
           break;
         case HC_K_CG_DIV:
-          hc::col_div<double>(g, hc::CD_CG, Gx, Gy, c->d64, nullptr, c->q64, nullptr, nullptr, ts,
-                              c->stream);
-          break;
-        case HC_K_CG_UPDATE:
-          hc::cg_update<double>(g, (cx<double>*)c->stage, c->r64, c->d64,
-                                c->q64, ts, c->stream);
+          hc::col_div_upd(g, Gx, Gy, c->d64, (cx<double>*)c->stage, c->r64, ts, c->stream);
           break;
         case HC_K_RES_GRAD:
         case HC_K_SPLIT_GRAD:
@@ -3931,6 +3969,11 @@ int hc_time_kernel(hc_ctx* c, int kernel, int reps, double* ms_per_launch) {
       }
     }
   };
+  // <d, A d> of the current direction, which the timed pass forms its step length from
+  if (kernel == HC_K_CG_DIV && c->dim == 2 && !c->refined)
+    hc::row_apply<double, double>(c->gd, c->G64, c->G64 + ns, (const double*)c->m[0],
+                                  (const double*)c->m[1], (const double*)c->rf, c->q64,
+                                  (cx<double>*)c->stage, ts, c->stream);
   launch();  // warm-up
   CU(cudaGetLastError());
   cudaEvent_t e0, e1;

@@ -160,7 +160,7 @@ struct SolveState {
   double user_kappa;         // > 0: fixed kappa
   double outer_rtol2;        // cg_rtol^2
   int refined;               // 1: FP32 inner CG with FP64 refinement
-  int pad0_;
+  int timing;                // hc_time_kernel's scratch state: step lengths stay 0, nothing ends the loop
   int it;                    // CG iterations of the running solve
   int maxit;                 // cap
   int done;                  // running CG finished (converged or capped)

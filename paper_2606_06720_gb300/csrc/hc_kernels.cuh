@@ -869,7 +869,7 @@ __device__ __forceinline__ void cg_alpha_from(SolveState* st, double gkg, double
   if (dq > 0 && isfinite(dq)) {
     st->alpha = st->rho / dq;
     st->alpha_f = (float)st->alpha;
-  } else {
+  } else if (!st->timing) {
     // breakdown: <d, A d> is not positive (d without a component in the range
     // of A) or not finite.  The plain solve then stops unconverged unless its
     // residual already meets the tolerance; a refined inner solve leaves that
@@ -1358,7 +1358,7 @@ __device__ __forceinline__ void cg_step_finish(SolveState* st, double rr, double
   st->rnorm2 = rr;
   st->beta = st->rho > 0 ? rz / st->rho : 0.0;
   st->beta_f = (float)st->beta;
-  st->rho = rz;
+  st->rho = st->timing ? 0.0 : rz;
   st->it += 1;
   st->total_it += 1;
   if (!isfinite(rr)) {
@@ -2822,8 +2822,9 @@ void col_div(const Geo<T>& g0, int mode, const cx<T>* Qx, const cx<T>* Qy, const
         case CD_PLAIN:
           kp_col_div<T, CD_PLAIN><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
           break;
-        case CD_CG:
-          kp_col_div<T, CD_CG><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
+        case CD_CG:  // FP32 alone (plain FP64: col_div_upd)
+          if constexpr (std::is_same<T, float>::value)
+            kp_col_div<T, CD_CG><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
           break;
         case CD_RESID:
           kp_col_div<T, CD_RESID><<<g.pgrid, nt, ps, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
@@ -2845,7 +2846,8 @@ void col_div(const Geo<T>& g0, int mode, const cx<T>* Qx, const cx<T>* Qy, const
       k_col_div<T, CD_PLAIN><<<nb, nt, sm, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
       break;
     case CD_CG:
-      k_col_div<T, CD_CG><<<nb, nt, sm, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
+      if constexpr (std::is_same<T, float>::value)
+        k_col_div<T, CD_CG><<<nb, nt, sm, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
       break;
     case CD_RESID:
       k_col_div<T, CD_RESID><<<nb, nt, sm, s>>>(g, Qx, Qy, d, b, out, r32, delta32, st);
@@ -2975,7 +2977,7 @@ void set_smem_limits_t() {
   allow_smem(k_col_heat<T>);
   allow_smem(k_col_gradnorm<T>);
   allow_smem(k_col_div<T, CD_PLAIN>);
-  allow_smem(k_col_div<T, CD_CG>);
+  if constexpr (std::is_same<T, float>::value) allow_smem(k_col_div<T, CD_CG>);
   allow_smem(k_col_div<T, CD_RESID>);
   allow_smem(k_col_div<T, CD_RESID_REFINE>);
   if constexpr (std::is_same<T, float>::value) {
@@ -2984,7 +2986,7 @@ void set_smem_limits_t() {
   }
   if constexpr (!seq_fields<T>()) {
     allow_smem(kp_col_div<T, CD_PLAIN>);
-    allow_smem(kp_col_div<T, CD_CG>);
+    if constexpr (std::is_same<T, float>::value) allow_smem(kp_col_div<T, CD_CG>);
     allow_smem(kp_col_div<T, CD_RESID>);
     allow_smem(kp_col_div<T, CD_RESID_REFINE>);
     allow_smem(kp_col_heat<T>);

@@ -41,11 +41,9 @@ void set_smem_limits_df() {
   allow_smem(k_col_fwd<df64, 2>);
   allow_smem(k_col_inv<df64>);
   allow_smem(k_col_div<df64, CD_PLAIN>);
-  allow_smem(k_col_div<df64, CD_CG>);
   allow_smem(k_col_div<df64, CD_RESID>);
   allow_smem(k_col_div<df64, CD_RESID_REFINE>);
   allow_smem(kp_col_div<df64, CD_PLAIN>);
-  allow_smem(kp_col_div<df64, CD_CG>);
   allow_smem(kp_col_div<df64, CD_RESID>);
   allow_smem(kp_col_div<df64, CD_RESID_REFINE>);
   allow_smem(kp_col_grad<df64, CG_PLAIN>);

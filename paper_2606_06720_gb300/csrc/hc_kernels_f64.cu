@@ -29,8 +29,6 @@ template void col_div<double>(const Geo<double>&, int, const cx<double>*, const 
 template void col_heat<double>(const Geo<double>&, cx<double>*, cx<double>*, SolveState*, cudaStream_t);
 template void col_gradnorm<double>(const Geo<double>&, const cx<double>*, const cx<double>*, SolveState*, int,
                                  cudaStream_t);
-template void cg_update<double>(const Geo<double>&, cx<double>*, cx<double>*, const cx<double>*,
-                                const cx<double>*, SolveState*, cudaStream_t);
 template void convert<double, float>(const float*, double*, size_t, cudaStream_t);
 template void convert<float, double>(const double*, float*, size_t, cudaStream_t);
 template void convert<double, double>(const double*, double*, size_t, cudaStream_t);

@@ -57,9 +57,12 @@ extern "C" {
 #define HC_STOP_STATUS 3    /* a step failed (HC_ENONFINITE) */
 
 /* Arithmetic of the path. */
-#define HC_FP64_PLAIN 0   /* FP64 fields and pointwise arithmetic; power-of-two transforms of 64 points or
-                             more in 64-bit block fixed point, whose error is below that of the
-                             same transform in IEEE FP64 */
+#define HC_FP64_PLAIN 0   /* FP64 fields and pointwise arithmetic; transforms in 64-bit block fixed
+                             point (powers of two below 64 points: FP64).  The error of a 2D
+                             transform, powers of two, is below 8 * 2^-53 of its result's L2 norm
+                             (measured 0.5-1.4e-16; FP64 passes 1.1-2.9e-16): relative to the whole
+                             transform, not to each value, so values far below the norm keep
+                             fewer bits */
 #define HC_FP32_REFINED 1 /* FFTs, operator applies and split step in FP32; pressure solve wrapped in
                              FP64 iterative refinement (FP64 residual, FP64 correction accumulation,
                              FP64 dot products and null-space projection) */
@@ -452,9 +455,11 @@ void hc_batch_destroy(hc_batch* batch);
  *   nx, ny: powers of two in [8, 4096] with nx*ny <= HC_NOALLOC_MAX_POINTS;
  *           anything else (or a null pointer) returns HC_EINVAL.
  *   stream: cudaStream_t (NULL: legacy default stream); the call only enqueues
- *           work on it and returns (the first call on a device waits, see below).  CUDA failures of its own launches return
- *           HC_ECUDA; a non-sticky error left pending on the calling thread by
- *           earlier work is cleared on entry (cudaGetLastError), not reported.
+ *           work on it and returns (the first call on a device waits, see
+ *           below).  CUDA failures of its own launches return HC_ECUDA; a
+ *           non-sticky error left pending on the calling thread by earlier work
+ *           is cleared on entry (cudaGetLastError), not reported.
+ * Fixed-point transforms as HC_FP64_PLAIN's, with twiddles of FP64 accuracy.
  * Scratch lives in one fixed 640 KiB static device array of the library
  * (present on every GPU the process uses, until the process exits); the call
  * allocates nothing and calls no allocating routine.  All calls share that

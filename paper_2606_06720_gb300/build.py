@@ -26,7 +26,8 @@ BUILD_DIR = os.path.join(HERE, "_build")
 CHECK_SOURCE = "hc_api.cu"   # the only unit HC_CHECK changes
 
 SOURCES = ["hc_kernels_f32.cu", "hc_kernels_f64.cu", "hc_kernels_fx.cu", "hc_kernels_df.cu",
-           "hc_kernels3d_f32.cu", "hc_kernels3d_f64.cu", "hc_kernels3d_fx.cu", "hc_kernels3d_df.cu", "hc_cgloop.cu", "hc_batch.cu", "hc_generic.cu", "hc_api.cu",
+           "hc_kernels3d_f32.cu", "hc_kernels3d_f64.cu", "hc_kernels3d_fx.cu",
+           "hc_kernels3d_df.cu", "hc_cgloop.cu", "hc_batch.cu", "hc_generic.cu", "hc_api.cu",
            "hc_noalloc.cu"]
 HEADERS = ["hc_internal.cuh", "hc_fixed.cuh", "hc_kernels.cuh", "hc_kernels3d.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

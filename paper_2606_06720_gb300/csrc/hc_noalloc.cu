@@ -139,7 +139,7 @@ extern "C" int hc_spectrum_noalloc(const double* f, double* out, int nx, int ny,
   // Every call rewrites the part of the intermediate that it reads, so nothing
   // carried over from an earlier call is used.  The column pass may start while
   // the row pass drains (it waits before its first read): with the tables kept
-  // and the narrower CTAs a 256^2 call takes 25 us where four launches in 8 and
+  // and the narrower CTAs a 256^2 call takes 26.7 us where four launches in 8 and
   // 32 CTAs took 39 (67 with FP64 passes).  What is left is the latency of one
   // warp's instructions: each thread carries 8 points through three passes.
   hc::k_row_r2c<fx64><<<ny >> g.lrpc, rpc << (g.lnx - 3), (size_t)rpc * nx * sizeof(cx<double>), s>>>(
